@@ -65,7 +65,8 @@ struct DevState {
     int *flag = nullptr;
     int *mvstatus = nullptr;         // matvec status word (bit 4: tensor-core wait gave up)
     int m2l_kernel = 0;              // 0 FP64 SIMT, 1 FP32 SIMT, 2 tcgen05 streamed, 3 tcgen05 persistent
-    cf *ephase = nullptr;            // persistent kernel: e^{i d phi} per pair, d = -(p+2)..p+2
+    cf *ephase = nullptr;            // sector kernel: phases G[d] per pair
+    void *mepk = nullptr;            // ... and the packed multipole expansions it reads
     int nsm = 0;
     cd *stage = nullptr;             // [2][N][3] for host-buffer matvec
     cudaEvent_t ev[9]{};
@@ -202,6 +203,22 @@ int64_t m2l_work_items(const lmfmm_ctx *ctx, int bn, int prob, std::vector<M2LWo
         }
     }
     return ncols;
+}
+
+// Work items of the sector kernel: per geometry, runs of at most `pairs` pairs.
+void sec_work_items(const lmfmm_ctx *ctx, int pairs, int prob, std::vector<M2LWork> &mw)
+{
+    for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
+        const Geom &g = ctx->geoms[gi];
+        for (int64_t q = g.pair0; q < g.pair1; q += pairs) {
+            M2LWork w{};
+            w.geom = (int)gi;
+            w.pair0 = q;
+            w.npair = (int)std::min<int64_t>(pairs, g.pair1 - q);
+            w.prob = prob;
+            mw.push_back(w);
+        }
+    }
 }
 
 // Tabulate a list of geometries into `tab` (device), batching node factors
@@ -459,10 +476,10 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     const int64_t N = ctx->N, nbox = (int64_t)ctx->boxes.size();
     // memory estimate (tables dominate)
     const bool img_path = ctx->prm.precision == LMFMM_MIXED &&
-                          (ctx->prm.tensor_cores == 1 || ctx->prm.tensor_cores == 3) && m2l_tc2_supported(p);
+                          (ctx->prm.tensor_cores == 1 || ctx->prm.tensor_cores == 3) && m2l_sec_supported(p);
     double need = (double)ctx->geoms.size() * NTAB * P * P * 16.0 +
-                  (img_path ? (double)m2l_tc2_image_bytes(p, (int64_t)ctx->geoms.size()) +
-                                  (double)ctx->m2l.size() * (2 * p + 5) * 8.0
+                  (img_path ? (double)m2l_sec_image_bytes(p, (int64_t)ctx->geoms.size()) +
+                                  (double)ctx->m2l.size() * m2l_sec_phases(p) * 8.0
                             : 0.0) +
                   (double)nbox * 6 * P * 16.0 + (double)ctx->tgroups.size() * 2 * P * P * 16.0 +
                   (double)ctx->n_near_pp * 13 * 16.0 + (double)N * 200.0;
@@ -516,7 +533,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     const bool f32 = ctx->prm.precision == LMFMM_MIXED;
     d->m2l_kernel = !f32 ? 0
                     : ctx->prm.tensor_cores == 0 ? 1
-                    : ((ctx->prm.tensor_cores == 1 || ctx->prm.tensor_cores == 3) && m2l_tc2_supported(p)) ? 3
+                    : ((ctx->prm.tensor_cores == 1 || ctx->prm.tensor_cores == 3) && m2l_sec_supported(p)) ? 3
                     : m2l_tc_supported(p) ? 2 : 1;
     const size_t esz = f32 ? sizeof(cf) : sizeof(cd);
     {
@@ -586,29 +603,15 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         TRY(dupload(ctx, &d->geoms, hg));
         if (d->m2l_kernel == 3) {
             unsigned char *img = nullptr;
-            TRY(dalloc(ctx, &img, m2l_tc2_image_bytes(p, (int64_t)hg.size())));
-            launch_tile_tables(p, 0, (int64_t)hg.size(), d->geoms, d->comps, tab64, img, st);
+            TRY(dalloc(ctx, &img, m2l_sec_image_bytes(p, (int64_t)hg.size())));
+            launch_sec_image(p, (int64_t)hg.size(), d->geoms, d->comps, tab64, img, st);
             CK(cudaGetLastError());
             CK(cudaStreamSynchronize(st));
             dfree(ctx, tab64);
             d->tab = img;
             CK(cudaDeviceGetAttribute(&d->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-            TRY(dalloc(ctx, &d->yscr, m2l_tc2_scratch_floats(p, d->nsm)));
-            // phases of every pair: powers in FP64, rounded once to FP32
-            const int MW = 2 * p + 5;
-            std::vector<cf> ph(ctx->m2l.size() * (size_t)MW);
-            for (size_t i = 0; i < ctx->m2l.size(); ++i) {
-                const cd b{ctx->m2l[i].cphi, ctx->m2l[i].sphi};
-                cd e{1.0, 0.0};
-                cf *row = ph.data() + i * MW + (p + 2);
-                row[0] = cf{1.f, 0.f};
-                for (int m = 1; m <= p + 2; ++m) {
-                    e = e * b;
-                    row[m] = cf{(float)e.x, (float)e.y};
-                    row[-m] = cf{(float)e.x, (float)-e.y};
-                }
-            }
-            TRY(dupload(ctx, &d->ephase, ph));
+            // one scratch for the M2L and the translations, which run one after the other
+            TRY(dalloc(ctx, &d->yscr, std::max(m2l_sec_scratch_floats(p, d->nsm), trans_tc2_scratch_floats(p, d->nsm))));
         } else if (f32) {
             cf *t32 = nullptr;
             TRY(dalloc(ctx, &t32, ctx->geoms.size() * (size_t)NTAB * P * P));
@@ -625,8 +628,18 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     }
     TRY(dupload(ctx, &d->m2l, ctx->m2l));
     std::vector<M2LWork> mw;
-    const int64_t ncols = m2l_work_items(ctx, d->m2l_kernel >= 2 ? m2l_tc_cols()
-                                                : f32 ? gemm_cols<float>() : gemm_cols<double>(), 0, mw);
+    const int64_t ncols = 9 * (int64_t)ctx->m2l.size();   // helical columns: nine table applications per pair
+    if (d->m2l_kernel == 3) {
+        TRY(dalloc(ctx, &d->ephase, ctx->m2l.size() * (size_t)m2l_sec_phases(p)));
+        unsigned char *pk = nullptr;
+        TRY(dalloc(ctx, &pk, m2l_sec_packed_bytes(p, nbox)));
+        d->mepk = pk;
+        launch_pair_phases(p, (int64_t)ctx->m2l.size(), d->m2l, d->ephase, st);
+        CK(cudaGetLastError());
+        sec_work_items(ctx, m2l_sec_pairs(), 0, mw);
+    } else {
+        m2l_work_items(ctx, d->m2l_kernel == 2 ? m2l_tc_cols() : f32 ? gemm_cols<float>() : gemm_cols<double>(), 0, mw);
+    }
     TRY(dupload(ctx, &d->m2lwork, mw));
     d->n_m2lwork = (int64_t)mw.size();
     // translation matrices (exact addition theorem, host)
@@ -700,7 +713,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         }
         TRY(dupload(ctx, &d->tchild, ctx->tpair_child));
         TRY(dupload(ctx, &d->tparent, ctx->tpair_parent));
-        d->trans_tc = d->m2l_kernel == 3 && ctx->prm.tensor_cores == 3;
+        d->trans_tc = d->m2l_kernel == 3 && ctx->prm.tensor_cores == 3 && trans_tc2_supported(p);
         if (d->trans_tc) {
             // M2M / L2L on the persistent tensor-core kernel: tiled bf16 three-piece
             // images of the scaled FP64 matrices, items of 21 pairs (63 helical columns)
@@ -813,7 +826,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     S.n_near_pairs = (int64_t)ctx->near.size();
     S.n_near_point_pairs = ctx->n_near_pp;
     S.n_quad_nodes = qtot;
-    S.bytes_tables = d->m2l_kernel == 3 ? (double)m2l_tc2_image_bytes(p, (int64_t)ctx->geoms.size())
+    S.bytes_tables = d->m2l_kernel == 3 ? (double)m2l_sec_image_bytes(p, (int64_t)ctx->geoms.size())
                      : (double)ctx->geoms.size() * NTAB * P * P * (f32 ? 8.0 : 16.0);
     S.ms_setup = std::chrono::duration<double, std::milli>(t1 - t0).count();
     S.m2l_columns = ncols;
@@ -906,13 +919,21 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
     }
     if (parts & MV_M2L) {
     nl += d->n_m2lwork > 0;   // M2L
-    CK(cudaMemsetAsync(le, 0, (size_t)nbox * 3 * P * sizeof(cx<T>), st));
+    bool packed = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (d->m2l_kernel == 3) {
+            launch_sec_pack(p, nbox, me, d->mepk, le, st);   // clears le too
+            packed = true;
+            ++nl;
+        }
+    }
+    if (!packed) CK(cudaMemsetAsync(le, 0, (size_t)nbox * 3 * P * sizeof(cx<T>), st));
     if (!own_m2l) {
         // the batch's merged launch applies this problem's M2L
     } else if constexpr (std::is_same<T, float>::value) {
         if (d->m2l_kernel == 3) {
-            CK(launch_m2l_tc2(p, d->n_m2lwork, d->m2lwork, d->geoms, d->m2l, d->ephase, d->tab,
-                              me, le, d->yscr, d->nsm, d->mvstatus, st));
+            CK(launch_m2l_sec(p, d->n_m2lwork, d->m2lwork, TcProb{d->m2l, d->ephase, d->tab, d->mepk, le}, nullptr, d->yscr,
+                              d->nsm, d->mvstatus, st));
         }
         else if (d->m2l_kernel == 2)
             CK(launch_m2l_tc(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
@@ -1175,7 +1196,7 @@ lmfmm_status batch_work(lmfmm_batch *b, int variant, M2LWork **dst, int64_t *n)
 {
     std::vector<std::vector<M2LWork>> per(b->ctxs.size());
     for (size_t i = 0; i < b->ctxs.size(); ++i)
-        m2l_work_items(b->ctxs[i], (variant & 2) ? m2l_tc_cols() / 2 : m2l_tc_cols(), (int)i, per[i]);
+        sec_work_items(b->ctxs[i], (variant & 2) ? m2l_sec_pairs() / 2 : m2l_sec_pairs(), (int)i, per[i]);
     std::vector<M2LWork> all;
     if (variant & 1) {
         for (size_t k = 0;; ++k) {
@@ -1212,7 +1233,7 @@ lmfmm_status batch_record(lmfmm_batch *b, const void *const *J, void *const *Phi
     if (b->merged) {
         if (cudaMemsetAsync(b->status, 0, sizeof(int), st) != cudaSuccess) return LMFMM_ERR_CUDA;
         DevState *d0 = DS(b->ctxs[0]);
-        if (launch_m2l_tc2_batch(b->p, b->nwork, b->dwork, b->dprobs, d0->yscr, d0->nsm, b->status, st) !=
+        if (launch_m2l_sec(b->p, b->nwork, b->dwork, TcProb{}, b->dprobs, d0->yscr, d0->nsm, b->status, st) !=
             cudaSuccess)
             return LMFMM_ERR_CUDA;
     }
@@ -1256,7 +1277,7 @@ lmfmm_status lmfmm_batch_create(lmfmm_batch **out, lmfmm_ctx *const *ctxs, int n
         std::vector<TcProb> hp(n);
         for (int i = 0; i < n; ++i) {
             DevState *d = DS(ctxs[i]);
-            hp[i] = TcProb{d->geoms, d->m2l, d->ephase, d->tab, (const cf *)d->me, (cf *)d->le};
+            hp[i] = TcProb{d->m2l, d->ephase, d->tab, d->mepk, (cf *)d->le};
         }
         if (cudaMalloc((void **)&b->dprobs, n * sizeof(TcProb)) != cudaSuccess ||
             cudaMemcpy(b->dprobs, hp.data(), n * sizeof(TcProb), cudaMemcpyHostToDevice) != cudaSuccess)
@@ -1331,10 +1352,9 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream)
     if (cudaSetDevice(b->device) != cudaSuccess) return LMFMM_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
     DevState *d0 = DS(b->ctxs[0]);
-    const int P = (b->p + 1) * (b->p + 1);
     // defined inputs for the timing runs
     for (lmfmm_ctx *c : b->ctxs)
-        if (cudaMemsetAsync(DS(c)->me, 0, c->boxes.size() * 3 * (size_t)P * sizeof(cf), st) != cudaSuccess)
+        if (cudaMemsetAsync(DS(c)->mepk, 0, m2l_sec_packed_bytes(b->p, (int64_t)c->boxes.size()), st) != cudaSuccess)
             return LMFMM_ERR_CUDA;
     cudaEvent_t e0, e1;
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return LMFMM_ERR_CUDA;
@@ -1347,7 +1367,7 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream)
         float tmin = 1e30f;
         for (int rep = 0; rep < 4; ++rep) {
             cudaEventRecord(e0, st);
-            launch_m2l_tc2_batch(b->p, nw, w, b->dprobs, d0->yscr, d0->nsm, b->status, st);
+            launch_m2l_sec(b->p, nw, w, TcProb{}, b->dprobs, d0->yscr, d0->nsm, b->status, st);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0;

@@ -1,7 +1,6 @@
-// M2L (and, in translation mode, M2M / L2L) of the mixed form on the
-// 5th-generation tensor cores (tcgen05).  Two kernels: k_m2l_tc2 (v2 below,
-// persistent, three-piece bf16 operands, p <= 12) and k_m2l_tc (this part,
-// streamed operands, TF32 hi/lo, p <= 15).
+// Tensor-core kernels (tcgen05) of the mixed form beside the sector M2L of k_m2l_sec.cu:
+// k_m2l_tc (this part: M2L with streamed operands, TF32 hi/lo, p <= 15, for p > 12 and on
+// request) and k_trans_tc2 (v2 below: M2M and L2L, persistent, three-piece bf16, p <= 12).
 //
 // k_m2l_tc: a work item applies one scaled table A (P x P complex, row (nu,mu), column
 // (n',m')) to up to 64 phase-shifted source expansions, exactly as the FP32
@@ -366,43 +365,39 @@ __global__ void __launch_bounds__(NT) k_m2l_tc(int p, int MT, uint32_t tmem_cols
 }
 
 // ====================================================================== v2
-// Persistent, warp-specialised form with the operand roles exchanged:
-//   D (128 x NR) = X (128 x K) T'^T,
+// M2M and L2L, persistent and warp-specialised, with the operand roles exchanged:
+//   D (128 x NR) = X (128 x K) T^T,
 // whose 128 rows are real columns -- rows 2c, 2c+1 hold (Re x, -Im x) and
-// (Im x, Re x) of complex column c, giving Re (T' x) and Im (T' x) -- and
-// whose NR >= P columns are the table rows (nu, mu).  The table enters as
+// (Im x, Re x) of complex column c, giving Re (T x) and Im (T x) -- and whose NR >= P
+// columns are the rows of the translation matrix T.  The matrix enters as
 // the B operand unchanged in shape (K = interleaved Re/Im input index); it
 // is stored once per build as three bf16 planes (x ~ x1 + x2 + x3, each the
 // bf16 rounding of what the previous pieces leave) in exactly the
-// shared-memory image of each K-step, with the factors of the M2L that depend
-// only on the degrees folded in:
-//   T'[nu mu][n' m'] = (-i)^nu f_t^nu  T[nu mu][n' m']  i^n' f_s^n'
-// (f = -1 where a downward component or a mirrored box flips odd powers,
-// else 1; these are exact in any precision).  What is left per column is one
-// complex factor per input order m' (phase e^{i m' phi} and i^m') and one per
-// output order mu.  Roles (576 threads, one CTA per SM -- the tensor memory
+// shared-memory image of each K-step.  A work item is 21 box pairs of one matrix, three
+// helical columns each.  Roles (576 threads, one CTA per SM -- the tensor memory
 // holds one CTA's accumulators, so latency is hidden by more warps per role):
 //   warps 0-7   X producers, two groups of four warps (one per tensor-memory
 //               lane quadrant), group g writing K-step g of every chunk: the
-//               work item's 64 columns, coefficients prefetched V2_D chunks
-//               ahead, phase-shifted, split once into three bf16 pieces (the
+//               work item's columns, coefficients prefetched V2_D chunks
+//               ahead, split once into three bf16 pieces (the
 //               two rows of a column share the pieces) and written into a
 //               V2_SX-slot tensor-memory ring (A operand);
 //   warps 8-15  epilogue, two warps per lane quadrant taking alternate row
 //               slabs: accumulators -> a per-CTA column-major scratch in global
 //               memory through a per-warp shared tile (L2-resident; tensor
-//               memory is free for the next item at once), then the output
-//               factors and float2 atomics into the local expansions, then the
-//               column data of the item two ahead;
-//   warp 16     one bulk copy per table chunk into an S_T-slot shared ring;
+//               memory is free for the next item at once), then
+//               float2 atomics into the destination expansions, then the
+//               column records of the item two ahead;
+//   warp 16     one bulk copy per matrix chunk into an S_T-slot shared ring;
 //   warp 17     MMA issue, per K-step of 16 real K: X1 T1 into one accumulator,
 //               X1 T2 + X2 T1 + X1 T3 + X2 T2 + X3 T1 into a second (the tensor
 //               core truncates small addends against a large accumulator).
 // A chunk is V2_KS MMA K-steps, so that waits, fences and commits are paid
 // once per V2_KS steps; ring positions advance as counters (no division in the
-// loops).  In translation mode (M2M, L2L) the chunks run from the highest
-// input degree down.  Every wait is bounded; a wait that gives up sets bit 4
-// of the status word and its role stops.
+// loops).  The chunks run from the highest input degree down: the accumulator truncates
+// relative to its running sum, so the dominant low-degree terms come last and the
+// low-degree outputs see few truncations at full size.  Every wait is bounded; a wait
+// that gives up sets bit 4 of the status word and its role stops.
 namespace {
 
 constexpr int V2_KS = 2;           // MMA K-steps (16 real K each) per ring chunk
@@ -425,11 +420,10 @@ constexpr uint32_t V2_SMEM_MAX = 227 * 1024;
 
 struct V2Col {
     int64_t in_base, out_base;   // (box * 3 + helical v) * P of the source / target
-    int pp, kap;                 // pair within the work item, signed kappa
 };
 
 struct V2Plan {
-    uint32_t NR, nchunk, SB, CB, ST, MO, g_bytes, cols_bytes, meta_bytes, meta, tabs, mm_n, dtile, bars, total;
+    uint32_t NR, nchunk, SB, CB, ST, meta_bytes, meta, dtile, bars, total;
 };
 
 __host__ __device__ inline V2Plan v2_plan(int p)
@@ -440,29 +434,17 @@ __host__ __device__ inline V2Plan v2_plan(int p)
     s.nchunk = (uint32_t)(((P + 7) / 8 + V2_KS - 1) / V2_KS);   // chunks of V2_KS K-steps
     s.SB = s.NR * 32 * V2_NPC;                      // image of a K-step: V2_NPC planes of NR rows x 16 bf16
     s.CB = V2_KS * s.SB;
-    s.MO = 2 * p + 1;                               // orders -p..p
-    s.g_bytes = BN * s.MO * 8;                      // one factor table: [64][2p+1] complex
-    s.cols_bytes = BN * (uint32_t)sizeof(V2Col);
-    s.meta_bytes = 2 * s.g_bytes + s.cols_bytes;    // G, O, column records
-    s.mm_n = V2_KC * s.nchunk;                      // order table, whole chunks (>= P)
+    s.meta_bytes = BN * (uint32_t)sizeof(V2Col);
     const uint32_t dtile_bytes = V2_EW * 16 * V2_DS * 4;   // per epilogue warp: 16 rows x 32 lanes
     const uint32_t fixed =
-        2 * s.meta_bytes + 2 * s.mm_n + 32 + dtile_bytes + 16 + (2 * V2_ST_MAX + 2 * V2_SX + 12) * 8 + 16;
+        2 * s.meta_bytes + 32 + dtile_bytes + 16 + (2 * V2_ST_MAX + 2 * V2_SX + 12) * 8 + 16;
     uint32_t st = (V2_SMEM_MAX - fixed) / s.CB;
     s.ST = st > V2_ST_MAX ? V2_ST_MAX : st;
     s.meta = s.ST * s.CB;
-    s.tabs = (s.meta + 2 * s.meta_bytes + 15) & ~15u;
-    s.dtile = (s.tabs + 2 * s.mm_n + 15) & ~15u;
+    s.dtile = (s.meta + 2 * s.meta_bytes + 15) & ~15u;
     s.bars = (s.dtile + dtile_bytes + 15) & ~15u;
     s.total = s.bars + (2 * V2_ST_MAX + 2 * V2_SX + 12) * 8 + 16;
     return s;
-}
-
-__device__ __forceinline__ cf lds_cf(uint32_t a)
-{
-    cf v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(a));
-    return v;
 }
 
 // three-piece bf16 split of a pair, x ~ b1 + b2 + b3 per component (b1 =
@@ -482,146 +464,38 @@ __device__ __forceinline__ void v2_split_bf16(float lo, float hi, uint32_t (&w)[
     }
 }
 
-// i^k v, exact
-__device__ __forceinline__ cf mul_ipow(int k, cf v)
+// column records of an item: three helical columns per box pair
+__device__ __forceinline__ void v2_fill(int P, const M2LWork &w, const int64_t *tsrc, const int64_t *tdst, V2Col *cols,
+                                        int tid, int nthr)
 {
-    switch (k & 3) {
-    case 0: return v;
-    case 1: return cf{-v.y, v.x};
-    case 2: return cf{-v.x, -v.y};
-    default: return cf{v.y, -v.x};
-    }
-}
-
-// per-item column data, all exact transforms of the pair phases
-// E[pp][d] = e^{i d phi} (FP64-computed, stored FP32):
-//   input factors  G[pp][m'] = i^m' f_s^m' E[m'],
-//   output factors O[col][mh] = coef i^(1+kappa) (-i)^mu f_t^mu E[kappa - mu],
-//   mu = +-mh (sign of kappa), coef in {1/2, 1, -1/2};
-// and the column records.  One warp per pair or column row, one lane per
-// order (2p+1 <= 32), so that the fill has no division and no divergence.
-__device__ __forceinline__ void v2_fill_meta(int p, int P, const M2LWork &w, const M2LPair *pairs,
-                                             const cf *ephase, bool flip_in, bool flip_out, cf *G, cf *O,
-                                             V2Col *cols, int tid, int nthr)
-{
-    const int MO = 2 * p + 1, MW = 2 * p + 5;
-    const int t = w.t, ncpp = (t == 1) ? 1 : 2, ncol = w.npair * ncpp;
-    const int lane = tid & 31, wi = tid >> 5, nw = nthr >> 5;
-    const int m = lane - p;                      // order of this lane
-    // rows per warp: at most RB (npair, ncol <= 64 over nw >= 8 warps); every
-    // global load of the fill is issued before the first use
-    constexpr int RB = 8;
-    M2LPair pr{};
-    if (tid < ncol) pr = pairs[w.pair0 + (ncpp == 1 ? tid : tid >> 1)];
-    cf vg[RB], vo[RB];
-    if (lane < MO) {
-#pragma unroll
-        for (int i = 0; i < RB; ++i) {
-            const int pp = min(wi + i * nw, w.npair - 1);
-            vg[i] = ephase[(w.pair0 + pp) * MW + (p + 2) + m];
-        }
-#pragma unroll
-        for (int i = 0; i < RB; ++i) {
-            const int col = min(wi + i * nw, ncol - 1);
-            const int pp = ncpp == 1 ? col : col >> 1;
-            const ColSpec &cs = c_cols[t][ncpp == 1 ? 0 : col & 1];
-            const int mu = cs.kap < 0 ? -m : m;
-            vo[i] = ephase[(w.pair0 + pp) * MW + (p + 2) + cs.kap - mu];
-        }
-#pragma unroll
-        for (int i = 0; i < RB; ++i) {
-            const int pp = wi + i * nw;
-            if (pp >= w.npair) break;
-            cf x = mul_ipow(m, vg[i]);
-            if (flip_in && (m & 1)) x = -x;
-            G[pp * MO + lane] = x;
-        }
-#pragma unroll
-        for (int i = 0; i < RB; ++i) {
-            const int col = wi + i * nw;
-            if (col >= ncol) break;
-            const ColSpec &cs = c_cols[t][ncpp == 1 ? 0 : col & 1];
-            const int mu = cs.kap < 0 ? -m : m;
-            float cf0 = (float)cs.coef;
-            if (cs.kap < 0 && (cs.kap & 1)) cf0 = -cf0;
-            if (flip_out && (mu & 1)) cf0 = -cf0;
-            O[col * MO + lane] = cf0 * mul_ipow(1 + cs.kap - mu, vo[i]);
-        }
-    }
-    static_assert(BN <= V2_ET, "one column record per epilogue thread");
-    if (tid < BN) {
-        V2Col q{};
-        if (tid < ncol) {
-            const ColSpec &cs = c_cols[t][ncpp == 1 ? 0 : tid & 1];
-            q.in_base = (pr.src * 3 + cs.vin) * (int64_t)P;
-            q.out_base = (pr.tgt * 3 + cs.vout) * (int64_t)P;
-            q.pp = ncpp == 1 ? tid : tid >> 1;
-            q.kap = cs.kap;
-        }
-        cols[tid] = q;
-    }
-}
-
-__device__ __forceinline__ void v2_fill_trans(int p, int P, const M2LWork &w, const int64_t *tsrc,
-                                              const int64_t *tdst, cf *G, cf *O, V2Col *cols, int tid, int nthr)
-{
-    const int MO = 2 * p + 1, ncol = 3 * w.npair;
-    for (int e = tid; e < BN * MO; e += nthr) {
-        G[e] = cf{1.f, 0.f};
-        O[e] = cf{1.f, 0.f};
-    }
     for (int col = tid; col < BN; col += nthr) {
         V2Col q{};
-        if (col < ncol) {
+        if (col < 3 * w.npair) {
             const int pp = col / 3, v = col - 3 * pp;
             q.in_base = (tsrc[w.pair0 + pp] * 3 + v) * (int64_t)P;
             q.out_base = (tdst[w.pair0 + pp] * 3 + v) * (int64_t)P;
-            q.pp = pp;
-            q.kap = 0;
         }
         cols[col] = q;
     }
 }
 
-// complex columns of a work item
-__device__ __forceinline__ int v2_ncol(const M2LWork &w, int mode)
-{
-    return mode == 0 ? w.npair * ((w.t == 1) ? 1 : 2) : 3 * w.npair;
-}
-
 }  // namespace
 
 __global__ void __launch_bounds__(V2_THREADS, 1)
-    k_m2l_tc2(int p, int mode, int64_t nwork, const M2LWork *work, const GeomDev *geoms, const M2LPair *pairs, const cf *ephase, const int64_t *tsrc, const int64_t *tdst,
-              const uint32_t *timg, const cf *me, cf *le, float *yscr,
-              int *status, const TcProb *probs)
+    k_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc, const int64_t *tdst,
+                const unsigned char *img, const cf *in, cf *out, float *yscr, int *status)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     const int P = (p + 1) * (p + 1);
     const V2Plan sp = v2_plan(p);
-    const int NR = (int)sp.NR, nchunk = (int)sp.nchunk, ST = (int)sp.ST, MO = (int)sp.MO;
-    // translations take the inputs from the highest degrees down: the accumulator
-    // truncates relative to its running sum, so the dominant low-degree terms come
-    // last and the low-degree outputs see few truncations at full size
-    const bool krev = mode == 1;
-    short *MM = (short *)(smraw + sp.tabs);   // order m of index k = n^2 + n + m (0 beyond P)
+    const int NR = (int)sp.NR, nchunk = (int)sp.nchunk, ST = (int)sp.ST;
     uint64_t *bars = (uint64_t *)(smraw + sp.bars);
     uint64_t *tfull = bars, *tempty = bars + V2_ST_MAX, *xfull = bars + 2 * V2_ST_MAX,
              *xempty = xfull + V2_SX;
     uint64_t *accfull = xempty + V2_SX, *accempty = accfull + 1, *metafull = accfull + 2,
              *fin = accfull + 6, *ydone = accfull + 7, *yfree = accfull + 8;
     uint32_t *tslot = (uint32_t *)(accfull + 9);
-    auto meta_G = [&](int slot) { return (cf *)(smraw + sp.meta + slot * sp.meta_bytes); };
-    auto meta_O = [&](int slot) { return (cf *)(smraw + sp.meta + slot * sp.meta_bytes + sp.g_bytes); };
-    auto meta_cols = [&](int slot) {
-        return (V2Col *)(smraw + sp.meta + slot * sp.meta_bytes + 2 * sp.g_bytes);
-    };
-
-    // the arrays of an item's problem: the launch's own, or a batch entry
-    auto prob = [&](const M2LWork &w) {
-        if (probs) return probs[w.prob];
-        return TcProb{geoms, pairs, ephase, timg, me, le};
-    };
+    auto meta_cols = [&](int slot) { return (V2Col *)(smraw + sp.meta + slot * sp.meta_bytes); };
 
     float *Y = yscr + (size_t)blockIdx.x * NR * 128;   // [complex column][r], complex
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -647,12 +521,6 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
         tc::mbar_init(yfree, V2_ET);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
-    for (int k = tid; k < (int)sp.mm_n; k += V2_THREADS) {
-        int n = (int)sqrtf((float)k + 0.5f);
-        while ((n + 1) * (n + 1) <= k) ++n;
-        while (n * n > k) --n;
-        MM[k] = k < P ? (short)(k - n * n - n) : (short)0;
-    }
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -666,16 +534,14 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
             int s = 0;
             for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x) {
                 const M2LWork w = work[it];
-                const TcProb pd = prob(w);
-                const int64_t ti = mode == 0 ? pd.geoms[w.geom].tab_index * NTAB + w.t : (int64_t)w.geom;
-                const unsigned char *src = (const unsigned char *)pd.img + (size_t)ti * nchunk * sp.CB;
+                const unsigned char *src = img + (size_t)w.geom * nchunk * sp.CB;
                 for (int c = 0; c < nchunk; ++c) {
                     if (g >= (uint32_t)ST && !tc::mbar_wait(&tempty[s], ph ^ 1, WAIT_POLLS)) {
                         failed = true;
                         break;
                     }
                     tc::mbar_expect_tx(&tfull[s], sp.CB);
-                    tc::bulk_g2s(smraw + s * sp.CB, src + (size_t)(krev ? nchunk - 1 - c : c) * sp.CB, sp.CB,
+                    tc::bulk_g2s(smraw + s * sp.CB, src + (size_t)(nchunk - 1 - c) * sp.CB, sp.CB,
                                  &tfull[s]);
                     ++g;
                     if (++s == ST) {
@@ -760,7 +626,6 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
         uint32_t xph = 0;
         for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x, ++li) {
             const int slot = li & 1;
-            cf *G = meta_G(slot);
             V2Col *cols = meta_cols(slot);
             const M2LWork w = work[it];
             // column data of the item, filled by the epilogue warps
@@ -769,40 +634,18 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
                 failed = true;
                 break;
             }
-            const int ncol = v2_ncol(w, mode);
+            const int ncol = 3 * w.npair;
             const bool valid = cc < ncol;
-            V2Col q{};
-            if (valid) q = cols[cc];
-            const bool neg = q.kap < 0;
-            const uint32_t gr = tc::smem_u32(G + q.pp * MO + p);   // input factors of the column
-            const cf *pme = prob(w).me;
-            const cf *src = pme + q.in_base;
+            const cf *src = valid ? in + cols[cc].in_base : in;
             constexpr int KQ = 4;                  // inputs per lane and chunk
             const int kk0 = 8 * pg + KQ * b;       // first of them within the chunk
             float2 pre[V2_D][KQ];
-            const uint32_t mm0 = tc::smem_u32(MM);
-            // orders m' of this lane's inputs (one 8-byte load of the order table)
-            auto orders = [&](int ch, int(&mo)[KQ]) {
-                uint32_t w0, w1;
-                asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(w0), "=r"(w1) : "r"(mm0 + 2 * (V2_KC * ch + kk0)));
-                mo[0] = (int)(short)(w0 & 0xffff);
-                mo[1] = (int)(short)(w0 >> 16);
-                mo[2] = (int)(short)(w1 & 0xffff);
-                mo[3] = (int)(short)(w1 >> 16);
-            };
-            // input (n', m') reads the expansion at (n', +-m'): index k or k - 2m'.
             // Loads are unconditional (from a clamped address) so that they stay in
             // flight until their use V2_D chunks later; the mask is applied there.
             auto fetch = [&](int c, float2(&v)[KQ]) {
-                const int ch = krev ? nchunk - 1 - c : c;
-                int mo[KQ];
-                orders(ch, mo);
+                const int ch = nchunk - 1 - c;
 #pragma unroll
-                for (int h = 0; h < KQ; ++h) {
-                    const int k = min(V2_KC * ch + kk0 + h, P - 1);
-                    const cf *a = valid ? src + (neg ? k - 2 * mo[h] : k) : pme;
-                    v[h] = *(const float2 *)a;
-                }
+                for (int h = 0; h < KQ; ++h) v[h] = *(const float2 *)(src + min(V2_KC * ch + kk0 + h, P - 1));
             };
 #pragma unroll
             for (int u = 0; u < V2_D; ++u)
@@ -812,23 +655,21 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
                 for (int u = 0; u < V2_D; ++u) {
                     const int c = c0 + u;
                     if (c >= nchunk) break;
-                    const int ch = krev ? nchunk - 1 - c : c;   // data chunk
+                    const int ch = nchunk - 1 - c;   // data chunk
                     bool okw = g < (uint32_t)V2_SX || tc::mbar_wait(&xempty[xs], xph ^ 1, WAIT_POLLS);
                     if (__any_sync(0xffffffffu, !okw)) {
                         failed = true;
                         break;
                     }
                     tc::fence_after();
-                    int mo[KQ];
-                    orders(ch, mo);
-                    // the lane's four inputs, phase-shifted and split once: word j of
+                    // the lane's four inputs, split once: word j of
                     // input h holds piece j of (Re, Im)
                     uint32_t own[KQ][V2_NPC], oth[KQ][V2_NPC];
 #pragma unroll
                     for (int h = 0; h < KQ; ++h) {
                         cf y{0.f, 0.f};
                         if (valid && V2_KC * ch + kk0 + h < P)
-                            y = lds_cf(gr + 8 * (neg ? -mo[h] : mo[h])) * cf{pre[u][h].x, pre[u][h].y};
+                            y = cf{pre[u][h].x, pre[u][h].y};
                         v2_split_bf16(y.x, y.y, own[h]);
                     }
 #pragma unroll
@@ -873,17 +714,9 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
         const int q4 = warp & 3, half = ea / 128;     // lane quadrant, slab parity
         const uint32_t lane_base = tbase + ((uint32_t)(32 * q4) << 16);
         const int ew = ea >> 5;                       // epilogue warp 0 .. V2_EW-1
-        int rm[V2_RJ];                                // order m of rows lane + 32 i
-#pragma unroll
-        for (int i = 0; i < V2_RJ; ++i) rm[i] = MM[min(lane + 32 * i, P - 1)];
         // column data of item w into meta slot `slot`, then release it to the producers
         auto fill = [&](const M2LWork &w, int slot) {
-            const TcProb pd = prob(w);
-            if (mode == 0)
-                v2_fill_meta(p, P, w, pd.pairs, pd.ephase, (w.flags & 1) != 0, (w.flags & 2) != 0, meta_G(slot),
-                             meta_O(slot), meta_cols(slot), ea, V2_ET);
-            else
-                v2_fill_trans(p, P, w, tsrc, tdst, meta_G(slot), meta_O(slot), meta_cols(slot), ea, V2_ET);
+            v2_fill(P, w, tsrc, tdst, meta_cols(slot), ea, V2_ET);
             tc::mbar_arrive(&metafull[slot]);
         };
         for (int i = 0; i < 2; ++i)
@@ -934,9 +767,7 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
                 failed = true;
                 break;
             }
-            const int ncol = v2_ncol(wc, mode);
-            cf *const ple = prob(wc).le;
-            const cf *O = meta_O(slot);
+            const int ncol = 3 * wc.npair;
             const V2Col *cols = meta_cols(slot);
             // one column per epilogue warp at a time, two in flight: lane j of a
             // column takes rows r = lane + 32 i; the column record is warp-uniform
@@ -955,18 +786,11 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
                 for (int h = 0; h < 2; ++h) {
                     if (h == 1 && !two) break;
                     const int cc = h ? c2 : c;
-                    const V2Col &cq = cols[cc];
-                    const int64_t ob = cq.out_base;
-                    const bool kneg = cq.kap < 0;
-                    const cf *Oc = O + cc * MO + p;
+                    cf *o = out + cols[cc].out_base;
 #pragma unroll
                     for (int i = 0; i < V2_RJ; ++i) {
                         const int r = lane + 32 * i;
-                        if (r < P) {
-                            const cf yy = Oc[rm[i]] * cf{y[h][i].x, y[h][i].y};
-                            // output (nu, mu) with mu = +-mh: index r or r - 2 mh
-                            atomicAdd((float2 *)(ple + ob + (kneg ? r - 2 * rm[i] : r)), make_float2(yy.x, yy.y));
-                        }
+                        if (r < P) atomicAdd((float2 *)(o + r), y[h][i]);
                     }
                 }
             }
@@ -1003,48 +827,6 @@ __host__ __device__ inline size_t v2_img_off(int r, int kk)
     return (size_t)(((r >> 3) * 256 + (kk >> 3) * 128 + (r & 7) * 16 + (kk & 7) * 2) >> 1);
 }
 
-// table image of the persistent kernel: per (geometry, table) nchunk * V2_KS
-// K-steps (zero beyond P), each V2_NPC bf16 planes of NR rows x 16 real K,
-// from the FP64 table with the level scaling s_t^nu s_s^n' and the degree
-// factors (-i)^nu f_t^nu, i^n' f_s^n' applied before the split
-__global__ void k_tile_tables(int p, int64_t g0, int64_t ng, const GeomDev *geoms, const CompDev *comps,
-                              const cd *tab64, __nv_bfloat16 *img)
-{
-    const int P = (p + 1) * (p + 1);
-    const V2Plan sp = v2_plan(p);
-    const int NR = (int)sp.NR, nsub = (int)sp.nchunk * V2_KS;
-    const int64_t gi = g0 + blockIdx.y;
-    const int t = blockIdx.z;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= nsub * NR * 8 || gi >= g0 + ng) return;
-    const int c = e / (NR * 8), rem = e % (NR * 8), r = rem >> 3, i = rem & 7;   // input 8c + i
-    const int k = 8 * c + i;
-    const GeomDev &g = geoms[gi];
-    cd v{0.0, 0.0};
-    if (r < P && k < P) {
-        int nu = (int)sqrt((double)r + 0.5), n1 = (int)sqrt((double)k + 0.5);
-        while ((nu + 1) * (nu + 1) <= r) ++nu;
-        while (nu * nu > r) --nu;
-        while ((n1 + 1) * (n1 + 1) <= k) ++n1;
-        while (n1 * n1 > k) --n1;
-        const CompDev cp = comps[g.comp];
-        const bool flip_in = (cp.s < 0) != (cp.has_src_refl != 0);
-        const bool flip_out = (cp.s < 0) != (cp.has_tgt_refl != 0);
-        const double f = pow(g.scale_t, (double)nu) * pow(g.scale_s, (double)n1) *
-                         ((flip_in && (n1 & 1)) ? -1.0 : 1.0) * ((flip_out && (nu & 1)) ? -1.0 : 1.0);
-        const cd a = tab64[((gi - g0) * NTAB + t) * (int64_t)P * P + (int64_t)r * P + k];
-        v = ipow<double>(n1 - nu) * (f * a);   // i^n' (-i)^nu = i^(n' - nu)
-    }
-    __nv_bfloat16 re[V2_NPC], im[V2_NPC];
-    v2_split3(v.x, re);
-    v2_split3(v.y, im);
-    __nv_bfloat16 *sub = img + ((size_t)(g.tab_index * NTAB + t) * nsub + c) * (size_t)(NR * 16 * V2_NPC);
-    for (int pc = 0; pc < V2_NPC; ++pc) {
-        sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i)] = re[pc];
-        sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i + 1)] = im[pc];
-    }
-}
-
 namespace {
 int tc_mtiles(int p) { return (2 * (p + 1) * (p + 1) + 127) / 128; }
 uint32_t tc_tmem_cols(int MT)
@@ -1078,71 +860,26 @@ cudaError_t launch_m2l_tc(int p, int64_t nwork, const M2LWork *work, const GeomD
     return cudaGetLastError();
 }
 
-bool m2l_tc2_supported(int p)
+bool trans_tc2_supported(int p)
 {
     return p >= 1 && v2_plan(p).NR <= (uint32_t)V2_NR_MAX && 2 * v2_plan(p).NR + V2_SX * V2_XW <= 512 &&
            v2_plan(p).ST >= 4;
 }
 
-size_t m2l_tc2_image_bytes(int p, int64_t ngeom)
-{
-    const V2Plan sp = v2_plan(p);
-    return (size_t)ngeom * NTAB * sp.nchunk * sp.CB;
-}
-
-size_t m2l_tc2_scratch_floats(int p, int nsm) { return (size_t)nsm * 128 * v2_plan(p).NR; }
-
-void launch_tile_tables(int p, int64_t g0, int64_t ng, const GeomDev *geoms, const CompDev *comps,
-                        const cd *tab64, void *img, cudaStream_t st)
-{
-    if (ng <= 0) return;
-    const V2Plan sp = v2_plan(p);
-    dim3 grid((sp.nchunk * V2_KS * sp.NR * 8 + 255) / 256, (unsigned)ng, NTAB);
-    k_tile_tables<<<grid, 256, 0, st>>>(p, g0, ng, geoms, comps, tab64, (__nv_bfloat16 *)img);
-}
-
-static cudaError_t launch_tc2(int p, int mode, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-                              const M2LPair *pairs, const cf *ephase, const int64_t *tsrc,
-                              const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
-                              int *status, cudaStream_t st)
-{
-    if (nwork <= 0) return cudaSuccess;
-    if (!m2l_tc2_supported(p) || nsm < 1) return cudaErrorInvalidValue;
-    const int64_t grid = std::min<int64_t>(nwork, (int64_t)nsm);
-    // each CTA takes all 512 tensor-memory columns: ask for more than half of
-    // an SM's shared memory so that no two CTAs are resident on one SM
-    const size_t smem = std::max<size_t>(v2_plan(p).total, 116 * 1024);
-    k_m2l_tc2<<<(unsigned)grid, V2_THREADS, smem, st>>>(p, mode, nwork, work, geoms, pairs, ephase, tsrc,
-                                                        tdst, (const uint32_t *)img, in, out, yscr, status, nullptr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_m2l_tc2_batch(int p, int64_t nwork, const M2LWork *work, const TcProb *probs, float *yscr,
-                                 int nsm, int *status, cudaStream_t st)
-{
-    if (nwork <= 0) return cudaSuccess;
-    if (!m2l_tc2_supported(p) || nsm < 1) return cudaErrorInvalidValue;
-    const int64_t grid = std::min<int64_t>(nwork, (int64_t)nsm);
-    const size_t smem = std::max<size_t>(v2_plan(p).total, 116 * 1024);
-    k_m2l_tc2<<<(unsigned)grid, V2_THREADS, smem, st>>>(p, 0, nwork, work, nullptr, nullptr, nullptr, nullptr,
-                                                        nullptr, nullptr, nullptr, nullptr, yscr, status, probs);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_m2l_tc2(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-                           const M2LPair *pairs, const cf *ephase, const void *img,
-                           const cf *me, cf *le, float *yscr, int nsm, int *status, cudaStream_t st)
-{
-    return launch_tc2(p, 0, nwork, work, geoms, pairs, ephase, nullptr, nullptr, img, me, le, yscr, nsm,
-                      status, st);
-}
+size_t trans_tc2_scratch_floats(int p, int nsm) { return (size_t)nsm * 128 * v2_plan(p).NR; }
 
 cudaError_t launch_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc,
                              const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
                              int *status, cudaStream_t st)
 {
-    return launch_tc2(p, 1, nwork, work, nullptr, nullptr, nullptr, tsrc, tdst, img, in, out, yscr, nsm,
-                      status, st);
+    if (nwork <= 0) return cudaSuccess;
+    if (!trans_tc2_supported(p) || nsm < 1) return cudaErrorInvalidValue;
+    // each CTA takes all 512 tensor-memory columns: ask for more than half of
+    // an SM's shared memory so that no two CTAs are resident on one SM
+    const size_t smem = std::max<size_t>(v2_plan(p).total, 116 * 1024);
+    k_trans_tc2<<<(unsigned)std::min<int64_t>(nwork, (int64_t)nsm), V2_THREADS, smem, st>>>(
+        p, nwork, work, tsrc, tdst, (const unsigned char *)img, in, out, yscr, status);
+    return cudaGetLastError();
 }
 
 size_t tc2_matrix_bytes(int p)
@@ -1178,7 +915,8 @@ cudaError_t configure_m2l_tc()
 {
     cudaError_t e = cudaFuncSetAttribute(k_m2l_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_m2l_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize, V2_SMEM_MAX);
+    e = cudaFuncSetAttribute(k_trans_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize, V2_SMEM_MAX);
+    return e != cudaSuccess ? e : configure_m2l_sec();
 }
 
 }  // namespace lmf

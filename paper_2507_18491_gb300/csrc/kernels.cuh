@@ -66,15 +66,14 @@ struct M2LWork {        // one M2L table applied to a chunk of pairs of one geom
     int prob, pad;      // problem of a batched launch (TcProb index), else 0
 };
 
-// per-problem arrays of a batched persistent M2L launch (k_m2l_tc2): one
-// problem's geometries, pairs, pair phases, table image and scales, and its
-// multipole / local expansions
+// per-problem arrays of a persistent M2L launch (k_m2l_sec): one problem's pairs,
+// pair phases and matrix image (one block per geometry), its packed multipole expansions
+// and its local expansions
 struct TcProb {
-    const GeomDev *geoms;
     const M2LPair *pairs;
     const cf *ephase;
     const void *img;
-    const cf *me;
+    const void *me;
     cf *le;
 };
 
@@ -148,29 +147,36 @@ cudaError_t configure_m2l_tc();
 cudaError_t launch_m2l_tc(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
                           const CompDev *comps, const M2LPair *pairs, const cf *tab, const cf *me,
                           cf *le, int *status, cudaStream_t st);
-// persistent warp-specialised variant (p <= 12) on a pre-tiled image of the
-// tables in three bf16 pieces (launch_tile_tables from the FP64 tables);
-// ephase holds e^{i d phi} of every pair, d = -(p+2)..p+2 ([npair][2p+5],
-// FP32 from FP64); yscr holds m2l_tc2_scratch_floats(p, nsm) floats, nsm =
-// CTAs of the launch (the SM count)
-bool m2l_tc2_supported(int p);
-size_t m2l_tc2_image_bytes(int p, int64_t ngeom);
-size_t m2l_tc2_scratch_floats(int p, int nsm);
-void launch_tile_tables(int p, int64_t g0, int64_t ng, const GeomDev *geoms, const CompDev *comps,
-                        const cd *tab64, void *img, cudaStream_t st);
-cudaError_t launch_m2l_tc2(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-                           const M2LPair *pairs, const cf *ephase, const void *img,
-                           const cf *me, cf *le, float *yscr, int nsm, int *status, cudaStream_t st);
-// the M2L of several problems (same p) in one persistent launch: work items
-// carry their problem index into probs (device array)
-cudaError_t launch_m2l_tc2_batch(int p, int64_t nwork, const M2LWork *work, const TcProb *probs, float *yscr,
-                                 int nsm, int *status, cudaStream_t st);
-// M2M or L2L on the same kernel: items M2LWork{geom = translation group, t = 0,
+// k_m2l_sec.cu: persistent tensor-core M2L of the mixed form (p <= 12) on the mirror
+// sectors of sector.cuh.  Items M2LWork{geom, npair <= 64, pair0, prob}; img is the
+// image of the sector matrices in three bf16 pieces (launch_sec_image from the FP64
+// tables); ephase holds G[d] = i^d e^{i d phi} of every pair, d = -(p+1)..p, in rows of
+// m2l_sec_phases(p) entries (FP32 from FP64); yscr holds m2l_sec_scratch_floats(p, nsm)
+// floats, nsm = CTAs of the launch (the SM count)
+bool m2l_sec_supported(int p);
+int m2l_sec_pairs();             // pairs of a full work item
+int m2l_sec_phases(int p);
+size_t m2l_sec_image_bytes(int p, int64_t ngeom);
+size_t m2l_sec_scratch_floats(int p, int nsm);
+cudaError_t configure_m2l_sec();
+void launch_sec_image(int p, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64, void *img,
+                      cudaStream_t st);
+void launch_pair_phases(int p, int64_t npair, const M2LPair *pairs, cf *out, cudaStream_t st);
+// packs the multipole expansions me into what the kernel reads (TcProb::me,
+// m2l_sec_packed_bytes) and clears the local expansions le
+size_t m2l_sec_packed_bytes(int p, int64_t nbox);
+void launch_sec_pack(int p, int64_t nbox, const cf *me, void *packed, cf *le, cudaStream_t st);
+// probs: the problems of a batched launch (device array), or null with one problem in `one`
+cudaError_t launch_m2l_sec(int p, int64_t nwork, const M2LWork *work, const TcProb &one, const TcProb *probs,
+                           float *yscr, int nsm, int *status, cudaStream_t st);
+// M2M or L2L on a persistent tensor-core kernel (k_m2l_tc.cu, p <= 12): items M2LWork{geom = translation group, t = 0,
 // npair, pair0} over pairs (tsrc[q], tdst[q]), 3 helical columns each; img holds
 // one tiled matrix per group (tile_matrix_tc2, tc2_matrix_bytes(p) each)
 cudaError_t launch_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc,
                              const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
                              int *status, cudaStream_t st);
+bool trans_tc2_supported(int p);
+size_t trans_tc2_scratch_floats(int p, int nsm);
 size_t tc2_matrix_bytes(int p);
 void tile_matrix_tc2(int p, const cd *M, void *img);   // host: P x P row-major (row = output index)
 template <typename T>
