@@ -55,9 +55,10 @@ struct DevState {
     int64_t n_s2twork = 0;
     S2TRowT *s2tworkT = nullptr;     // transposed near field: (near pair, source) rows
     int64_t n_s2tworkT = 0;
-    int64_t *fpairs = nullptr;       // free-space near leaf pairs [n][2] (source, target)
-    S2TRowT *frows = nullptr, *frowsT = nullptr;   // ... by target / by source point
-    int64_t n_frows = 0, n_frowsT = 0;
+    // free-space near field: runs of sorted points near every leaf, as target / as source
+    int *froff = nullptr, *froffT = nullptr, *fbox = nullptr;
+    FreeRun *fruns = nullptr, *frunsT = nullptr;
+    bool free_near = false;
     // position gradient (allocated by the first lmfmm_gradient call): checkpoints
     // of the forward pass's local expansions and helical charges, a field buffer,
     // and 20 derivative integrals per near point pair
@@ -794,22 +795,36 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         }
         TRY(dupload(ctx, &d->s2tworkT, swT));
         d->n_s2tworkT = (int64_t)swT.size();
-        // free-space near field
-        std::vector<int64_t> fp;
-        std::vector<S2TRowT> fr, frT;
-        for (size_t i = 0; i < ctx->free_near.size(); ++i) {
-            const auto &pr = ctx->free_near[i];
-            fp.push_back(pr.first);
-            fp.push_back(pr.second);
-            const Box &bs = ctx->boxes[pr.first], &bt = ctx->boxes[pr.second];
-            for (int64_t ii = 0; ii < bt.p1 - bt.p0; ++ii) fr.push_back(S2TRowT{(int64_t)i, (int)ii, 0});
-            for (int64_t jj = 0; jj < bs.p1 - bs.p0; ++jj) frT.push_back(S2TRowT{(int64_t)i, (int)jj, 0});
+        // free-space near field: the near leaves of a leaf, consecutive sorted points joined
+        d->free_near = !ctx->free_near.empty();
+        if (d->free_near) {
+            std::vector<int> fb(N, 0);
+            for (int64_t li : leaves)
+                for (int64_t q = ctx->boxes[li].p0; q < ctx->boxes[li].p1; ++q) fb[q] = (int)li;
+            TRY(dupload(ctx, &d->fbox, fb));
+            for (int tr = 0; tr < 2; ++tr) {
+                std::vector<std::pair<int64_t, int64_t>> pr(ctx->free_near.size());   // (row leaf, column leaf)
+                for (size_t i = 0; i < pr.size(); ++i) {
+                    pr[i] = ctx->free_near[i];
+                    if (!tr) std::swap(pr[i].first, pr[i].second);
+                }
+                std::sort(pr.begin(), pr.end());
+                std::vector<int> off(nbox + 1, 0);
+                std::vector<FreeRun> runs;
+                size_t i = 0;
+                for (int64_t b = 0; b < nbox; ++b) {
+                    const size_t r0 = runs.size();
+                    for (; i < pr.size() && pr[i].first == b; ++i) {
+                        const Box &c = ctx->boxes[pr[i].second];
+                        if (runs.size() > r0 && runs.back().p0 + runs.back().n == c.p0) runs.back().n += (int)(c.p1 - c.p0);
+                        else runs.push_back(FreeRun{c.p0, (int)(c.p1 - c.p0), 0});
+                    }
+                    off[b + 1] = (int)runs.size();
+                }
+                TRY(dupload(ctx, tr ? &d->froffT : &d->froff, off));
+                TRY(dupload(ctx, tr ? &d->frunsT : &d->fruns, runs));
+            }
         }
-        TRY(dupload(ctx, &d->fpairs, fp));
-        TRY(dupload(ctx, &d->frows, fr));
-        TRY(dupload(ctx, &d->frowsT, frT));
-        d->n_frows = (int64_t)fr.size();
-        d->n_frowsT = (int64_t)frT.size();
     }
     TRY(check_flag(ctx));
     ctx->built = true;
@@ -968,8 +983,10 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
     leaf_l2p<T>(ctx, le, d->ph, false, st);
     CK(cudaEventRecord(d->ev[5], st));
     launch_s2t_apply8(d->n_s2twork, d->s2twork, d->near, d->boxes, d->s2t, d->qh, d->ph, st);
-    launch_p2p_free(d->n_frows, d->frows, d->fpairs, d->boxes, d->xyz, ctx->med, d->qh, d->ph, false, st);
-    nl += d->n_frows > 0;
+    if (d->free_near) {
+        launch_p2p_free(N, d->fbox, d->froff, d->fruns, d->boxes, d->xyz, ctx->med, d->qh, d->ph, false, st);
+        ++nl;
+    }
     CK(cudaEventRecord(d->ev[6], st));
     launch_scatter_out(N, d->perm, d->ph, Phi, dtype, cj, st);
     nl += (d->nleaves > 0) + (d->n_s2twork > 0) + (N > 0);   // L2P, near field, scatter
@@ -1022,8 +1039,10 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     leaf_l2p<T>(ctx, me, d->qh, true, st);
     CK(cudaEventRecord(d->ev[5], st));
     launch_s2t_apply8_tr(d->n_s2tworkT, d->s2tworkT, d->near, d->boxes, d->s2t, d->ph, d->qh, st);
-    launch_p2p_free(d->n_frowsT, d->frowsT, d->fpairs, d->boxes, d->xyz, ctx->med, d->ph, d->qh, true, st);
-    nl += d->n_frowsT > 0;
+    if (d->free_near) {
+        launch_p2p_free(N, d->fbox, d->froffT, d->frunsT, d->boxes, d->xyz, ctx->med, d->ph, d->qh, true, st);
+        ++nl;
+    }
     CK(cudaEventRecord(d->ev[6], st));
     launch_scatter_tr(N, d->perm, d->qh, out, dtype, cj, st);
     nl += (d->nleaves > 0) + (d->n_s2tworkT > 0) + (N > 0);

@@ -207,10 +207,14 @@ struct S2TRowT {
 };
 void launch_s2t_apply8_tr(int64_t nrow, const S2TRowT *rows, const NearPair *near, const BoxDev *boxes,
                           const cd *coef8, const cd *phb, cd *qhb, cudaStream_t st);
-// free-space near field over leaf pairs ([2 * pair] = source leaf, [+1] =
-// target leaf); rows {pair, point index within the row box}: targets (forward,
-// out = ph) or sources (transposed, out = qh_bar)
-void launch_p2p_free(int64_t nrow, const S2TRowT *rows, const int64_t *pairs, const BoxDev *boxes,
+// free-space near field: per leaf box b the runs [roff[b], roff[b + 1]) of sorted points
+// near it, one warp per sorted point (pt_box: its leaf).  Forward: points are targets, out =
+// ph; transposed: points are sources, out = qh_bar
+struct FreeRun {
+    int64_t p0;
+    int n, pad;
+};
+void launch_p2p_free(int64_t N, const int *pt_box, const int *roff, const FreeRun *runs, const BoxDev *boxes,
                      const double *xyz, const MediumDev &M, const cd *in, cd *out, bool transposed, cudaStream_t st);
 // transposes of the helical maps: ph_bar = S^T y (caller order -> sorted),
 // out = G^T qh_bar (sorted -> caller order), optional conjugation of y / out
