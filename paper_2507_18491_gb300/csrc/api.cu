@@ -68,6 +68,10 @@ struct DevState {
     int m2l_kernel = 0;              // 0 FP64 SIMT, 1 FP32 SIMT, 2 tcgen05 streamed, 3 tcgen05 persistent
     cf *ephase = nullptr;            // sector kernel: phases G[d] per pair
     void *mepk = nullptr;            // ... and the packed multipole expansions it reads
+    // FP64 form on the tensor cores (k_m2l_oz.cu): images of the sector blocks and their
+    // transposes, packed inputs, per-CTA scratch
+    bool oz = false;
+    void *ozimg = nullptr, *ozimgT = nullptr, *ozpk = nullptr, *ozscr = nullptr;
     int nsm = 0;
     cd *stage = nullptr;             // [2][N][3] for host-buffer matvec
     cudaEvent_t ev[9]{};
@@ -491,6 +495,14 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
                    std::to_string(fr / 1e9) + " GB free (reduce p or raise theta/depth)";
         return LMFMM_ERR_OOM;
     }
+    CK(cudaDeviceGetAttribute(&d->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
+    // FP64 form: the tensor-core M2L holds two images of 16 bytes per sector entry (the SIMT
+    // kernels one table of 16 bytes); where both do not fit, the SIMT kernels run
+    if (ctx->prm.precision == LMFMM_FP64 && m2l_oz_supported(p)) {
+        const double oz_need = 2.0 * (double)m2l_oz_image_bytes(p, (int64_t)ctx->geoms.size()) +
+                               (double)m2l_oz_packed_bytes(p, nbox) + (double)m2l_oz_scratch_bytes(p, d->nsm);
+        d->oz = need + oz_need <= 0.85 * (double)fr;
+    }
     CK(cudaMalloc((void **)&d->flag, sizeof(int)));
     d->allocs.push_back(d->flag);
     CK(cudaMemset(d->flag, 0, sizeof(int)));
@@ -610,7 +622,6 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             CK(cudaStreamSynchronize(st));
             dfree(ctx, tab64);
             d->tab = img;
-            CK(cudaDeviceGetAttribute(&d->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
             // one scratch for the M2L and the translations, which run one after the other
             TRY(dalloc(ctx, &d->yscr, std::max(m2l_sec_scratch_floats(p, d->nsm), trans_tc2_scratch_floats(p, d->nsm))));
         } else if (f32) {
@@ -621,6 +632,22 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             CK(cudaStreamSynchronize(st));
             dfree(ctx, tab64);
             d->tab = t32;
+        } else if (d->oz) {
+            const int64_t ng = (int64_t)hg.size();
+            unsigned char *q[4] = {};
+            TRY(dalloc(ctx, &q[0], m2l_oz_image_bytes(p, ng)));
+            TRY(dalloc(ctx, &q[1], m2l_oz_image_bytes(p, ng)));
+            TRY(dalloc(ctx, &q[2], m2l_oz_packed_bytes(p, nbox)));
+            TRY(dalloc(ctx, &q[3], m2l_oz_scratch_bytes(p, d->nsm)));
+            launch_oz_image(p, false, ng, d->geoms, d->comps, tab64, q[0], st);
+            launch_oz_image(p, true, ng, d->geoms, d->comps, tab64, q[1], st);
+            CK(cudaGetLastError());
+            CK(cudaStreamSynchronize(st));
+            dfree(ctx, tab64);
+            d->ozimg = q[0];
+            d->ozimgT = q[1];
+            d->ozpk = q[2];
+            d->ozscr = q[3];
         } else {
             launch_scale_tables<double>(p, 0, (int64_t)hg.size(), d->geoms, tab64, tab64, st);
             CK(cudaGetLastError());
@@ -638,6 +665,13 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         launch_pair_phases(p, (int64_t)ctx->m2l.size(), d->m2l, d->ephase, st);
         CK(cudaGetLastError());
         sec_work_items(ctx, m2l_sec_pairs(), 0, mw);
+    } else if (d->oz) {
+        // smaller items where full ones would leave SMs idle
+        for (int pairs = m2l_oz_pairs(); pairs >= m2l_oz_pairs() / 4; pairs /= 2) {
+            mw.clear();
+            sec_work_items(ctx, pairs, 0, mw);
+            if ((int64_t)mw.size() >= d->nsm) break;
+        }
     } else {
         m2l_work_items(ctx, d->m2l_kernel == 2 ? m2l_tc_cols() : f32 ? gemm_cols<float>() : gemm_cols<double>(), 0, mw);
     }
@@ -842,7 +876,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     S.n_near_point_pairs = ctx->n_near_pp;
     S.n_quad_nodes = qtot;
     S.bytes_tables = d->m2l_kernel == 3 ? (double)m2l_sec_image_bytes(p, (int64_t)ctx->geoms.size())
-                     : (double)ctx->geoms.size() * NTAB * P * P * (f32 ? 8.0 : 16.0);
+                     : d->oz ? 2.0 * (double)m2l_oz_image_bytes(p, (int64_t)ctx->geoms.size())
+                             : (double)ctx->geoms.size() * NTAB * P * P * (f32 ? 8.0 : 16.0);
     S.ms_setup = std::chrono::duration<double, std::milli>(t1 - t0).count();
     S.m2l_columns = ncols;
     S.m2l_kernel = d->m2l_kernel;
@@ -934,7 +969,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
     }
     if (parts & MV_M2L) {
     nl += d->n_m2lwork > 0;   // M2L
-    bool packed = false;
+    bool packed = d->oz;   // the tensor-core kernels clear le themselves
     if constexpr (std::is_same<T, float>::value) {
         if (d->m2l_kernel == 3) {
             launch_sec_pack(p, nbox, me, d->mepk, le, st);   // clears le too
@@ -956,6 +991,10 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
         else
             launch_m2l_t<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
                             (const cx<T> *)d->tab, me, le, st);
+    } else if (d->oz) {
+        CK(launch_m2l_oz(p, false, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimg, nbox, me, le,
+                         d->ozpk, d->ozscr, d->nsm, d->mvstatus, st));
+        ++nl;
     } else {
         launch_m2l_t<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
                         (const cx<T> *)d->tab, me, le, st);
@@ -1026,8 +1065,19 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
         nl += w1 > w0;
     }
     CK(cudaEventRecord(d->ev[2], st));
-    CK(cudaMemsetAsync(me, 0, (size_t)nbox * 3 * P * sizeof(cx<T>), st));
-    launch_m2l_tr<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l, (const cx<T> *)d->tab, le, me, st);
+    bool done = false;
+    if constexpr (std::is_same<T, double>::value) {
+        if (d->oz) {
+            CK(launch_m2l_oz(p, true, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimgT, nbox, le, me,
+                             d->ozpk, d->ozscr, d->nsm, d->mvstatus, st));
+            done = true;
+            ++nl;
+        }
+    }
+    if (!done) {
+        CK(cudaMemsetAsync(me, 0, (size_t)nbox * 3 * P * sizeof(cx<T>), st));
+        launch_m2l_tr<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l, (const cx<T> *)d->tab, le, me, st);
+    }
     nl += d->n_m2lwork > 0;
     CK(cudaEventRecord(d->ev[3], st));
     for (int lev = 1; lev <= ctx->depth; ++lev) {   // M2M^T: parents into children

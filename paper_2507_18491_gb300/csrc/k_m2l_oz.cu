@@ -1,0 +1,516 @@
+// M2L of the FP64 form, and its transpose, on the 5th-generation tensor cores (tcgen05), on
+// the mirror sectors of sector.cuh.
+//
+// The chip has 2 FP64 multiply-adds per clock and SM but 4096 bf16 ones, so the contraction
+// runs on integers (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59 (2012), with digits on a common grid per row): every operand is a 64-bit
+// fixed-point number, written as eight signed base-256 digits (a bf16 holds every integer
+// up to 256), and the products of digits i and j are summed per diagonal d = i + j in an FP32
+// accumulator of its own.  Digits are at most 128 in size, so a diagonal's sum over K real
+// inputs is an integer below (d + 1) K 2^14: exact (below 2^24) for d = 0 up to K = 1024, and
+// for the later diagonals, whose digits are spread evenly over +-128, sqrt(K) instead of K.
+// The 36 products with d <= 7 are formed; what is left out is 2^-64 of the largest entry, 11
+// bits below an FP64 rounding.  The eight sums are put together as 64-bit integers and
+// converted once.
+//
+// Grids: the matrix rows carry their own power of two; the inputs carry one per
+// source box, after the degrees have been brought to one size by 2^c_n ~ (2n + 1)!! (the
+// scaled expansions fall like 1/(2n + 1)!!, the matrix columns grow like it and take 2^-c_n).
+//
+// One CTA per SM walks the work items (up to 64 pairs of one geometry).  Per sector: all
+// threads form the inputs (FP64 phases, digits by integer operations) into a per-CTA image
+// in global memory (L2), then per tile of 64 matrix rows one thread streams input and matrix
+// K-steps through a shared ring, one issues the MMAs (8 accumulators x 64 columns: all of
+// tensor memory; consecutive MMAs go to different accumulators), and all threads turn the
+// accumulators into FP64 sums in a scratch.  At the end one warp per pair combines the two
+// sectors and adds [3][P] with one bulk reduction.  The FP64 pipe (phases, conversions) and
+// the ring's traffic bound it, not the MMAs.  Every wait is bounded; a wait that gives up
+// sets bit 4 of the status word.
+#include <algorithm>
+
+#include "sector.cuh"
+#include "tc.cuh"
+
+namespace lmf {
+
+namespace {
+
+constexpr int OZ_S = 8;            // digits
+constexpr int OZ_BN = 64;          // pairs per work item
+constexpr int OZ_NT = 64;          // matrix rows per tile
+constexpr int OZ_T = 512;          // threads
+constexpr int OZ_W = OZ_T / 32;
+constexpr int OZ_ST = 3;           // ring slots
+constexpr uint32_t OZ_A = OZ_S * 128 * 32;          // bytes of an input K-step (8 complex inputs)
+constexpr uint32_t OZ_SLOT = OZ_A + OZ_S * OZ_NT * 32;
+constexpr int OZ_POLLS = 1 << 22;
+constexpr int OZ_PMAX = 16;
+
+struct OzPlan {
+    int p, P, D[2], nk[2], rows;   // rows: D0 + D1
+    uint32_t sec_img[2], img_bytes;
+    uint32_t o_ph, o_ent, o_pair, o_bars, smem, ph_bytes, stage_bytes;
+    int out_warps;
+};
+
+__host__ __device__ inline int oz_tile_rows(int D, int t)
+{
+    const int r = D - t * OZ_NT;
+    return r >= OZ_NT ? OZ_NT : (r + 15) & ~15;
+}
+
+OzPlan oz_plan(int p)
+{
+    OzPlan s{};
+    s.p = p;
+    s.P = (p + 1) * (p + 1);
+    uint32_t img = 0;
+    for (int e = 0; e < 2; ++e) {
+        s.D[e] = sec_dim(p, e);
+        s.nk[e] = (s.D[e] + 7) / 8;
+        s.sec_img[e] = img;
+        for (int t = 0; t * OZ_NT < s.D[e]; ++t) img += (uint32_t)(s.nk[e] * OZ_S * oz_tile_rows(s.D[e], t) * 32);
+    }
+    s.img_bytes = img;
+    s.rows = s.D[0] + s.D[1];
+    s.ph_bytes = (uint32_t)(2 * p + 2) * 16 + 16;      // padded against bank conflicts
+    s.stage_bytes = (uint32_t)(3 * s.P) * 16;
+    s.o_ph = OZ_ST * OZ_SLOT;
+    s.o_ent = s.o_ph + OZ_BN * s.ph_bytes;
+    s.o_pair = (s.o_ent + (uint32_t)s.nk[0] * 8 * 4 + 15) & ~15u;
+    s.o_bars = s.o_pair + OZ_BN * (uint32_t)sizeof(M2LPair);
+    s.smem = s.o_bars + (2 * OZ_ST + 2) * 8 + 16;
+    s.out_warps = std::min<int>(OZ_W, (OZ_ST * OZ_SLOT) / s.stage_bytes);
+    return s;
+}
+
+// exponent that brings degree n to the size of degree 0: 2^c_n ~ (2n + 1)!!
+__host__ __device__ inline int oz_cn(int n)
+{
+    double f = 1.0;
+    for (int i = 1; i <= n; ++i) f *= 2.0 * i + 1.0;
+    int e;
+    frexp(f, &e);
+    return e - 1;
+}
+
+struct __align__(16) OzIn {        // one input: its two coefficients
+    double x, y, z, w;
+};
+
+// the eight digits of x, |x| < 1 - 2^-8 (the first digit would leave a byte beyond): x = sum_j s_j 2^(-7 - 8 j), s_j in [-128, 127], as floats'
+// upper halves (bf16, exact).  The fixed-point number comes from the bits of x; adding 128
+// to every digit but the first makes the bytes of the sum the digits plus 128.
+__device__ __forceinline__ void oz_digits(double x, uint32_t (&w)[OZ_S])
+{
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)(u >> 52) & 0x7ff;
+    const unsigned long long man = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
+    const int sh = ex - 1012;                       // x 2^63 = man 2^sh
+    long long q = sh >= 0 ? (long long)(man << (sh > 10 ? 10 : sh)) : (long long)(sh > -64 ? man >> -sh : 0ull);
+    if (u >> 63) q = -q;
+    const unsigned long long t = (unsigned long long)q + 0x8080808080808080ull;   // first digit too: its byte is signed + 128
+    const uint32_t hi = (uint32_t)(t >> 32), lo = (uint32_t)t;
+#pragma unroll
+    for (int j = 0; j < OZ_S; ++j) {
+        const uint32_t b = __byte_perm(j < 4 ? hi : lo, 0x4b000000u, 0x7440 + (3 - (j & 3)));   // 2^23 + byte
+        w[j] = __float_as_uint(__uint_as_float(b) - 8388736.f);                                 // - (2^23 + 128)
+    }
+}
+
+__device__ __forceinline__ void mma_f16_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "l"(da), "l"(db), "r"(idesc), "r"(acc));
+}
+
+__device__ __forceinline__ double2 lds_d2(uint32_t a)
+{
+    double2 v;
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a));
+    return v;
+}
+
+// transposed: the same walk with the matrices transposed, the phases conjugated and the roles
+// of the pair's boxes exchanged (in: local, out: multipole expansions)
+__global__ void __launch_bounds__(OZ_T, 1)
+    k_m2l_oz(const __grid_constant__ OzPlan sp, int transposed, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+             const unsigned char *img, const double *rscale, const OzIn *packed, const double *bscale, cd *out,
+             unsigned char *xscr, double *yscr, int *status)
+{
+    extern __shared__ __align__(1024) unsigned char smraw[];
+    const int p = sp.p, P = sp.P, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint32_t *ent = (uint32_t *)(smraw + sp.o_ent);
+    M2LPair *pr = (M2LPair *)(smraw + sp.o_pair);
+    uint64_t *full = (uint64_t *)(smraw + sp.o_bars), *empty = full + OZ_ST, *accfull = empty + OZ_ST;
+    uint32_t *tslot = (uint32_t *)(accfull + 1);
+    const uint32_t ph0 = tc::smem_u32(smraw + sp.o_ph);
+    unsigned char *X = xscr + (size_t)blockIdx.x * sp.nk[0] * OZ_A;
+    double2 *Y = (double2 *)yscr + (size_t)blockIdx.x * OZ_BN * sp.rows;   // [pair][row]
+    const int D0e = sp.nk[0] * 8;
+
+    if (warp == 0) tc::tmem_alloc(tslot, 512);
+    if (tid == 0) {
+        for (int s = 0; s < OZ_ST; ++s) {
+            tc::mbar_init(&full[s], 1);
+            tc::mbar_init(&empty[s], 1);
+        }
+        tc::mbar_init(accfull, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;");
+    }
+    for (int j = tid; j < D0e; j += OZ_T) ent[j] = j < sp.D[0] ? sec_word(p, j) : 0u;
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tbase = *tslot;
+    bool failed = false;
+    uint32_t g = 0;        // K-steps through the ring so far (producer and MMA thread count alike)
+    uint32_t ntile = 0;    // tiles so far
+
+    for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x) {
+        const M2LWork w = work[it];
+        // pair records and phases G[d] (conjugated for the transpose), d = -(p+1)..p
+        if (tid < w.npair) {
+            const M2LPair q = pairs[w.pair0 + tid];
+            pr[tid] = q;
+            cd b = mul_i(cd{q.cphi, q.sphi}), e{1.0, 0.0};
+            if (transposed) b = conj(b);
+            double2 *row = (double2 *)(smraw + sp.o_ph + tid * sp.ph_bytes) + (p + 1);
+            for (int d = 0; d <= p + 1; ++d) {
+                if (d <= p) row[d] = double2{e.x, e.y};
+                row[-d] = double2{e.x, -e.y};
+                e = e * b;
+            }
+        }
+        __syncthreads();
+        for (int sec = 0; sec < 2 && !failed; ++sec) {
+            const int D = sp.D[sec], nk = sp.nk[sec];
+            // ---- inputs: thread -> (pair, four inputs = 16 bytes of both rows of the pair)
+            for (int e = tid; e < OZ_BN * 2 * nk; e += OZ_T) {
+                const int c = e & (OZ_BN - 1), hk = e / OZ_BN;       // hk: half K-step
+                uint32_t rr[OZ_S][4], ri[OZ_S][4];                    // rows 2c and 2c + 1, one word per input
+                const int64_t box = c < w.npair ? (transposed ? pr[c].tgt : pr[c].src) : 0;
+                const OzIn *src = packed + box * D0e + 4 * hk;
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    cd y{0.0, 0.0};
+                    if (c < w.npair) {
+                        const OzIn v = src[h];
+                        const uint32_t we = ent[4 * hk + h];
+                        const double2 G = lds_d2(ph0 + c * sp.ph_bytes + 16 * ((we >> 20) & 63));
+                        // W entries subtract conj(G) b in the even sector, C entries add conj(G) c
+                        const double s = (int)((we >> 26) & 1) == sec ? -1.0 : 1.0;
+                        const double bx = s * v.z, by = s * v.w;
+                        y.x = fma(G.x, v.x + bx, G.y * (by - v.y));
+                        y.y = fma(G.x, v.y + by, G.y * (v.x - bx));
+                    }
+                    uint32_t wr[OZ_S], wi[OZ_S];
+                    oz_digits(y.x, wr);
+                    oz_digits(y.y, wi);
+#pragma unroll
+                    for (int j = 0; j < OZ_S; ++j) {
+                        rr[j][h] = __byte_perm(wr[j], wi[j] ^ 0x80000000u, 0x7632);   // (Re, -Im)
+                        ri[j][h] = __byte_perm(wi[j], wr[j], 0x7632);                 // (Im, Re)
+                    }
+                }
+                unsigned char *o = X + (size_t)(hk >> 1) * OZ_A + (hk & 1) * 128;
+                const int r0 = 2 * c;
+                const uint32_t off = (r0 >> 3) * 256 + (r0 & 7) * 16;   // row 2c + 1 follows 16 bytes on
+#pragma unroll
+                for (int j = 0; j < OZ_S; ++j) {
+                    *(uint4 *)(o + j * 4096 + off) = make_uint4(rr[j][0], rr[j][1], rr[j][2], rr[j][3]);
+                    *(uint4 *)(o + j * 4096 + off + 16) = make_uint4(ri[j][0], ri[j][1], ri[j][2], ri[j][3]);
+                }
+            }
+            asm volatile("fence.proxy.async;" ::: "memory");   // the bulk copies read what was written here
+            __syncthreads();
+            const unsigned char *tile = img + (size_t)w.geom * sp.img_bytes + sp.sec_img[sec];
+            const double *rs = rscale + (size_t)w.geom * sp.rows + (sec ? sp.D[0] : 0);
+            for (int t = 0; t * OZ_NT < D && !failed; ++t, ++ntile) {
+                const int N = oz_tile_rows(D, t);
+                const uint32_t bb = (uint32_t)(OZ_S * N * 32);
+                if (warp == 0 && lane == 0) {
+                    for (int s = 0; s < nk; ++s) {
+                        const uint32_t q = g + s, sl = q % OZ_ST;
+                        if (q >= OZ_ST && !tc::mbar_wait(&empty[sl], (q / OZ_ST - 1) & 1, OZ_POLLS)) {
+                            failed = true;
+                            break;
+                        }
+                        tc::mbar_expect_tx(&full[sl], OZ_A + bb);
+                        tc::bulk_g2s(smraw + sl * OZ_SLOT, X + (size_t)s * OZ_A, OZ_A, &full[sl]);
+                        tc::bulk_g2s(smraw + sl * OZ_SLOT + OZ_A, tile + (size_t)s * bb, bb, &full[sl]);
+                    }
+                } else if (warp == 1 && lane == 0) {
+                    const uint32_t idesc = tc::idesc_bf16(128, N);
+                    const uint64_t pa = 4096 >> 4, pb = (uint32_t)(N * 32) >> 4;
+                    for (int s = 0; s < nk; ++s) {
+                        const uint32_t q = g + s, sl = q % OZ_ST;
+                        if (!tc::mbar_wait(&full[sl], (q / OZ_ST) & 1, OZ_POLLS)) {
+                            failed = true;
+                            break;
+                        }
+                        tc::fence_after();
+                        const uint64_t da = tc::sdesc(tc::smem_u32(smraw + sl * OZ_SLOT), 128, 256);
+                        const uint64_t db = tc::sdesc(tc::smem_u32(smraw + sl * OZ_SLOT + OZ_A), 128, 256);
+#pragma unroll
+                        for (int j = 0; j < OZ_S; ++j)
+#pragma unroll
+                            for (int i = 0; i + j < OZ_S; ++i)
+                                mma_f16_ss(tbase + (i + j) * OZ_NT, da + i * pa, db + j * pb, idesc,
+                                           (s > 0 || j > 0) ? 1u : 0u);
+                        tc::commit(&empty[sl]);
+                    }
+                    tc::commit(accfull);
+                }
+                __syncwarp();
+                g += nk;
+                if (!tc::mbar_wait(accfull, ntile & 1, OZ_POLLS)) failed = true;
+                tc::fence_after();
+                // ---- accumulators -> FP64: warp -> lane quadrant warp % 4, 16 columns
+                const int q4 = warp & 3, cg = warp >> 2, row = 32 * q4 + lane;
+                if (32 * q4 < 2 * w.npair) {
+                    for (int c0 = 16 * cg; c0 < 16 * cg + 16 && c0 < N; c0 += 8) {
+                        uint32_t v[OZ_S][8];
+#pragma unroll
+                        for (int d = 0; d < OZ_S; ++d)
+                            tc::tmem_ld8(tbase + ((uint32_t)(32 * q4) << 16) + d * OZ_NT + c0, v[d]);
+                        tc::tmem_ld_wait();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            const int r = t * OZ_NT + c0 + i;
+                            if (r >= D) break;
+                            auto a = [&](int d) { return __float2int_rn(__uint_as_float(v[d][i])); };
+                            const long long hi = (((long long)a(0) << 16) + ((long long)a(1) << 8) + a(2)) * 256 + a(3);
+                            const long long lo = (((long long)a(4) << 16) + ((long long)a(5) << 8) + a(6)) * 256 + a(7);
+                            const double c1 = rs[r];                    // 2^(row exponent - 38)
+                            const double y = c1 * ((double)hi + 0x1p-32 * (double)lo);
+                            ((double *)(Y + (size_t)(row >> 1) * sp.rows + (sec ? sp.D[0] : 0) + r))[row & 1] = y;
+                        }
+                    }
+                }
+                tc::fence_before();
+                if (__syncthreads_or(failed)) failed = true;
+                tc::fence_after();
+                tile += (size_t)nk * bb;
+            }
+        }
+        if (failed) break;
+        // ---- outputs: the phases take the source box's power of two
+        for (int e = tid; e < w.npair * (2 * p + 2); e += OZ_T) {
+            const int c = e / (2 * p + 2), d = e - c * (2 * p + 2);
+            double2 *G = (double2 *)(smraw + sp.o_ph + c * sp.ph_bytes) + d;
+            const double f = bscale[transposed ? pr[c].tgt : pr[c].src];
+            *G = double2{f * G->x, f * G->y};
+        }
+        __syncthreads();
+        if (warp < sp.out_warps) {
+            double2 *sg = (double2 *)(smraw + warp * sp.stage_bytes);   // the ring is idle here
+            for (int c = warp; c < w.npair; c += sp.out_warps) {
+                const double2 *y0 = Y + (size_t)c * sp.rows, *y1 = y0 + sp.D[0];
+                asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                __syncwarp();
+                for (int r = lane; r < sp.D[0]; r += 32) {
+                    const double2 ye = y0[r], yo = r < sp.D[1] ? y1[r] : double2{0.0, 0.0};
+                    const uint32_t we = ent[r];
+                    const double2 G = lds_d2(ph0 + c * sp.ph_bytes + 16 * ((we >> 20) & 63));
+                    const double2 s{ye.x + yo.x, ye.y + yo.y};
+                    double2 d{ye.x - yo.x, ye.y - yo.y};
+                    sg[we & 1023] = double2{fma(G.x, s.x, G.y * s.y), fma(G.x, s.y, -G.y * s.x)};
+                    if (!(we >> 26 & 1)) d = double2{-d.x, -d.y};
+                    if (!(we >> 27 & 1))
+                        sg[(we >> 10) & 1023] = double2{fma(G.x, d.x, -G.y * d.y), fma(G.x, d.y, G.y * d.x)};
+                }
+                tc::fence_smem_async();
+                __syncwarp();
+                if (lane == 0)
+                    asm volatile(
+                        "cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f64 [%0], [%1], %2;\n\t"
+                        "cp.async.bulk.commit_group;" ::"l"(out + (transposed ? pr[c].src : pr[c].tgt) * 3 * P),
+                        "r"(tc::smem_u32(sg)), "r"(sp.stage_bytes)
+                        : "memory");
+            }
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+        }
+        tc::fence_smem_async();   // the next bulk copies write where the staging rows were
+        __syncthreads();
+    }
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+    if (failed) {
+        // copies and MMAs still in flight land before the CTA leaves
+        if (tid == 0)
+            for (int s = 0; s < OZ_ST; ++s) tc::mbar_wait(&full[s], 0, 1 << 12), tc::mbar_wait(&full[s], 1, 1 << 12);
+        atomicOr(status, 4);
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tbase, 512);
+}
+
+// one warp per row of a geometry's sector block (transposed: of its transpose, with the C
+// entries of order 0 doubled as outputs and halved as inputs, as the shared input and output
+// maps count them): the row's power of two, then its digits in the K-step images
+__global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan sp, int transposed,
+                                                  const GeomDev *geoms, const CompDev *comps, const cd *tab64,
+                                                  unsigned char *img, double *rscale)
+{
+    __shared__ double ps[OZ_PMAX + 1], pt[OZ_PMAX + 1];
+    __shared__ int cn[OZ_PMAX + 1];
+    const int64_t gi = blockIdx.y;
+    const GeomDev &gm = geoms[gi];
+    if (threadIdx.x <= sp.p) {
+        double a = 1.0, b = 1.0;
+        for (int i = 0; i < (int)threadIdx.x; ++i) {
+            a *= gm.scale_s;
+            b *= gm.scale_t;
+        }
+        ps[threadIdx.x] = a;
+        pt[threadIdx.x] = b;
+        cn[threadIdx.x] = oz_cn(threadIdx.x);
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row >= sp.rows) return;
+    const int sec = row >= sp.D[0], r = row - (sec ? sp.D[0] : 0), D = sp.D[sec];
+    const CompDev cp = comps[gm.comp];
+    const bool fi = (cp.s < 0) != (cp.has_src_refl != 0), fo = (cp.s < 0) != (cp.has_tgt_refl != 0);
+    const cd *tab = tab64 + gi * NTAB * (int64_t)sp.P * sp.P;
+    const SecEntry er = sec_entry(sp.p, r);
+    auto value = [&](int k) {
+        const SecEntry ek = sec_entry(sp.p, k);
+        cd v;
+        if (!transposed) {
+            v = sec_scaled(er, ek, fi, fo, pt, ps, sec_value(sp.p, sec, er, ek, tab));
+        } else {
+            v = sec_scaled(ek, er, fi, fo, pt, ps, sec_value(sp.p, sec, ek, er, tab));
+            if (er.c && er.m == 0) v = 2.0 * v;
+            if (ek.c && ek.m == 0) v = 0.5 * v;
+        }
+        const double f = ldexp(1.0, -cn[ek.n]);
+        return f * v;
+    };
+    double mx = 0.0;
+    for (int k = lane; k < D; k += 32) {
+        const cd v = value(k);
+        mx = fmax(mx, fmax(fabs(v.x), fabs(v.y)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    int e = 0;
+    if (mx > 0.0) {
+        frexp(mx, &e);
+        ++e;                                   // mx < 2^(e - 1)
+    }
+    if (lane == 0) rscale[gi * sp.rows + row] = ldexp(1.0, e - 38);
+    const double f = ldexp(1.0, -e);
+    const int t = r / OZ_NT, rl = r - t * OZ_NT, N = oz_tile_rows(D, t), nk = sp.nk[sec];
+    // the tiles before this one are full
+    unsigned char *o = img + gi * (size_t)sp.img_bytes + sp.sec_img[sec] + (size_t)t * nk * OZ_S * OZ_NT * 32 +
+                       (rl >> 3) * 256 + (rl & 7) * 16;
+    for (int k = lane; k < nk * 8; k += 32) {
+        cd v{0.0, 0.0};
+        if (k < D) v = f * value(k);
+        uint32_t wr[OZ_S], wi[OZ_S];
+        oz_digits(v.x, wr);
+        oz_digits(v.y, wi);
+        unsigned char *q = o + (size_t)(k >> 3) * (OZ_S * N * 32) + ((k & 7) >> 2) * 128 + (k & 3) * 4;
+#pragma unroll
+        for (int j = 0; j < OZ_S; ++j) *(uint32_t *)(q + (size_t)j * N * 32) = __byte_perm(wr[j], wi[j], 0x7632);
+    }
+}
+
+// packed inputs of every box: entry j's two coefficients, scaled by 2^c_n and by the box's
+// power of two so that the sum of two of them is below 1 in size (bscale: the power taken
+// out, NaN where a coefficient is not finite); clears the box's output expansion
+__global__ void __launch_bounds__(128) k_oz_pack(int p, int n8, int D0, const cd *in, OzIn *pk, double *bscale,
+                                                 cd *out)
+{
+    __shared__ int emax[4], cn[OZ_PMAX + 1];
+    const int P = (p + 1) * (p + 1), P3 = 3 * P;
+    const int64_t box = blockIdx.x;
+    const cd *m = in + box * P3;
+    if (threadIdx.x <= p) cn[threadIdx.x] = oz_cn(threadIdx.x);
+    __syncthreads();
+    int e = -4096;                              // exponent field of the largest scaled part
+    for (int j = threadIdx.x; j < P3; j += blockDim.x) {
+        const cd v = m[j];
+        const int ex = max((int)(__double_as_longlong(v.x) >> 52) & 0x7ff, (int)(__double_as_longlong(v.y) >> 52) & 0x7ff);
+        if (ex == 0x7ff) e = 8192;
+        else if (ex > 0) e = max(e, ex - 1022 + cn[sec_entry(p, j % P).n]);   // |v| 2^c_n < 2^e
+        out[box * P3 + j] = cd{0.0, 0.0};
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+    if ((threadIdx.x & 31) == 0) emax[threadIdx.x >> 5] = e;
+    __syncthreads();
+    e = max(max(emax[0], emax[1]), max(emax[2], emax[3]));
+    const bool bad = e >= 8192, zero = e == -4096;
+    const int sh = (bad || zero) ? 0 : e + 2;   // two coefficients of parts below 2^e: below 2^(e + 1.5) each part
+    if (threadIdx.x == 0) bscale[box] = bad ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, sh);
+    for (int j = threadIdx.x; j < n8; j += blockDim.x) {
+        OzIn v{0.0, 0.0, 0.0, 0.0};
+        if (j < D0 && !bad) {
+            const uint32_t w = sec_word(p, j);
+            const cd a = m[w & 1023], b = m[(w >> 10) & 1023];
+            const int k = cn[sec_entry(p, j).n] - sh;
+            v = OzIn{ldexp(a.x, k), ldexp(a.y, k), ldexp(b.x, k), ldexp(b.y, k)};
+        }
+        pk[box * n8 + j] = v;
+    }
+}
+
+}  // namespace
+
+bool m2l_oz_supported(int p) { return p >= 1 && p <= OZ_PMAX; }
+int m2l_oz_pairs() { return OZ_BN; }
+size_t m2l_oz_image_bytes(int p, int64_t ngeom)
+{
+    const OzPlan sp = oz_plan(p);
+    return (size_t)ngeom * (sp.img_bytes + (size_t)sp.rows * sizeof(double));
+}
+size_t m2l_oz_packed_bytes(int p, int64_t nbox) { return (size_t)nbox * (oz_plan(p).nk[0] * 8 * sizeof(OzIn) + sizeof(double)); }
+size_t m2l_oz_scratch_bytes(int p, int nsm)
+{
+    const OzPlan sp = oz_plan(p);
+    return (size_t)nsm * ((size_t)sp.nk[0] * OZ_A + (size_t)OZ_BN * sp.rows * sizeof(double2));
+}
+
+void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
+                     void *img, cudaStream_t st)
+{
+    const OzPlan sp = oz_plan(p);
+    double *rs = (double *)((unsigned char *)img + (size_t)ng * sp.img_bytes);
+    cudaMemsetAsync(img, 0, (size_t)ng * sp.img_bytes, st);   // rows beyond the block stay zero
+    for (int64_t g0 = 0; g0 < ng; g0 += 32768) {              // grid.y is limited to 65535
+        const int64_t nb = std::min<int64_t>(32768, ng - g0);
+        k_oz_image<<<dim3((sp.rows + 7) / 8, (unsigned)nb), 256, 0, st>>>(
+            sp, transposed, geoms + g0, comps, tab64 + g0 * NTAB * (int64_t)sp.P * sp.P,
+            (unsigned char *)img + (size_t)g0 * sp.img_bytes, rs + g0 * sp.rows);
+    }
+}
+
+cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int nsm,
+                          int *status, cudaStream_t st)
+{
+    if (!m2l_oz_supported(p) || nsm < 1) return cudaErrorInvalidValue;
+    const OzPlan sp = oz_plan(p);
+    const int n8 = sp.nk[0] * 8;
+    double *bs = (double *)((unsigned char *)packed + (size_t)nbox * n8 * sizeof(OzIn));
+    if (nbox > 0) k_oz_pack<<<(unsigned)nbox, 128, 0, st>>>(p, n8, sp.D[0], in, (OzIn *)packed, bs, out);
+    if (nwork <= 0) return cudaGetLastError();
+    unsigned char *x = (unsigned char *)scratch;
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(nwork, nsm), OZ_T, std::max<size_t>(sp.smem, 116 * 1024), st>>>(
+        sp, transposed ? 1 : 0, nwork, work, pairs, (const unsigned char *)img,
+        (const double *)((const unsigned char *)img + (size_t)ngeom * sp.img_bytes), (const OzIn *)packed, bs, out, x,
+        (double *)(x + (size_t)nsm * sp.nk[0] * OZ_A), status);
+    return cudaGetLastError();
+}
+
+cudaError_t configure_m2l_oz()
+{
+    return cudaFuncSetAttribute(k_m2l_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
+}  // namespace lmf

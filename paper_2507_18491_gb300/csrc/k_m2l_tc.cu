@@ -916,7 +916,8 @@ cudaError_t configure_m2l_tc()
     cudaError_t e = cudaFuncSetAttribute(k_m2l_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_trans_tc2, cudaFuncAttributeMaxDynamicSharedMemorySize, V2_SMEM_MAX);
-    return e != cudaSuccess ? e : configure_m2l_sec();
+    if (e != cudaSuccess || (e = configure_m2l_sec()) != cudaSuccess) return e;
+    return configure_m2l_oz();
 }
 
 }  // namespace lmf

@@ -169,6 +169,21 @@ void launch_sec_pack(int p, int64_t nbox, const cf *me, void *packed, cf *le, cu
 // probs: the problems of a batched launch (device array), or null with one problem in `one`
 cudaError_t launch_m2l_sec(int p, int64_t nwork, const M2LWork *work, const TcProb &one, const TcProb *probs,
                            float *yscr, int nsm, int *status, cudaStream_t st);
+// k_m2l_oz.cu: M2L of the FP64 form on the tensor cores, operands as eight base-256 digits.
+// out is cleared, then out[tgt] += M in[src] over the items' pairs (transposed: in over the
+// targets, out over the sources); img from launch_oz_image (m2l_oz_image_bytes), packed and
+// scratch of the sizes below
+bool m2l_oz_supported(int p);
+int m2l_oz_pairs();
+size_t m2l_oz_image_bytes(int p, int64_t ngeom);
+size_t m2l_oz_packed_bytes(int p, int64_t nbox);
+size_t m2l_oz_scratch_bytes(int p, int nsm);
+cudaError_t configure_m2l_oz();
+void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
+                     void *img, cudaStream_t st);
+cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int nsm,
+                          int *status, cudaStream_t st);
 // M2M or L2L on a persistent tensor-core kernel (k_m2l_tc.cu, p <= 12): items M2LWork{geom = translation group, t = 0,
 // npair, pair0} over pairs (tsrc[q], tdst[q]), 3 helical columns each; img holds
 // one tiled matrix per group (tile_matrix_tc2, tc2_matrix_bytes(p) each)
