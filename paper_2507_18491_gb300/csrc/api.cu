@@ -926,6 +926,16 @@ static void leaf_l2p(lmfmm_ctx *ctx, const cx<T> *in, cd *out, bool p2m_basis, c
     launch_l2p<T>(p, d->nleaves, d->leaves, d->boxes, d->xyz, in, ctx->med, d->lscale, out, st, p2m_basis, false);
 }
 
+// Y += A X over the pairs of translation items (one level of M2M or L2L); the FP64 form reads
+// the transposes AT
+template <typename T>
+static void translate(int p, int64_t nwork, const GemmWork *work, const cx<T> *A, const cx<T> *AT, const int64_t *src,
+                      const int64_t *dst, cx<T> *x, cudaStream_t st)
+{
+    if constexpr (std::is_same<T, double>::value) launch_trans_fp64(p, nwork, work, AT, src, dst, x, x, st);
+    else launch_group_gemm_t<T>(p, nwork, work, A, src, dst, x, x, true, st);
+}
+
 // stages of one matvec, for the batched launch: the upward pass (gather, P2M,
 // M2M), the M2L (own_m2l = false: only the clearing of the local expansions,
 // the M2L itself runs in the batch's merged launch), the downward pass
@@ -940,6 +950,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
     const int64_t N = ctx->N, nbox = (int64_t)ctx->boxes.size();
     cx<T> *me = (cx<T> *)d->me, *le = (cx<T> *)d->le;
     const cx<T> *tup = (const cx<T> *)d->tup, *tdn = (const cx<T> *)d->tdn;
+    const cx<T> *tupT = (const cx<T> *)d->tupT, *tdnT = (const cx<T> *)d->tdnT;
     int nl = 0;   // kernels launched (launchers skip empty work)
     if (parts & MV_UP) {
     CK(cudaEventRecord(d->ev[0], st));
@@ -961,8 +972,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
             }
         }
         int64_t w0 = d->gwork_off[lev], w1 = d->gwork_off[lev + 1];
-        launch_group_gemm_t<T>(p, w1 - w0, d->gwork + w0, tup, d->tchild, d->tparent, me, me, true,
-                               st);
+        translate<T>(p, w1 - w0, d->gwork + w0, tup, tupT, d->tchild, d->tparent, me, st);
         nl += w1 > w0;
     }
     CK(cudaEventRecord(d->ev[2], st));
@@ -1013,9 +1023,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
             }
         }
         int64_t w0 = d->gwork_off[lev], w1 = d->gwork_off[lev + 1];
-        // a child has one parent: reductions (fire and forget) rather than read-modify-write
-        launch_group_gemm_t<T>(p, w1 - w0, d->gwork + w0, tdn, d->tparent, d->tchild, le, le, true,
-                               st);
+        translate<T>(p, w1 - w0, d->gwork + w0, tdn, tdnT, d->tparent, d->tchild, le, st);
         nl += w1 > w0;
     }
     CK(cudaEventRecord(d->ev[4], st));
@@ -1061,7 +1069,7 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     CK(cudaEventRecord(d->ev[1], st));
     for (int lev = ctx->depth; lev >= 1; --lev) {   // L2L^T: children into parents
         int64_t w0 = d->gwork_off[lev], w1 = d->gwork_off[lev + 1];
-        launch_group_gemm_t<T>(p, w1 - w0, d->gwork + w0, tdnT, d->tchild, d->tparent, le, le, true, st);
+        translate<T>(p, w1 - w0, d->gwork + w0, tdnT, (const cx<T> *)d->tdn, d->tchild, d->tparent, le, st);
         nl += w1 > w0;
     }
     CK(cudaEventRecord(d->ev[2], st));
@@ -1082,7 +1090,7 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     CK(cudaEventRecord(d->ev[3], st));
     for (int lev = 1; lev <= ctx->depth; ++lev) {   // M2M^T: parents into children
         int64_t w0 = d->gwork_off[lev], w1 = d->gwork_off[lev + 1];
-        launch_group_gemm_t<T>(p, w1 - w0, d->gwork + w0, tupT, d->tparent, d->tchild, me, me, true, st);
+        translate<T>(p, w1 - w0, d->gwork + w0, tupT, (const cx<T> *)d->tup, d->tparent, d->tchild, me, st);
         nl += w1 > w0;
     }
     CK(cudaEventRecord(d->ev[4], st));

@@ -179,6 +179,53 @@ __global__ void __launch_bounds__(256) k_group_gemm(int p, const GemmWork *work,
     });
 }
 
+// M2M / L2L in double: bound by the FP64 pipe (2 multiply-adds per clock and SM), which any
+// tile shape feeds, so a CTA takes 32 rows x 2 box pairs, one output per thread: the upper
+// levels' few pairs then spread over the chip (a CTA of 64 rows x 10 pairs took 105 us per
+// level at p = 6, on a handful of SMs).  matsT: transposed matrices ([k][r]), read coalesced.
+constexpr int TF_PAIRS = 2;
+__global__ void __launch_bounds__(32 * 3 * TF_PAIRS) k_trans_fp64(int p, const GemmWork *work, const cd *matsT,
+                                                                  const int64_t *src, const int64_t *dst, const cd *in,
+                                                                  cd *out)
+{
+    extern __shared__ unsigned char smraw[];
+    const int P = (p + 1) * (p + 1);
+    double2 *X = (double2 *)smraw;               // [column][k]
+    const GemmWork w = work[blockIdx.x];
+    const int lane = threadIdx.x & 31, c = threadIdx.x >> 5;
+    const int pp = blockIdx.z * TF_PAIRS + c / 3, v = c % 3;
+    if (blockIdx.z * TF_PAIRS >= w.npair) return;
+    const bool live = pp < w.npair;
+    double2 *x = X + (size_t)c * P;              // each warp reads its own column
+    if (live) {
+        const double2 *q = (const double2 *)(in + (src[w.pair0 + pp] * 3 + v) * P);
+        for (int k = lane; k < P; k += 32) x[k] = q[k];
+    }
+    __syncwarp();
+    const int r = blockIdx.y * 32 + lane;
+    if (!live || r >= P) return;
+    const double2 *A = (const double2 *)(matsT + (int64_t)w.group * P * P) + r;
+    cd acc0{0.0, 0.0}, acc1{0.0, 0.0};
+    int k = 0;
+    for (; k + 4 <= P; k += 4) {
+        double2 a[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) a[u] = A[(int64_t)(k + u) * P];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const double2 xv = x[k + u];
+            cmac(u & 1 ? acc1 : acc0, cd{a[u].x, a[u].y}, cd{xv.x, xv.y});
+        }
+    }
+    for (; k < P; ++k) {
+        const double2 a = A[(int64_t)k * P], xv = x[k];
+        cmac(acc0, cd{a.x, a.y}, cd{xv.x, xv.y});
+    }
+    double *o = (double *)(out + (dst[w.pair0 + pp] * 3 + v) * P + r);
+    atomicAdd(o, acc0.x + acc1.x);
+    atomicAdd(o + 1, acc0.y + acc1.y);
+}
+
 // --------------------------------------------------------------------- M2L
 
 // The M2L of eq. M2L_scale_with_Tnmu with T = (-i)^nu i^(n'+1+d) s^(nu+mu+n'+m')
@@ -403,6 +450,15 @@ void launch_group_gemm_t(int p, int64_t nwork, const GemmWork *work, const cx<T>
                                                                     out, atomic);
 }
 
+void launch_trans_fp64(int p, int64_t nwork, const GemmWork *work, const cd *matsT, const int64_t *src,
+                       const int64_t *dst, const cd *in, cd *out, cudaStream_t st)
+{
+    if (nwork <= 0) return;
+    const int P = (p + 1) * (p + 1), most = gemm_cols<double>() / 3;   // pairs of a full item
+    k_trans_fp64<<<dim3((unsigned)nwork, (P + 31) / 32, (most + TF_PAIRS - 1) / TF_PAIRS), 32 * 3 * TF_PAIRS,
+                   (size_t)3 * TF_PAIRS * P * sizeof(double2), st>>>(p, work, matsT, src, dst, in, out);
+}
+
 template <typename T>
 void launch_m2l_t(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
                   const CompDev *comps, const M2LPair *pairs, const cx<T> *tab, const cx<T> *me,
@@ -438,9 +494,6 @@ void launch_scale_tables(int p, int64_t g0, int64_t ng, const GeomDev *geoms, co
 template void launch_group_gemm_t<float>(int, int64_t, const GemmWork *, const cf *,
                                          const int64_t *, const int64_t *, const cf *, cf *, bool,
                                          cudaStream_t);
-template void launch_group_gemm_t<double>(int, int64_t, const GemmWork *, const cd *,
-                                          const int64_t *, const int64_t *, const cd *, cd *,
-                                          bool, cudaStream_t);
 template void launch_m2l_t<float>(int, int64_t, const M2LWork *, const GeomDev *, const CompDev *,
                                   const M2LPair *, const cf *, const cf *, cf *, cudaStream_t);
 template void launch_m2l_t<double>(int, int64_t, const M2LWork *, const GeomDev *,
@@ -460,7 +513,6 @@ cudaError_t configure_trans_kernels()
     const int big = 220 * 1024;
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_group_gemm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
-    if ((e = cudaFuncSetAttribute(k_group_gemm<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
     if ((e = cudaFuncSetAttribute(k_m2l<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
     if ((e = cudaFuncSetAttribute(k_m2l<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
     if ((e = cudaFuncSetAttribute(k_m2l_tr<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, big))) return e;
@@ -468,7 +520,6 @@ cudaError_t configure_trans_kernels()
     // these CTAs hold ~100 KB of shared memory: take the whole carveout so that two fit on an SM
     const int mx = (int)cudaSharedmemCarveoutMaxShared;
     if ((e = cudaFuncSetAttribute(k_group_gemm<float>, cudaFuncAttributePreferredSharedMemoryCarveout, mx))) return e;
-    if ((e = cudaFuncSetAttribute(k_group_gemm<double>, cudaFuncAttributePreferredSharedMemoryCarveout, mx))) return e;
     if ((e = cudaFuncSetAttribute(k_m2l<float>, cudaFuncAttributePreferredSharedMemoryCarveout, mx))) return e;
     if ((e = cudaFuncSetAttribute(k_m2l<double>, cudaFuncAttributePreferredSharedMemoryCarveout, mx))) return e;
     return configure_m2l_tc();

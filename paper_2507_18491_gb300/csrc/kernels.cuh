@@ -127,6 +127,9 @@ template <typename T>
 void launch_group_gemm_t(int p, int64_t nwork, const GemmWork *work, const cx<T> *mats,
                          const int64_t *src, const int64_t *dst, const cx<T> *in, cx<T> *out,
                          bool atomic, cudaStream_t st);
+// M2M / L2L of the FP64 form: matsT holds the transposed matrices
+void launch_trans_fp64(int p, int64_t nwork, const GemmWork *work, const cd *matsT, const int64_t *src,
+                       const int64_t *dst, const cd *in, cd *out, cudaStream_t st);
 template <typename T>
 void launch_m2l_t(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
                   const CompDev *comps, const M2LPair *pairs, const cx<T> *tab, const cx<T> *me,

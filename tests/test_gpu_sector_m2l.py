@@ -47,8 +47,9 @@ def test_mixed_form(p):
 # 10: 187 = 2 x 64 + 64), the largest order (16: 442 = 6 x 64 + 64)
 @pytest.mark.parametrize("p", [1, 4, 7, 10, 16])
 def test_fp64_form(p):
-    ref = _simt(p)
     w, op = _op(p)
+    # FP32 expansions overflow beyond p = 13 (NaN in the SIMT mixed form): the sum over all pairs there
+    ref = _simt(p) if p <= 13 else op.direct(torch.from_numpy(w.J).cuda()).cpu().numpy()
     rng = np.random.default_rng(p)
     mv = lambda x: op.matvec(torch.from_numpy(x).cuda()).cpu().numpy()  # noqa: E731
     a = mv(w.J)
