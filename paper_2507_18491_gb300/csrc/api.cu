@@ -677,90 +677,61 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     }
     TRY(dupload(ctx, &d->m2lwork, mw));
     d->n_m2lwork = (int64_t)mw.size();
-    // translation matrices (exact addition theorem, host)
+    // translation matrices (exact addition theorem), on the device from the groups' factors
     {
-        std::vector<int64_t> goff;
-        std::vector<int> gl;
-        std::vector<double> gv;
-        gaunt_table(p, goff, gl, gv);
-        size_t ngr = ctx->tgroups.size();
-        std::vector<cd> hup(ngr * (size_t)P * P), hdn(ngr * (size_t)P * P);
-        std::vector<int> deg(P);
-        for (int n = 0; n <= p; ++n)
-            for (int m = -n; m <= n; ++m) deg[n * n + n + m] = n;
-        for (size_t i = 0; i < ngr; ++i) {
+        const int64_t ngr = (int64_t)ctx->tgroups.size();
+        const int nfac = trans_factor_count(p);
+        std::vector<double> fac((size_t)ngr * nfac), gw, gP;
+        std::vector<double2> scl(ngr);
+        for (int64_t i = 0; i < ngr; ++i) {
             const TransGroup &g = ctx->tgroups[i];
-            cd *U = &hup[i * P * P], *V = &hdn[i * P * P];
-            translation_matrix(p, zc(ctx->med.k[g.layer].x, ctx->med.k[g.layer].y), g.t, goff, gl,
-                               gv, U, V);
+            trans_factors(p, zc(ctx->med.k[g.layer].x, ctx->med.k[g.layer].y), g.t, &fac[i * nfac]);
             // scaled expansions: M~ = M / s^n, L~ = L s^nu, s = |k| S_level
-            double sc = kabs(g.layer) * lev_size(g.level), sp = kabs(g.layer) * lev_size(g.level - 1);
-            for (int r = 0; r < P; ++r)
-                for (int c = 0; c < P; ++c) {
-                    double fu = std::pow(sc, deg[c]) / std::pow(sp, deg[r]);
-                    double fd = std::pow(sc, deg[r]) / std::pow(sp, deg[c]);
-                    U[r * P + c] = fu * U[r * P + c];
-                    V[r * P + c] = fd * V[r * P + c];
-                }
+            scl[i] = double2{kabs(g.layer) * lev_size(g.level), kabs(g.layer) * lev_size(g.level - 1)};
         }
+        gaunt_nodes(p, gw, gP);
+        double *dw = nullptr, *dP = nullptr, *dGt = nullptr, *dfac = nullptr;
+        double2 *dsc = nullptr;
+        cd *up64 = nullptr, *dn64 = nullptr;
+        TRY(dupload(ctx, &dw, gw));
+        TRY(dupload(ctx, &dP, gP));
+        TRY(dupload(ctx, &dfac, fac));
+        TRY(dupload(ctx, &dsc, scl));
+        TRY(dalloc(ctx, &dGt, (size_t)P * P * (p + 1)));
+        TRY(dalloc(ctx, &up64, (size_t)ngr * P * P));
+        TRY(dalloc(ctx, &dn64, (size_t)ngr * P * P));
+        launch_trans_build(p, (int)gw.size(), dw, dP, dGt, ngr, dfac, dsc, up64, dn64, st);
+        CK(cudaGetLastError());
+        d->trans_tc = d->m2l_kernel == 3 && ctx->prm.tensor_cores == 3 && trans_tc2_supported(p);
         // the SIMT forms also keep the transposes (the transposed operator runs on them)
         const bool want_tr = d->m2l_kernel <= 1;
-        std::vector<cd> hupT, hdnT;
-        if (want_tr) {
-            hupT.resize(hup.size());
-            hdnT.resize(hdn.size());
-            for (size_t i = 0; i < ngr; ++i)
-                for (int r = 0; r < P; ++r)
-                    for (int c = 0; c < P; ++c) {
-                        hupT[i * P * P + (size_t)c * P + r] = hup[i * P * P + (size_t)r * P + c];
-                        hdnT[i * P * P + (size_t)c * P + r] = hdn[i * P * P + (size_t)r * P + c];
-                    }
-        }
-        if (f32) {
-            auto to32 = [](const std::vector<cd> &a) {
-                std::vector<cf> o(a.size());
-                for (size_t i = 0; i < a.size(); ++i) o[i] = cf{(float)a[i].x, (float)a[i].y};
-                return o;
-            };
-            cf *a1 = nullptr, *a2 = nullptr;
-            TRY(dupload(ctx, &a1, to32(hup)));
-            TRY(dupload(ctx, &a2, to32(hdn)));
-            d->tup = a1;
-            d->tdn = a2;
-            if (want_tr) {
-                TRY(dupload(ctx, &a1, to32(hupT)));
-                TRY(dupload(ctx, &a2, to32(hdnT)));
-                d->tupT = a1;
-                d->tdnT = a2;
+        if (!f32) {
+            d->tup = up64;
+            d->tdn = dn64;
+            cd *a1 = nullptr;
+            for (int q = 0; q < 2; ++q) {
+                TRY(dalloc(ctx, &a1, (size_t)ngr * P * P));
+                launch_trans_copy<double>(p, ngr, true, q ? dn64 : up64, a1, st);
+                (q ? d->tdnT : d->tupT) = a1;
             }
-        } else {
-            cd *a1 = nullptr, *a2 = nullptr;
-            TRY(dupload(ctx, &a1, hup));
-            TRY(dupload(ctx, &a2, hdn));
-            d->tup = a1;
-            d->tdn = a2;
-            if (want_tr) {
-                TRY(dupload(ctx, &a1, hupT));
-                TRY(dupload(ctx, &a2, hdnT));
-                d->tupT = a1;
-                d->tdnT = a2;
+        } else if (!d->trans_tc) {
+            cf *a1 = nullptr;
+            for (int q = 0; q < (want_tr ? 4 : 2); ++q) {
+                TRY(dalloc(ctx, &a1, (size_t)ngr * P * P));
+                launch_trans_copy<float>(p, ngr, q >= 2, (q & 1) ? dn64 : up64, a1, st);
+                (q == 0 ? d->tup : q == 1 ? d->tdn : q == 2 ? d->tupT : d->tdnT) = a1;
             }
         }
         TRY(dupload(ctx, &d->tchild, ctx->tpair_child));
         TRY(dupload(ctx, &d->tparent, ctx->tpair_parent));
-        d->trans_tc = d->m2l_kernel == 3 && ctx->prm.tensor_cores == 3 && trans_tc2_supported(p);
         if (d->trans_tc) {
             // M2M / L2L on the persistent tensor-core kernel: tiled bf16 three-piece
             // images of the scaled FP64 matrices, items of 21 pairs (63 helical columns)
-            const size_t mw = tc2_matrix_bytes(p) / 4;
-            std::vector<uint32_t> iu(ngr * mw), id(ngr * mw);
-            for (size_t i = 0; i < ngr; ++i) {
-                tile_matrix_tc2(p, &hup[i * P * P], &iu[i * mw]);
-                tile_matrix_tc2(p, &hdn[i * P * P], &id[i * mw]);
-            }
-            uint32_t *a1 = nullptr, *a2 = nullptr;
-            TRY(dupload(ctx, &a1, iu));
-            TRY(dupload(ctx, &a2, id));
+            unsigned char *a1 = nullptr, *a2 = nullptr;
+            TRY(dalloc(ctx, &a1, (size_t)ngr * tc2_matrix_bytes(p)));
+            TRY(dalloc(ctx, &a2, (size_t)ngr * tc2_matrix_bytes(p)));
+            launch_tile_matrices(p, ngr, up64, a1, st);
+            launch_tile_matrices(p, ngr, dn64, a2, st);
             d->tupi = a1;
             d->tdni = a2;
             std::vector<M2LWork> tw;
@@ -768,7 +739,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             const int per = m2l_tc_cols() / 3;
             for (int lev = 1; lev <= ctx->depth; ++lev) {
                 d->twork_off[lev] = (int64_t)tw.size();
-                for (size_t gi = 0; gi < ngr; ++gi) {
+                for (int64_t gi = 0; gi < ngr; ++gi) {
                     const TransGroup &g = ctx->tgroups[gi];
                     if (g.level != lev) continue;
                     for (int64_t q = g.pair0; q < g.pair1; q += per) {
@@ -784,20 +755,26 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             TRY(dupload(ctx, &d->twork, tw));
         }
         // work items per child level
-        std::vector<GemmWork> gw;
+        std::vector<GemmWork> gwk;
         d->gwork_off.assign(ctx->depth + 2, 0);
         for (int lev = 1; lev <= ctx->depth; ++lev) {
-            d->gwork_off[lev] = (int64_t)gw.size();
+            d->gwork_off[lev] = (int64_t)gwk.size();
             for (size_t gi = 0; gi < ctx->tgroups.size(); ++gi) {
                 const TransGroup &g = ctx->tgroups[gi];
                 if (g.level != lev) continue;
                 int per = (f32 ? gemm_cols<float>() : gemm_cols<double>()) / 3;
                 for (int64_t q = g.pair0; q < g.pair1; q += per)
-                    gw.push_back(GemmWork{(int)gi, (int)std::min<int64_t>(per, g.pair1 - q), q});
+                    gwk.push_back(GemmWork{(int)gi, (int)std::min<int64_t>(per, g.pair1 - q), q});
             }
         }
-        d->gwork_off[ctx->depth + 1] = (int64_t)gw.size();
-        TRY(dupload(ctx, &d->gwork, gw));
+        d->gwork_off[ctx->depth + 1] = (int64_t)gwk.size();
+        TRY(dupload(ctx, &d->gwork, gwk));
+        CK(cudaStreamSynchronize(st));
+        for (void *q : {(void *)dw, (void *)dP, (void *)dGt, (void *)dfac, (void *)dsc}) dfree(ctx, q);
+        if (f32) {
+            dfree(ctx, up64);
+            dfree(ctx, dn64);
+        }
     }
     // near field
     TRY(dupload(ctx, &d->near, ctx->near));

@@ -666,6 +666,58 @@ static void sph_bessel_ld(lz z, int L, std::vector<lz> &j)
     for (auto &v : j) v *= sc;
 }
 
+// Gauss-Legendre nodes of the Gaunt integrals of orders up to (2p, p, p): weights (times
+// 2 pi) and P~_l^m (l <= 2p, m >= 0) at every node
+void gaunt_nodes(int p, std::vector<double> &w, std::vector<double> &Pq)
+{
+    const int nq = 2 * p + 4, nt = (2 * p + 1) * (2 * p + 2) / 2;
+    w.resize(nq);
+    Pq.resize((size_t)nq * nt);
+    const ld pi = 3.14159265358979323846264338327950288L;
+    std::vector<ld> P;
+    for (int i = 0; i < nq; ++i) {
+        ld x = std::cos(pi * (i + 0.75L) / (nq + 0.5L)), dp = 0;
+        for (int it = 0; it < 100; ++it) {
+            ld p0 = 1, p1 = x;
+            for (int n = 2; n <= nq; ++n) {
+                const ld p2 = ((2 * n - 1) * x * p1 - (n - 1) * p0) / n;
+                p0 = p1;
+                p1 = p2;
+            }
+            dp = nq * (x * p1 - p0) / (x * x - 1);
+            const ld dx = p1 / dp;
+            x -= dx;
+            if (std::fabs((double)dx) < 1e-22) break;
+        }
+        w[i] = (double)(4 * pi / ((1 - x * x) * dp * dp));
+        legendre_ld(2 * p, x, std::sqrt(1 - x * x), P);
+        for (int e = 0; e < nt; ++e) Pq[(size_t)i * nt + e] = (double)P[e];
+    }
+}
+
+// factors of W(t) that do not depend on the entry, as doubles: i^l j_l(k |t|) (complex,
+// l <= 2p), P~_l^m(t^) (m >= 0), 4 pi e^{-i mu phi} (complex, mu = -2p..2p)
+void trans_factors(int p, zc kk, const double t[3], double *out)
+{
+    const int lmax = 2 * p;
+    const ld tn = std::sqrt((ld)t[0] * t[0] + (ld)t[1] * t[1] + (ld)t[2] * t[2]);
+    std::vector<lz> jl;
+    sph_bessel_ld(lz(kk.real(), kk.imag()) * tn, lmax, jl);
+    for (int l = 0; l <= lmax; ++l) {
+        const lz v = ((l & 1) ? lz(0, 1) : lz(1)) * jl[l] * (ld)((l & 2) ? -1 : 1);
+        *out++ = (double)v.real();
+        *out++ = (double)v.imag();
+    }
+    std::vector<ld> Pt;
+    legendre_ld(lmax, tn > 0 ? t[2] / tn : 1, tn > 0 ? std::sqrt((ld)t[0] * t[0] + (ld)t[1] * t[1]) / tn : 0, Pt);
+    for (int e = 0; e < (lmax + 1) * (lmax + 2) / 2; ++e) *out++ = (double)Pt[e];
+    const ld phi = std::atan2((ld)t[1], (ld)t[0]), fourpi = 4 * 3.14159265358979323846264338327950288L;
+    for (int mu = -lmax; mu <= lmax; ++mu) {
+        *out++ = (double)(fourpi * std::cos(mu * phi));
+        *out++ = (double)(-fourpi * std::sin(mu * phi));
+    }
+}
+
 void translation_matrix(int p, zc kk, const double t[3], const std::vector<int64_t> &off,
                         const std::vector<int> &lval, const std::vector<double> &gval, cd *up,
                         cd *dn)

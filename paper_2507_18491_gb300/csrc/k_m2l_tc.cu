@@ -888,27 +888,33 @@ size_t tc2_matrix_bytes(int p)
     return (size_t)sp.nchunk * sp.CB;
 }
 
-void tile_matrix_tc2(int p, const cd *M, void *img_)
+// one thread per (row, input) of a group's image: zero beyond P
+__global__ void k_tile_matrices(int p, const cd *M, __nv_bfloat16 *img)
 {
     const int P = (p + 1) * (p + 1);
     const V2Plan sp = v2_plan(p);
     const int NR = (int)sp.NR, nsub = (int)sp.nchunk * V2_KS;
-    __nv_bfloat16 *img = (__nv_bfloat16 *)img_;
-    for (int c = 0; c < nsub; ++c)
-        for (int r = 0; r < NR; ++r)
-            for (int i = 0; i < 8; ++i) {
-                const int k = 8 * c + i;
-                cd v{0.0, 0.0};
-                if (r < P && k < P) v = M[(size_t)r * P + k];
-                __nv_bfloat16 re[V2_NPC], im[V2_NPC];
-                v2_split3(v.x, re);
-                v2_split3(v.y, im);
-                __nv_bfloat16 *sub = img + (size_t)c * NR * 16 * V2_NPC;
-                for (int pc = 0; pc < V2_NPC; ++pc) {
-                    sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i)] = re[pc];
-                    sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i + 1)] = im[pc];
-                }
-            }
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nsub * NR * 8) return;
+    const int c = e / (NR * 8), rem = e % (NR * 8), r = rem >> 3, i = rem & 7, k = 8 * c + i;
+    cd v{0.0, 0.0};
+    if (r < P && k < P) v = M[(size_t)blockIdx.y * P * P + (size_t)r * P + k];
+    __nv_bfloat16 re[V2_NPC], im[V2_NPC];
+    v2_split3(v.x, re);
+    v2_split3(v.y, im);
+    __nv_bfloat16 *sub = img + ((size_t)blockIdx.y * nsub + c) * (size_t)(NR * 16 * V2_NPC);
+    for (int pc = 0; pc < V2_NPC; ++pc) {
+        sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i)] = re[pc];
+        sub[(size_t)pc * NR * 16 + v2_img_off(r, 2 * i + 1)] = im[pc];
+    }
+}
+
+void launch_tile_matrices(int p, int64_t ng, const cd *M, void *img, cudaStream_t st)
+{
+    const V2Plan sp = v2_plan(p);
+    if (ng > 0)
+        k_tile_matrices<<<dim3((unsigned)((sp.nchunk * V2_KS * sp.NR * 8 + 255) / 256), (unsigned)ng), 256, 0, st>>>(
+            p, M, (__nv_bfloat16 *)img);
 }
 
 cudaError_t configure_m2l_tc()

@@ -210,4 +210,107 @@ cudaError_t configure_tab_kernels()
     return cudaFuncSetAttribute(k_tab_contract, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 160 * 1024);
 }
+// ---------------------------------------------------- translation matrices
+// Gaunt coefficients G(l; n', n) = int Y_l^(m-m') Y_n'^m' conj(Y_n^m) for l = |n - n'|,
+// |n - n'| + 2, ... (zero where l < |m - m'|), p + 1 per entry, by the Gauss-Legendre rule
+// that is exact for them.  One thread per entry: the quadrature is some 10^7 FP64 operations
+// at p = 12, which took the host (whose long double is software there) a second.
+__global__ void k_gaunt(int p, int nq, const double *w, const double *Pq, double *G)
+{
+    const int P = (p + 1) * (p + 1), nt = (2 * p + 1) * (2 * p + 2) / 2;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= P * P) return;
+    const int r = e / P, c = e % P;
+    int n = (int)sqrtf((float)r + 0.5f), n1 = (int)sqrtf((float)c + 0.5f);
+    while ((n + 1) * (n + 1) <= r) ++n;
+    while (n * n > r) --n;
+    while ((n1 + 1) * (n1 + 1) <= c) ++n1;
+    while (n1 * n1 > c) --n1;
+    const int m = r - n * n - n, m1 = c - n1 * n1 - n1, mu = m - m1;
+    const int am = abs(m), am1 = abs(m1), amu = abs(mu);
+    // P~_n^m = (-1)^m P~_n^|m| for m < 0
+    const int neg = ((m < 0 ? am : 0) + (m1 < 0 ? am1 : 0) + (mu < 0 ? amu : 0)) & 1;
+    for (int j = 0; j <= p; ++j) {
+        const int l = abs(n - n1) + 2 * j;
+        double s = 0.0;
+        if (l <= n + n1 && l >= amu) {
+            for (int q = 0; q < nq; ++q) {
+                const double *Q = Pq + (int64_t)q * nt;
+                s += w[q] * Q[l * (l + 1) / 2 + amu] * Q[n1 * (n1 + 1) / 2 + am1] * Q[n * (n + 1) / 2 + am];
+            }
+        }
+        G[(int64_t)e * (p + 1) + j] = neg ? -s : s;
+    }
+}
+
+// M2M = i^(n'-n) W(t) and L2L = i^(n-n') W(t) of every translation group, with the level
+// scaling M~ = M / s^n, L~ = L s^nu: W = sum_l i^l j_l(k |t|) P~_l^mu(t^) 4 pi e^{-i mu phi} G(l).
+// fac: trans_factors of the groups; sc: scales of the child and parent level
+__global__ void k_trans_build(int p, const double *G, const double *fac, int nfac, const double2 *sc, cd *up, cd *dn)
+{
+    const int P = (p + 1) * (p + 1);
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= P * P) return;
+    const int64_t g = blockIdx.y;
+    const int r = e / P, c = e % P;
+    int n = (int)sqrtf((float)r + 0.5f), n1 = (int)sqrtf((float)c + 0.5f);
+    while ((n + 1) * (n + 1) <= r) ++n;
+    while (n * n > r) --n;
+    while ((n1 + 1) * (n1 + 1) <= c) ++n1;
+    while (n1 * n1 > c) --n1;
+    const int mu = (r - n * n - n) - (c - n1 * n1 - n1), amu = abs(mu);
+    const double *jl = fac + g * nfac, *Pt = jl + 2 * (2 * p + 1), *ep = Pt + (2 * p + 1) * (2 * p + 2) / 2;
+    cd s{0.0, 0.0};
+    for (int j = 0; j <= p; ++j) {
+        const int l = abs(n - n1) + 2 * j;
+        if (l > n + n1) break;
+        if (l < amu) continue;
+        const double f = Pt[l * (l + 1) / 2 + amu] * G[(int64_t)e * (p + 1) + j];
+        s.x = fma(f, jl[2 * l], s.x);
+        s.y = fma(f, jl[2 * l + 1], s.y);
+    }
+    if (mu < 0 && (amu & 1)) s = -s;
+    s = s * cd{ep[2 * (mu + 2 * p)], ep[2 * (mu + 2 * p) + 1]};
+    double pc = 1.0, pr = 1.0, qc = 1.0, qr = 1.0;   // child, parent scale to the column's / row's degree
+    for (int i = 0; i < n1; ++i) {
+        pc *= sc[g].x;
+        qc *= sc[g].y;
+    }
+    for (int i = 0; i < n; ++i) {
+        pr *= sc[g].y;
+        qr *= sc[g].x;
+    }
+    const int64_t o = g * P * P + e;
+    up[o] = (pc / pr) * (ipow<double>(n1 - n) * s);
+    dn[o] = (qr / qc) * (ipow<double>(n - n1) * s);
+}
+
+// out = in (T != double: rounded once), transposed per matrix if tr
+template <typename T>
+__global__ void k_trans_copy(int P, int tr, const cd *in, cx<T> *out)
+{
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= P * P) return;
+    const int64_t g = (int64_t)blockIdx.y * P * P;
+    const cd v = in[g + (tr ? (e % P) * P + e / P : e)];
+    out[g + e] = cx<T>{(T)v.x, (T)v.y};
+}
+
+void launch_trans_build(int p, int nq, const double *w, const double *Pq, double *G, int64_t ng, const double *fac,
+                        const double2 *sc, cd *up, cd *dn, cudaStream_t st)
+{
+    const int P = (p + 1) * (p + 1), nb = (P * P + 127) / 128;
+    k_gaunt<<<nb, 128, 0, st>>>(p, nq, w, Pq, G);
+    if (ng > 0) k_trans_build<<<dim3(nb, (unsigned)ng), 128, 0, st>>>(p, G, fac, trans_factor_count(p), sc, up, dn);
+}
+
+template <typename T>
+void launch_trans_copy(int p, int64_t ng, bool tr, const cd *in, cx<T> *out, cudaStream_t st)
+{
+    const int P = (p + 1) * (p + 1);
+    if (ng > 0) k_trans_copy<T><<<dim3((P * P + 255) / 256, (unsigned)ng), 256, 0, st>>>(P, tr ? 1 : 0, in, out);
+}
+template void launch_trans_copy<float>(int, int64_t, bool, const cd *, cf *, cudaStream_t);
+template void launch_trans_copy<double>(int, int64_t, bool, const cd *, cd *, cudaStream_t);
+
 }  // namespace lmf

@@ -84,6 +84,14 @@ void launch_tab_batch(const GeomDev *dG, int g0, int nb, int qmax, const MediumD
                       const CompDev *dcomps, int p, const cd *dGten, const int *dcgidx,
                       cd *scratch, int64_t stride, cd *tab, int *dflag, cudaStream_t st);
 
+// translation matrices of ng groups on the device: the Gaunt coefficients (G: P^2 (p + 1)
+// doubles) from the nodes of gaunt_nodes, then M2M (up) and L2L (dn), [group][P][P]; fac
+// from trans_factors, sc the scales of the child and parent level
+void launch_trans_build(int p, int nq, const double *w, const double *Pq, double *G, int64_t ng, const double *fac,
+                        const double2 *sc, cd *up, cd *dn, cudaStream_t st);
+template <typename T>
+void launch_trans_copy(int p, int64_t ng, bool tr, const cd *in, cx<T> *out, cudaStream_t st);
+
 // k_fmm.cu
 cudaError_t configure_fmm_kernels();
 cudaError_t configure_tab_kernels();
@@ -189,14 +197,14 @@ cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, 
                           int *status, cudaStream_t st);
 // M2M or L2L on a persistent tensor-core kernel (k_m2l_tc.cu, p <= 12): items M2LWork{geom = translation group, t = 0,
 // npair, pair0} over pairs (tsrc[q], tdst[q]), 3 helical columns each; img holds
-// one tiled matrix per group (tile_matrix_tc2, tc2_matrix_bytes(p) each)
+// one tiled matrix per group (launch_tile_matrices, tc2_matrix_bytes(p) each)
 cudaError_t launch_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc,
                              const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
                              int *status, cudaStream_t st);
 bool trans_tc2_supported(int p);
 size_t trans_tc2_scratch_floats(int p, int nsm);
 size_t tc2_matrix_bytes(int p);
-void tile_matrix_tc2(int p, const cd *M, void *img);   // host: P x P row-major (row = output index)
+void launch_tile_matrices(int p, int64_t ng, const cd *M, void *img, cudaStream_t st);   // [ng][P][P], row = output index
 template <typename T>
 void launch_scale_tables(int p, int64_t g0, int64_t ng, const GeomDev *geoms, const cd *tab64,
                          cx<T> *tab, cudaStream_t st);
