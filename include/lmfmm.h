@@ -120,8 +120,9 @@ typedef struct {
     double ms_tabulate;    /* last build: M2L tabulation (node factors, Chebyshev integrals,
                               assembly), device time */
     double tab_flops;      /* ... its arithmetic: 8 real flops per complex multiply-add of the
-                              Chebyshev integrals (80 (tau, tau', table) combinations x (p+2)
-                              degrees x (2p+3) Bessel orders per node) and of the assembly
+                              Chebyshev integrals (80 (tau, tau', table) combinations, 50
+                              where source and target layer agree, x (p+2) degrees x (p+2)
+                              Bessel orders of one parity per node) and of the assembly
                               (5 P^2 (p+2) per geometry) */
     int adjoint_transposed; /* 1: lmfmm_matvec_adjoint applies the transposed operators (FP64
                                form, mixed form with tensor_cores = 0); 0: the reciprocity

@@ -569,6 +569,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     const double a = medium_a(ctx->med);
     std::vector<GeomDev> hg(ctx->geoms.size());
     int64_t qtot = 0;
+    double tab_terms = 0;   // per node: (tau, tau', table) combinations formed (10 of 16 within a layer)
     float ms_tab = 0.f;
     for (size_t i = 0; i < ctx->geoms.size(); ++i) {
         const Geom &g = ctx->geoms[i];
@@ -599,6 +600,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             return LMFMM_ERR_QUAD;
         }
         qtot += plan_nodes(gd.plan);
+        tab_terms += (double)plan_nodes(gd.plan) * NTAB * (c.l == c.lp ? 10 : 16);
         gd.tab_index = (int64_t)i;
         hg[i] = gd;
     }
@@ -864,7 +866,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     S.n_free_near_point_pairs = ctx->n_free_pp;
     S.ms_tabulate = ms_tab;
     S.adjoint_transposed = d->m2l_kernel <= 1;
-    S.tab_flops = 8.0 * (double)qtot * NTAB * 16 * (p + 2) * (2 * p + 3) +
+    S.tab_flops = 8.0 * tab_terms * (p + 2) * (p + 2) +
                   8.0 * (double)ctx->geoms.size() * NTAB * (double)P * P * (p + 2);
     return LMFMM_OK;
 }

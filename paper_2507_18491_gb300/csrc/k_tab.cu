@@ -85,48 +85,76 @@ __global__ void k_tab_nodes(const GeomDev *G, int g0, MediumDev M, const CompDev
     }
 }
 
-// I-breve[t][ts][tt][l][d] = sum_q base_t tau_s tau_t T_l J_d  for one
-// geometry, table t and source tau-type ts (blockIdx = (geometry, t*4+ts)).
-__global__ void k_tab_contract(const GeomDev *G, int g0, int LM, int DJ, const cd *Fb,
+// Bessel orders of I-breve that an entry can ask for: tau types 0, 1 belong to even orders m
+// and 2, 3 to odd ones, so d = m' - mu + kappa_t has one parity per (t, ts, tt) and only
+// every second order is formed: |d| = par + 2 h, h < tab_dh(DJ)
+__host__ __device__ inline int tab_par(int t, int ts, int tt)
+{
+    const int kap = t < 2 ? 0 : t < 4 ? 1 : 2;
+    return ((ts >> 1) + (tt >> 1) + kap) & 1;
+}
+__host__ __device__ inline int tab_dh(int DJ) { return (DJ + 1) / 2; }
+
+// I-breve[t][ts][tt][l][h] = sum_q base_t tau_s tau_t T_l J_d  for one
+// geometry, table t and source tau-type ts (blockIdx = (geometry, t*4+ts)).  In a
+// same-layer component the tau of both sides are the same functions: tt < ts is
+// the (tt, ts) block, which the assembly reads instead.
+__global__ void k_tab_contract(const GeomDev *G, int g0, const CompDev *comps, int LM, int DJ, const cd *Fb,
                                const cd *Fs, const cd *Ft, const cd *FT, const cd *FJ,
                                cd *Ibr, int64_t ibr_stride)
 {
     extern __shared__ unsigned char smraw[];
-    const int CH = 32;
+    const int CH = 32, DH = tab_dh(DJ);
     cd *W = (cd *)smraw;                 // [CH][4][LM]
     cd *Jc = W + CH * 4 * LM;            // [CH][DJ]
+    cd *Bq = Jc + CH * DJ;               // [CH][4]: base_t tau_s tau_t
     const GeomDev &g = G[g0 + blockIdx.x];
     int t = blockIdx.y / 4, ts = blockIdx.y % 4;
+    const CompDev c = comps[g.comp];
+    const int tt0 = c.l == c.lp ? ts : 0, ntt = 4 - tt0;
     int Q = g.plan.n1 + g.plan.nmid + 2 * g.plan.nray;
     const int64_t S = g.stride;
     int64_t o0 = g.node0;
-    const int NOUT = 4 * LM * DJ;
-    const int PER = 12;   // NOUT <= 12 * 256 for p <= 16
+    const int NOUT = ntt * LM * DH;
+    const int PER = 6;    // 4 LM DH <= 6 * 256 for p <= 16
     cd acc[PER];
-    for (int i = 0; i < PER; ++i) acc[i] = mkd(0.0);
+    int wi[PER], ji[PER];                // an output's W row and Bessel order
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        acc[i] = mkd(0.0);
+        const int out = min((int)(threadIdx.x + i * blockDim.x), NOUT - 1);
+        const int r = out / DH, tt = tt0 + r / LM;
+        wi[i] = r;
+        ji[i] = min(tab_par(t, ts, tt) + 2 * (out - r * DH), DJ - 1);
+    }
     for (int q0 = 0; q0 < Q; q0 += CH) {
         int nq = min(CH, Q - q0);
-        for (int e = threadIdx.x; e < nq * 4 * LM; e += blockDim.x) {
-            int q = e / (4 * LM), r = e % (4 * LM), tt = r / LM, l = r % LM;
-            int64_t o = o0 + q0 + q;
-            W[e] = Fb[t * S + o] * Fs[ts * S + o] * Ft[tt * S + o] * FT[l * S + o];
+        for (int e = threadIdx.x; e < nq * ntt; e += blockDim.x) {
+            const int q = e % nq, k = e / nq;
+            const int64_t o = o0 + q0 + q;
+            Bq[q * 4 + k] = Fb[t * S + o] * Fs[ts * S + o] * Ft[(tt0 + k) * S + o];
         }
         for (int e = threadIdx.x; e < nq * DJ; e += blockDim.x) {
             int q = e / DJ, dd = e % DJ;
             Jc[e] = FJ[dd * S + o0 + q0 + q];
         }
         __syncthreads();
+        for (int e = threadIdx.x; e < nq * ntt * LM; e += blockDim.x) {
+            int q = e / (ntt * LM), r = e % (ntt * LM), k = r / LM, l = r % LM;
+            W[q * 4 * LM + r] = Bq[q * 4 + k] * FT[l * S + o0 + q0 + q];
+        }
+        __syncthreads();
+#pragma unroll
         for (int i = 0; i < PER; ++i) {
-            int out = threadIdx.x + i * blockDim.x;
-            if (out >= NOUT) break;
-            int r = out / DJ, dd = out % DJ;
+            if ((int)(threadIdx.x + i * blockDim.x) >= NOUT) break;
             cd a = acc[i];
-            for (int q = 0; q < nq; ++q) a += W[q * 4 * LM + r] * Jc[q * DJ + dd];
+            for (int q = 0; q < nq; ++q) a += W[q * 4 * LM + wi[i]] * Jc[q * DJ + ji[i]];
             acc[i] = a;
         }
         __syncthreads();
     }
-    cd *dst = Ibr + (int64_t)blockIdx.x * ibr_stride + (int64_t)(t * 4 + ts) * NOUT;
+    cd *dst = Ibr + (int64_t)blockIdx.x * ibr_stride + (int64_t)((t * 4 + ts) * 4 + tt0) * LM * DH;
+#pragma unroll
     for (int i = 0; i < PER; ++i) {
         int out = threadIdx.x + i * blockDim.x;
         if (out < NOUT) dst[out] = acc[i];
@@ -144,7 +172,7 @@ __device__ inline int tau_type(int n, int am)
 
 // I-hat[t][row=(nu,mu)][col=(n',m')] = sgn(m') sgn(mu) sum_l G[(n',|m'|),(nu,|mu|)][l]
 //   * I-breve[t][tau(n',m')][tau(nu,mu)][l][|d|] * (-1)^d [d<0],  d = m' - mu + kappa_t
-__global__ void k_tab_assemble(const GeomDev *G, int g0, int p, int LM, int DJ, const cd *Gten,
+__global__ void k_tab_assemble(const GeomDev *G, int g0, const CompDev *comps, int p, int LM, int DJ, const cd *Gten,
                                const int *comp_gidx, const cd *Ibr, int64_t ibr_stride,
                                cd *tab)
 {
@@ -173,10 +201,16 @@ __global__ void k_tab_assemble(const GeomDev *G, int g0, int p, int LM, int DJ, 
     int ts = tau_type(n1, am1), tt = tau_type(nu, amu);
     const cd *Gp = Gten + ((int64_t)comp_gidx[g.comp] * T * T + (int64_t)(((n1 * (n1 + 1)) / 2 + am1) * T
                            + (nu * (nu + 1)) / 2 + amu)) * LM;
-    const cd *Ib = Ibr + (int64_t)blockIdx.z * ibr_stride + (int64_t)(t * 4 + ts) * (4 * LM * DJ)
-                   + (int64_t)tt * LM * DJ;
+    if (comps[g.comp].l == comps[g.comp].lp && tt < ts) {   // formed as (tt, ts)
+        const int x = tt;
+        tt = ts;
+        ts = x;
+    }
+    const int DH = tab_dh(DJ);
+    const cd *Ib = Ibr + (int64_t)blockIdx.z * ibr_stride + (int64_t)((t * 4 + ts) * 4 + tt) * LM * DH
+                   + ((ad - tab_par(t, ts, tt)) >> 1);
     cd s = mkd(0.0);
-    for (int l = 0; l < LM; ++l) s += Gp[l] * Ib[l * DJ + ad];
+    for (int l = 0; l < LM; ++l) s += Gp[l] * Ib[l * DH];
     tab[((int64_t)g.tab_index * NTAB + t) * P * P + e] = sgn * s;
 }
 
@@ -188,18 +222,17 @@ void launch_tab_batch(const GeomDev *dG, int g0, int nb, int qmax, const MediumD
                       cd *scratch, int64_t stride, cd *tab, int *dflag, cudaStream_t st)
 {
     const int LM = p + 2, DJ = 2 * p + 3, P = (p + 1) * (p + 1);
-    const int NOUT = 4 * LM * DJ;
-    const int64_t ibr_stride = (int64_t)NTAB * 4 * NOUT;
+    const int64_t ibr_stride = (int64_t)NTAB * 16 * LM * tab_dh(DJ);
     const int64_t S = stride;
     cd *Fb = scratch, *Fs = Fb + 5 * S, *Ft = Fs + 4 * S, *FT = Ft + 4 * S, *FJ = FT + LM * S;
     cd *Ibr = FJ + DJ * S;
     dim3 gn((qmax + 127) / 128, nb);
     k_tab_nodes<<<gn, 128, 0, st>>>(dG, g0, M, dcomps, LM, DJ, Fb, Fs, Ft, FT, FJ, dflag);
-    size_t sm = (size_t)(32 * 4 * LM + 32 * DJ) * sizeof(cd);
+    size_t sm = (size_t)(32 * 4 * LM + 32 * DJ + 32 * 4) * sizeof(cd);
     dim3 gc(nb, NTAB * 4);
-    k_tab_contract<<<gc, 256, sm, st>>>(dG, g0, LM, DJ, Fb, Fs, Ft, FT, FJ, Ibr, ibr_stride);
+    k_tab_contract<<<gc, 256, sm, st>>>(dG, g0, dcomps, LM, DJ, Fb, Fs, Ft, FT, FJ, Ibr, ibr_stride);
     dim3 ga((P * P + 255) / 256, NTAB, nb);
-    k_tab_assemble<<<ga, 256, 0, st>>>(dG, g0, p, LM, DJ, dGten, dcgidx, Ibr, ibr_stride, tab);
+    k_tab_assemble<<<ga, 256, 0, st>>>(dG, g0, dcomps, p, LM, DJ, dGten, dcgidx, Ibr, ibr_stride, tab);
 }
 
 }  // namespace lmf
