@@ -17,7 +17,7 @@
 // one before it waits for it (measured: 108 cycles per MMA whatever N from 112 to 176,
 // against N / 2 of arithmetic), so the five small products alternate between two
 // accumulators where three fit (N <= 128, p <= 8).
-// Roles (608 threads, one CTA per SM):
+// Roles (864 threads, one CTA per SM):
 //   warps 0-7   X producers, two groups of four warps (one per tensor-memory lane
 //               quadrant), group g writing K-step g of every chunk: the two coefficients of
 //               an input lie side by side in the packed expansions (k_sec_pack), so that a
@@ -26,15 +26,15 @@
 //               coefficient touches 32 lines per instruction: 0.95 against 0.76 ms for 397328
 //               pairs at p = 7); then one phase per input, the split into three pieces (the
 //               two rows of a pair share them) and the store into the tensor-memory ring;
-//   warps 8-15  epilogue: accumulators -> a per-CTA scratch in global memory (L2-resident)
+//   warps 8-23  epilogue: accumulators -> a per-CTA scratch in global memory (L2-resident)
 //               as four-row groups, 16 bytes per real column, so that every store
 //               instruction writes 512 contiguous bytes and tensor memory is free again at
 //               once; after the item's last tile one warp per pair combines the two
 //               sectors, applies the output phases into a shared staging row [3][P] and
 //               adds it to the pair's local expansions with one bulk reduction;
-//   warp 16     one bulk copy per matrix chunk into a shared-memory ring;
-//   warp 17     MMA issue;
-//   warp 18     bulk copies of the pair records and phases, one item ahead.
+//   warp 24     one bulk copy per matrix chunk into a shared-memory ring;
+//   warp 25     MMA issue;
+//   warp 26     bulk copies of the pair records and phases, one item ahead.
 // Every wait is bounded; a wait that gives up sets bit 4 of the status word and its role
 // stops.
 //
@@ -62,7 +62,7 @@ constexpr int SC_ST_MAX = 12;      // matrix ring slots
 constexpr int SC_XD = 3;           // stages of a producer warp's shared ring of packed inputs
 constexpr uint32_t SC_XROW = 144;  // bytes of a pair's K-step there: 8 inputs of 16 bytes, padded against bank conflicts
 constexpr uint32_t SC_XST = 16 * SC_XROW;
-constexpr int SC_PT = 256, SC_ET = 256;     // producer, epilogue threads
+constexpr int SC_PT = 256, SC_ET = 512;     // producer, epilogue threads
 constexpr int SC_EW = SC_ET / 32;
 constexpr int SC_WTMA = (SC_PT + SC_ET) / 32, SC_WMMA = SC_WTMA + 1, SC_WMETA = SC_WTMA + 2;
 constexpr int SC_THREADS = (SC_WMETA + 1) * 32;
@@ -78,7 +78,7 @@ struct SecTile {
 };
 
 struct SecPlan {
-    int p, P, D0, D1, ntile, nmax, nacc, SX, ST, nchunk0, yrows, npp;
+    int p, P, D0, D1, ntile, nmax, nacc, SX, ST, nchunk0, yrows, ews;
     uint32_t slot, img_bytes, ph_bytes, meta_bytes, stage_bytes;
     uint32_t o_meta, o_ent, o_xsrc, o_stage, o_bars, smem;
     SecTile t[SC_MAXT];
@@ -121,16 +121,16 @@ SecPlan sec_plan(int p)
     s.ph_bytes = (uint32_t)m2l_sec_phases(p) * 8;
     s.meta_bytes = SC_BN * (s.ph_bytes + (uint32_t)sizeof(M2LPair));
     s.stage_bytes = ((uint32_t)(3 * s.P + 2) * 8 + 15) & ~15u;
-    s.npp = s.D0 <= 128 ? 2 : 1;
+    s.ews = s.D0 <= 128 ? SC_EW : SC_EW / 2;   // epilogue warps that scatter: their staging rows take shared memory
     const uint32_t bars = (2 * SC_ST_MAX + 2 * SC_SX_MAX + 12) * 8 + 16;
     const uint32_t ent = (uint32_t)s.nchunk0 * SC_KC * 4;
-    const uint32_t fixed = 2 * s.meta_bytes + ent + SC_PT / 32 * SC_XD * SC_XST + SC_EW * s.npp * s.stage_bytes + bars;
+    const uint32_t fixed = 2 * s.meta_bytes + ent + SC_PT / 32 * SC_XD * SC_XST + s.ews * s.stage_bytes + bars;
     s.ST = (int)std::min<uint32_t>(SC_ST_MAX, (SC_SMEM_MAX - fixed) / s.slot);
     s.o_meta = s.ST * s.slot;
     s.o_ent = s.o_meta + 2 * s.meta_bytes;
     s.o_xsrc = s.o_ent + ent;
     s.o_stage = s.o_xsrc + SC_PT / 32 * SC_XD * SC_XST;
-    s.o_bars = s.o_stage + SC_EW * s.npp * s.stage_bytes;
+    s.o_bars = s.o_stage + s.ews * s.stage_bytes;
     s.smem = s.o_bars + bars;
     return s;
 }
@@ -155,13 +155,6 @@ __device__ __forceinline__ void split_bf16(float lo, float hi, uint32_t (&w)[SC_
             r = float2{r.x - f.x, r.y - f.y};
         }
     }
-}
-
-// A bulk reduction wants 16-byte alignment on both sides: 1 if the expansions of box `box`
-// start 8 bytes off it (their first element is then added by itself)
-__device__ __forceinline__ int stage_head(const cf *le, int64_t box, int P)
-{
-    return (int)(((uintptr_t)(le + box * 3 * P) >> 3) & 1);
 }
 
 // RJ: rows of the even sector per lane of an epilogue warp (32 RJ >= D0)
@@ -340,25 +333,25 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
         const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
         const uint32_t ent0 = tc::smem_u32(ent) + 4 * kk0;
         const uint32_t ring = tc::smem_u32(smraw + sp.o_xsrc) + warp * (SC_XD * SC_XST);
-        const size_t box_bytes = (size_t)sp.nchunk0 * SC_KC * 16;
+        const int64_t box_units = sp.nchunk0 * SC_KC;
         // fetch side: lane copies 16-byte unit lane % 8 of the lines of pairs lane / 8 + 4 i
         const uint32_t dst0 = ring + (lane >> 3) * SC_XROW + 16 * (lane & 7);
         int64_t fit = blockIdx.x;
         uint32_t fli = 0;
         int ft = sp.ntile, fc = 0, fst = 0;    // no tile open yet; next stage to fill
-        const unsigned char *fsrc[4];
-        bool fval[4] = {false, false, false, false};
+        const float4 *fme = nullptr;           // packed expansions of the item's problem
+        constexpr uint32_t NONE = 0xffffffffu;
+        uint32_t fsrc[4] = {NONE, NONE, NONE, NONE};   // boxes; none: no such pair
         auto fetch = [&]() -> bool {
             if (ft == sp.ntile && fit < nwork) {      // open the next item
                 const int slot = fli & 1;
                 if (!__all_sync(0xffffffffu, tc::mbar_wait(&metafull[slot], (fli >> 1) & 1, SC_POLLS))) return false;
                 const M2LWork w = work[fit];
-                const unsigned char *me = (const unsigned char *)prob(w).me;
+                fme = (const float4 *)prob(w).me + 8 * pg + (lane & 7);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     const int c = pq + (lane >> 3) + 4 * i;
-                    fval[i] = c < w.npair;
-                    if (fval[i]) fsrc[i] = me + meta_pair(slot)[c].src * box_bytes + 128 * pg + 16 * (lane & 7);
+                    fsrc[i] = c < w.npair ? (uint32_t)meta_pair(slot)[c].src : NONE;
                 }
                 ft = fc = 0;
                 ++fli;
@@ -367,10 +360,10 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
             if (ft < sp.ntile) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (fval[i])
+                    if (fsrc[i] != NONE)
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
                                          dst0 + fst * SC_XST + 4 * i * SC_XROW),
-                                     "l"(fsrc[i] + (size_t)fc * (SC_KC * 16))
+                                     "l"(fme + ((int64_t)fsrc[i] * box_units + fc * SC_KC))
                                      : "memory");
                 if (++fc == sp.t[ft].nchunk) {
                     fc = 0;
@@ -381,6 +374,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
             fst = fst + 1 == SC_XD ? 0 : fst + 1;
             return true;
         };
+        const uint32_t sel_lo = b ? 0x5476u : 0x3210u, sel_hi = b ? 0x1032u : 0x7654u, sgn = b ? 0u : 0x80000000u;
         uint32_t li = 0, g = 0, xph = 0;       // items, chunks of this CTA so far
         int xs = 0, cst = 0;                   // tensor-memory slot and stage of chunk g
         for (int u = 0; u < SC_XD - 1 && !failed; ++u) failed = !fetch();
@@ -427,15 +421,15 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
 #pragma unroll
                         for (int pc = 0; pc < SC_NPC; ++pc) oth[h][pc] = __shfl_xor_sync(0xffffffffu, own[h][pc], 1);
                     // the K-step's eight inputs in this lane's row: (Re, -Im) = negated high
-                    // half, (Im, Re) = swapped halves; columns piece-major, even K in the low half
+                    // half, (Im, Re) = swapped halves; columns piece-major, even K in the low
+                    // half.  One byte permutation picks own or partner's word and swaps
                     uint32_t rw[8 * SC_NPC];
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
 #pragma unroll
-                        for (int pc = 0; pc < SC_NPC; ++pc) {
-                            const uint32_t wv = (i < KQ) == (b == 0) ? own[i & (KQ - 1)][pc] : oth[i & (KQ - 1)][pc];
-                            rw[i + 8 * pc] = b ? __byte_perm(wv, 0, 0x1032) : (wv ^ 0x80000000u);
-                        }
+                        for (int pc = 0; pc < SC_NPC; ++pc)
+                            rw[i + 8 * pc] =
+                                __byte_perm(own[i & (KQ - 1)][pc], oth[i & (KQ - 1)][pc], i < KQ ? sel_lo : sel_hi) ^ sgn;
                     const uint32_t ta = lane_base + xb + SC_XW * xs + 8 * SC_NPC * pg;
                     static_assert(SC_KS == 2 && SC_NPC == 3, "two K-steps of 24 columns per chunk");
                     if (pg == 0) {
@@ -463,11 +457,11 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
     } else if (warp < SC_WTMA) {
         // ------------------------------------------------ epilogue
         const int ea = tid - SC_PT, ew = ea >> 5;     // epilogue warp 0 .. SC_EW-1
-        const int q4 = warp & 3, half = ea / 128;     // lane quadrant, slab parity
+        const int q4 = warp & 3, part = ea / 128;     // lane quadrant, first slab
         const uint32_t lane_base = tbase + ((uint32_t)(32 * q4) << 16);
-        constexpr int RB = RJ <= 4 ? RJ : 3;
-        constexpr int NPP = RJ <= 4 ? 2 : 1;          // sec_plan's npp
-        float2 *stage = (float2 *)(smraw + sp.o_stage + ew * sp.npp * sp.stage_bytes);
+        constexpr int RB = RJ == 4 ? 2 : 3;
+        constexpr int EWS = RJ <= 4 ? SC_EW : SC_EW / 2;   // sec_plan's ews
+        float2 *stage = (float2 *)(smraw + sp.o_stage + ew * sp.stage_bytes);
         const int yodd = sp.t[sp.ntile / 2].y0;       // scratch row of the odd sector
         uint32_t li = 0, tc_n = 0;
         for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x, ++li) {
@@ -488,7 +482,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
                 tc::fence_after();
                 const int N = sp.t[t].N;
                 float4 *Yt = (float4 *)Y + (size_t)(sp.t[t].y0 >> 2) * 128 + 32 * q4 + lane;
-                for (int c0 = 16 * half; c0 < N; c0 += 32) {   // N is a multiple of 16
+                for (int c0 = 16 * part; c0 < N; c0 += SC_ET / 8) {   // N is a multiple of 16
                     uint32_t va[16], vb[16];
                     tc::tmem_ld16(lane_base + sp.nmax + c0, va);
                     if (sp.nacc == 3) {
@@ -522,13 +516,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
             }
             cf *const le = prob(w).le;
             const uint32_t gr = tc::smem_u32(meta_ph(slot));
-            // NPP pairs at a time: their scratch rows are loaded together, and one proxy fence (it
-            // waits for the warp's outstanding memory operations) serves all of them
-            for (int c0 = ew; c0 < w.npair; c0 += NPP * SC_EW) {
-                const int np = NPP == 1 ? 1 : min(NPP, (w.npair - c0 + SC_EW - 1) / SC_EW);
-                // row i0 + i of pair c0 + 8 u; clamped where there is none, masked at use
-                auto load = [&](int u, int i0, float2 (&ye)[RB], float2 (&yo)[RB]) {
-                    const int c = min(c0 + u * SC_EW, SC_BN - 1);
+            for (int c = ew; ew < EWS && c < w.npair; c += EWS) {
+                // RB rows per lane and step
+                auto load = [&](int i0, float2 (&ye)[RB], float2 (&yo)[RB]) {
 #pragma unroll
                     for (int i = 0; i < RB; ++i) {
                         const int r = min(lane + 32 * (i0 + i), sp.D0 - 1), ro = yodd + min(r, sp.D1 - 1);
@@ -538,57 +528,51 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
                         yo[i] = float2{b[0], b[4]};
                     }
                 };
-                float2 ye[NPP][RB], yo[NPP][RB];
-#pragma unroll
-                for (int u = 0; u < NPP; ++u) load(u, 0, ye[u], yo[u]);
+                float2 ye[RB], yo[RB];
+                load(0, ye, yo);
+                cf *dst = le + meta_pair(slot)[c].tgt * 3 * P;
+                // the reduction wants 16-byte alignment on both sides: an odd first element and the
+                // last one left over are added by an atomic
+                const int head = (int)(((uintptr_t)dst >> 3) & 1), body = (3 * P - head) & ~1;
+                float2 *sg = stage + head;
                 asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
                 __syncwarp();
 #pragma unroll 1
                 for (int i0 = 0; i0 < RJ; i0 += RB) {
-                    if (i0 > 0) load(0, i0, ye[0], yo[0]);       // NPP == 1 where RJ > RB
+                    if (i0 > 0) load(i0, ye, yo);
+                    // no branch between the rows: their entry words and phases are fetched together
+                    uint32_t we[RB];
+                    cf G[RB];
 #pragma unroll
-                    for (int u = 0; u < NPP; ++u) {
-                        if (u >= np) break;
-                        const int c = c0 + u * SC_EW;
-                        float2 *sg = stage + u * (sp.stage_bytes / 8) + stage_head(le, meta_pair(slot)[c].tgt, P);
+                    for (int i = 0; i < RB; ++i) we[i] = ent[min(lane + 32 * (i0 + i), sp.D0 - 1)];
 #pragma unroll
-                        for (int i = 0; i < RB; ++i) {
-                            const int r = lane + 32 * (i0 + i);
-                            if (r < sp.D0) {
-                                if (r >= sp.D1) yo[u][i] = float2{0.f, 0.f};
-                                const uint32_t we = ent[r];
-                                const cf G = lds_c(gr + c * sp.ph_bytes + 8 * ((we >> 20) & 63));
-                                const float2 s{ye[u][i].x + yo[u][i].x, ye[u][i].y + yo[u][i].y};
-                                float2 d{ye[u][i].x - yo[u][i].x, ye[u][i].y - yo[u][i].y};
-                                sg[we & 1023] = float2{fmaf(G.x, s.x, G.y * s.y), fmaf(G.x, s.y, -G.y * s.x)};
-                                if (!(we >> 26 & 1)) d = float2{-d.x, -d.y};
-                                if (!(we >> 27 & 1))
-                                    sg[(we >> 10) & 1023] =
-                                        float2{fmaf(G.x, d.x, -G.y * d.y), fmaf(G.x, d.y, G.y * d.x)};
-                            }
-                        }
+                    for (int i = 0; i < RB; ++i) G[i] = lds_c(gr + c * sp.ph_bytes + 8 * ((we[i] >> 20) & 63));
+#pragma unroll
+                    for (int i = 0; i < RB; ++i) {
+                        const int r = lane + 32 * (i0 + i);
+                        const float ko = r < sp.D1 ? 1.f : 0.f, kd = (we[i] >> 26 & 1) ? 1.f : -1.f;
+                        const float2 o{ko * yo[i].x, ko * yo[i].y};
+                        const float2 s{ye[i].x + o.x, ye[i].y + o.y};
+                        const float2 d{kd * (ye[i].x - o.x), kd * (ye[i].y - o.y)};
+                        const cf g = G[i];
+                        if (r < sp.D0) sg[we[i] & 1023] = float2{fmaf(g.x, s.x, g.y * s.y), fmaf(g.x, s.y, -g.y * s.x)};
+                        if (r < sp.D0 && !(we[i] >> 27 & 1))
+                            sg[(we[i] >> 10) & 1023] = float2{fmaf(g.x, d.x, -g.y * d.y), fmaf(g.x, d.y, g.y * d.x)};
                     }
                 }
                 tc::fence_smem_async();
                 __syncwarp();
-                // lane 4u reduces pair u's body; its first and last odd elements go by atomics
-                if ((lane >> 2) < np) {
-                    const int u = lane >> 2, c = c0 + u * SC_EW;
-                    cf *dst = le + meta_pair(slot)[c].tgt * 3 * P;
-                    const int head = stage_head(le, meta_pair(slot)[c].tgt, P), body = (3 * P - head) & ~1;
-                    const float2 *sg = stage + u * (sp.stage_bytes / 8) + head;
-                    if ((lane & 3) == 0) {
-                        asm volatile("cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;" ::"l"(
-                                         dst + head),
-                                     "r"(tc::smem_u32(sg + head)), "r"((uint32_t)body * 8)
-                                     : "memory");
-                    } else if ((lane & 3) == 1 && head) {
-                        atomicAdd((float2 *)dst, sg[0]);
-                    } else if ((lane & 3) == 2 && head + body < 3 * P) {
-                        atomicAdd((float2 *)dst + head + body, sg[head + body]);
-                    }
+                if (lane == 0) {
+                    asm volatile(
+                        "cp.reduce.async.bulk.global.shared::cta.bulk_group.add.f32 [%0], [%1], %2;\n\t"
+                        "cp.async.bulk.commit_group;" ::"l"(dst + head),
+                        "r"(tc::smem_u32(sg + head)), "r"((uint32_t)body * 8)
+                        : "memory");
+                } else if (lane == 1 && head) {
+                    atomicAdd((float2 *)dst, sg[0]);
+                } else if (lane == 2 && head + body < 3 * P) {
+                    atomicAdd((float2 *)dst + head + body, sg[head + body]);
                 }
-                asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
             tc::mbar_arrive(yfree);
             __syncwarp();
