@@ -668,11 +668,16 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         CK(cudaGetLastError());
         sec_work_items(ctx, m2l_sec_pairs(), 0, mw);
     } else if (d->oz) {
-        // smaller items where full ones would leave SMs idle
-        for (int pairs = m2l_oz_pairs(); pairs >= m2l_oz_pairs() / 4; pairs /= 2) {
-            mw.clear();
-            sec_work_items(ctx, pairs, 0, mw);
-            if ((int64_t)mw.size() >= d->nsm) break;
+        // an item's time hardly depends on its pairs (padded products, one pass of phases): halve
+        // them while the items still make one round of CTAs
+        int pairs = m2l_oz_pairs();
+        sec_work_items(ctx, pairs, 0, mw);
+        while (pairs > m2l_oz_pairs() / 4) {
+            std::vector<M2LWork> half;
+            sec_work_items(ctx, pairs / 2, 0, half);
+            if ((int64_t)half.size() > d->nsm) break;
+            mw = half;
+            pairs /= 2;
         }
     } else {
         m2l_work_items(ctx, d->m2l_kernel == 2 ? m2l_tc_cols() : f32 ? gemm_cols<float>() : gemm_cols<double>(), 0, mw);
