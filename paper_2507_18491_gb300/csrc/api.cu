@@ -29,6 +29,7 @@ struct DevState {
     int *pt_box = nullptr;           // leaf box of every sorted point (mixed form)
     LeafUnit *units = nullptr;       // P2M units: at most 128 points of one leaf, largest first
     int64_t nunits = 0;
+    bool p2m_many = false;           // P2M by the kernel for units of many points
     bool leaf_fast = false;          // mixed form, p <= 15: P2M and L2P of k_leaf.cu
     cd *qh = nullptr, *ph = nullptr; // helical, sorted [N][3]
     void *me = nullptr, *le = nullptr; // [nbox][3][P], complex T (scaled)
@@ -539,6 +540,11 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         TRY(dupload(ctx, &d->pt_box, ptb));
         TRY(dupload(ctx, &d->units, units));
         d->nunits = (int64_t)units.size();
+        // k_p2m_ms takes a time per point, k_p2m_pt one per unit (two layers at depth 5, 7.5 / 30 / 60 /
+        // 120 points per unit: p = 6 45 / 84 / 143 / 239 against 65 / 74 / 86 / 127 us, p = 8 53 / 98 /
+        // 172 / 288 against 91 / 106 / 123 / 192, p = 12 73 / 139 / 242 / 415 against 204 / 210 / 236 / 339);
+        // they meet near 5 p points.  Not both in one call: two launches in a row lose more
+        d->p2m_many = N > 5 * p * d->nunits;
         d->leaf_fast = true;
     }
     TRY(dalloc(ctx, &d->qh, 3 * N));
@@ -887,7 +893,7 @@ static void leaf_p2m(lmfmm_ctx *ctx, const cd *in, cx<T> *out, bool l2p_basis, c
     const int p = ctx->prm.p;
     if constexpr (std::is_same<T, float>::value) {
         if (d->leaf_fast) {
-            launch_p2m_fast(p, d->nunits, d->units, d->boxes, d->xyz, in, ctx->med, d->lscale, out, !l2p_basis,
+            launch_p2m_fast(p, d->nunits, d->p2m_many, d->units, d->boxes, d->xyz, in, ctx->med, d->lscale, out, !l2p_basis,
                             l2p_basis ? 1.0 : 4.0 * 3.14159265358979323846, st);
             return;
         }

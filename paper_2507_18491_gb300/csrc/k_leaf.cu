@@ -15,7 +15,9 @@
 //             it goes (read through L1: the threads of a warp mostly share a leaf);
 //   k_p2m_ms  one warp per unit of at most 128 points of one leaf (units largest
 //             first); each lane keeps the coefficients of its own pair of orders
-//             in registers over a stream of points (see the kernel).
+//             in registers over a stream of points (see the kernel);
+//   k_p2m_pt  the same for units of many points: lanes take points, the sums over
+//             them are transposing butterflies.
 // The recurrence coefficients live in constant memory and every loop over
 // (n, m) is unrolled for the compile-time p, so they are immediate operands.
 #include <cmath>
@@ -329,12 +331,145 @@ __global__ void __launch_bounds__(32, 12) k_p2m_ms(const LeafUnit *units, const 
     }
 }
 
+// The same sums for units of many points, one warp per unit.  Each lane
+// takes up to four points.  It forms their seeds (cos theta, e^{-i phi} or e^{i phi}, radial
+// factors, charges) into its own columns of shared memory, then walks the orders m: the
+// Legendre recurrence in n of each of its points, the products with the three charges
+// added up in registers for n = m..p and both signs.  The sums over the lanes are one
+// transposing butterfly per order (a step halves the values a lane holds: NV (1 - 1/32)
+// shuffles for NV values instead of 5 NV), which leaves every lane with NV / 32 finished
+// coefficients.  Bound by the FP32 pipe; lanes = pairs of orders over a stream of points
+// instead kept 5 of 8 lanes busy at p = 8 and reloaded the seeds per order.
+constexpr int P2M_PTS = 4;
+
 template <int PP>
-void launch_p2m_pp(int64_t nunit, const LeafUnit *units, const BoxDev *boxes, const double *xyz, const cd *qh,
+struct P2mCols {                    // [.][lane + 32 k]
+    float x[128], sv[128], pm[128];
+    float2 e1[128], em[128], q[3][128], jr[PP + 1][128];
+};
+
+template <int N, int O, int NV>
+__device__ __forceinline__ void butterfly_sum(float (&a)[NV], int lane)
+{
+    const bool up = (lane & O) != 0;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) {
+        const float keep = up ? a[i + N / 2] : a[i], send = up ? a[i] : a[i + N / 2];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, O);
+    }
+    if constexpr (O > 1) butterfly_sum<N / 2, O / 2>(a, lane);
+}
+
+// order m of one unit: NV = 32-padded count of the floats of n = m..PP x signs x 3 x (re, im)
+template <int PP, int M_>
+__device__ __forceinline__ void p2m_order(P2mCols<PP> &sd, int np, int lane, cf *out, bool whole)
+{
+    constexpr int P = (PP + 1) * (PP + 1), NS = M_ == 0 ? 1 : 2, NC = (PP - M_ + 1) * NS * 6;
+    constexpr int NV = (NC + 31) / 32 * 32;
+    float a[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) a[i] = 0.f;
+#pragma unroll 1
+    for (int pt = lane; pt < np; pt += 32) {
+        const float x = sd.x[pt];
+        float pmm = c_lc[0];
+        float2 em{1.f, 0.f};
+        if constexpr (M_ > 0) {
+            const float2 e = sd.em[pt], e1 = sd.e1[pt];
+            pmm = -sd.pm[pt] * sd.sv[pt] * c_lc[M_];
+            em = float2{e.x * e1.x - e.y * e1.y, e.x * e1.y + e.y * e1.x};
+        }
+        sd.pm[pt] = pmm;
+        sd.em[pt] = em;
+        const float2 q0 = sd.q[0][pt], q1 = sd.q[1][pt], q2 = sd.q[2][pt];
+        float p0 = 0.f, p1 = 0.f;
+#pragma unroll
+        for (int n = M_; n <= PP; ++n) {
+            float pl;
+            if (n == M_) pl = pmm;
+            else if (n == M_ + 1) pl = c_ld[M_] * x * pmm;
+            else pl = c_la[n * (n + 1) / 2 + M_] * (x * p1 - c_lb[n * (n + 1) / 2 + M_] * p0);
+            p0 = p1;
+            p1 = pl;
+            const float2 jr = sd.jr[n][pt];
+            const float jx = pl * jr.x, jy = pl * jr.y;
+#pragma unroll
+            for (int h = 0; h < NS; ++h) {
+                // e^{i m phi}, or (-1)^m conj of it for -m
+                const float ex = (h && (M_ & 1)) ? -em.x : em.x, ey = (h && !(M_ & 1)) ? -em.y : em.y;
+                const float bx = jx * ex - jy * ey, by = jx * ey + jy * ex;
+                float *t = a + ((n - M_) * NS + h) * 6;
+                t[0] = fmaf(q0.x, bx, fmaf(-q0.y, by, t[0]));
+                t[1] = fmaf(q0.x, by, fmaf(q0.y, bx, t[1]));
+                t[2] = fmaf(q1.x, bx, fmaf(-q1.y, by, t[2]));
+                t[3] = fmaf(q1.x, by, fmaf(q1.y, bx, t[3]));
+                t[4] = fmaf(q2.x, bx, fmaf(-q2.y, by, t[4]));
+                t[5] = fmaf(q2.x, by, fmaf(q2.y, bx, t[5]));
+            }
+        }
+    }
+    butterfly_sum<NV, 16>(a, lane);
+    // the lane's values: those whose index has its bits, in steps of NV / 32
+    int base = 0;
+#pragma unroll
+    for (int o = 16, n = NV / 2; o > 0; o >>= 1, n >>= 1)
+        if (lane & o) base += n;
+#pragma unroll
+    for (int i = 0; i < NV / 32; ++i) {
+        const int e = base + i;
+        if (e < NC) {
+            const int c = e / 6, r = e - 6 * c, n = M_ + c / NS, h = c % NS;
+            float *o = (float *)(out + (r >> 1) * P + n * n + n + (h ? -M_ : M_)) + (r & 1);
+            if (whole) *o = a[i];
+            else atomicAdd(o, a[i]);
+        }
+    }
+}
+
+template <int PP, int M_>
+__device__ __forceinline__ void p2m_orders(P2mCols<PP> &sd, int np, int lane, cf *out, bool whole)
+{
+    p2m_order<PP, M_>(sd, np, lane, out, whole);
+    if constexpr (M_ < PP) p2m_orders<PP, M_ + 1>(sd, np, lane, out, whole);
+}
+
+template <int PP>
+__global__ void __launch_bounds__(32) k_p2m_pt(const LeafUnit *units, const BoxDev *boxes, const double *xyz,
+                                               const cd *qh, MediumDev M, LayerScale ls, cf *me, int conj_basis,
+                                               double scale)
+{
+    constexpr int P = (PP + 1) * (PP + 1);
+    __shared__ P2mCols<PP> sd;
+    const LeafUnit u = units[blockIdx.x];
+    const BoxDev b = boxes[u.box];
+    const int lane = threadIdx.x, np = (int)(u.i1 - u.i0);
+    static_assert(P2M_PTS * 32 == 128, "a unit's points");
+    for (int pt = lane; pt < np; pt += 32) {
+        const int64_t i = u.i0 + pt;
+        float x, sv;
+        cf e1, jr[PP + 1];
+        leaf_seed<PP>(M.k[b.layer], xyz[3 * i] - b.c[0], xyz[3 * i + 1] - b.c[1], xyz[3 * i + 2] - b.c[2],
+                      conj_basis != 0, scale, 1.0 / ls.s[b.layer], x, sv, e1, jr);
+        sd.x[pt] = x;
+        sd.sv[pt] = sv;
+        sd.e1[pt] = float2{e1.x, e1.y};
+#pragma unroll
+        for (int n = 0; n <= PP; ++n) sd.jr[n][pt] = float2{jr[n].x, jr[n].y};
+#pragma unroll
+        for (int v = 0; v < 3; ++v) sd.q[v][pt] = float2{(float)qh[3 * i + v].x, (float)qh[3 * i + v].y};
+    }
+    p2m_orders<PP, 0>(sd, np, lane, me + (int64_t)u.box * 3 * P, u.whole != 0);
+}
+
+template <int PP>
+void launch_p2m_pp(int64_t nunit, bool many, const LeafUnit *units, const BoxDev *boxes, const double *xyz, const cd *qh,
                    const MediumDev &M, const LayerScale &ls, cf *me, bool conj_basis, double scale, cudaStream_t st)
 {
     if (nunit <= 0) return;
-    k_p2m_ms<PP><<<(unsigned)nunit, 32, 0, st>>>(units, boxes, xyz, qh, M, ls, me, conj_basis ? 1 : 0, scale);
+    if (many)
+        k_p2m_pt<PP><<<(unsigned)nunit, 32, 0, st>>>(units, boxes, xyz, qh, M, ls, me, conj_basis ? 1 : 0, scale);
+    else
+        k_p2m_ms<PP><<<(unsigned)nunit, 32, 0, st>>>(units, boxes, xyz, qh, M, ls, me, conj_basis ? 1 : 0, scale);
 }
 
 template <int PP>
@@ -366,14 +501,14 @@ void launch_l2p_fast(int p, int64_t N, const int *pt_box, const BoxDev *boxes, c
     }
 }
 
-void launch_p2m_fast(int p, int64_t nunit, const LeafUnit *units, const BoxDev *boxes, const double *xyz,
+void launch_p2m_fast(int p, int64_t nunit, bool many, const LeafUnit *units, const BoxDev *boxes, const double *xyz,
                      const cd *qh, const MediumDev &M, const LayerScale &ls, cf *me, bool conj_basis, double scale,
                      cudaStream_t st)
 {
     switch (p) {
 #define LF_CASE(v)                                                                                           \
     case v:                                                                                                  \
-        launch_p2m_pp<v>(nunit, units, boxes, xyz, qh, M, ls, me, conj_basis, scale, st);                    \
+        launch_p2m_pp<v>(nunit, many, units, boxes, xyz, qh, M, ls, me, conj_basis, scale, st);                    \
         break;
         LF_CASES(LF_CASE)
 #undef LF_CASE

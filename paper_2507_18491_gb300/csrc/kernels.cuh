@@ -124,7 +124,8 @@ void launch_l2p_fast(int p, int64_t N, const int *pt_box, const BoxDev *boxes, c
                      cudaStream_t st);
 // P2M of the mixed form for p <= 15: one warp per unit, me (cf [box][3][P], zeroed
 // beforehand) += the coefficients of the helical charges qh (cd, sorted)
-void launch_p2m_fast(int p, int64_t nunit, const LeafUnit *units, const BoxDev *boxes, const double *xyz,
+// (many: the kernel for units of many points)
+void launch_p2m_fast(int p, int64_t nunit, bool many, const LeafUnit *units, const BoxDev *boxes, const double *xyz,
                      const cd *qh, const MediumDev &M, const LayerScale &ls, cf *me, bool conj_basis, double scale,
                      cudaStream_t st);
 

@@ -73,3 +73,18 @@ def test_fp64_form(p):
     assert rel(mv(w.J), a) < 1e-13
     op.check()
     op.close()
+
+
+@pytest.mark.parametrize("p", [2, 8, 12])
+def test_p2m_of_crowded_leaves(p):
+    # 69 points per unit on average, above the 5 p at which the kernel for many points takes over;
+    # units of a partial pass (69 = 2 x 32 + 5) and of one pass both occur.  FP32 expansions
+    # against the FP64 form: the mixed form's bar
+    w = W.paper_table_uniform(m=50000, layers=2, p=p)
+    J = torch.from_numpy(w.J).cuda()
+    out = []
+    for kw in (dict(), dict(precision=lmfmm.MIXED, tensor_cores=1)):
+        op = lmfmm.Operator(w.d, w.k, w.xyz, p=p, depth=4, theta=0.55, **kw).build()
+        out.append(op.matvec(J).cpu().numpy())
+        op.close()
+    assert rel(out[1], out[0]) < 2e-6
