@@ -118,6 +118,20 @@ __device__ __forceinline__ void oz_digits(double x, uint32_t (&w)[OZ_S])
     }
 }
 
+// c (hi + 2^-32 lo), c a power of two, |hi| and |lo| below 2^51, rounded once.  Two operations of
+// the FP64 pipe (conversions run there too): an integer added to the bits of 1.5 2^52 is a
+// double, the offsets of both terms come off in one subtraction, and c is an exponent.
+__device__ __forceinline__ double oz_value(long long hi, long long lo, double c)
+{
+    constexpr long long B = 0x4338000000000000ll;              // bits of 1.5 2^52
+    const double h = __longlong_as_double(B + hi), l = __longlong_as_double(B + lo);
+    const double v = fma(0x1p-32, l, h - (0x1.8p52 + 0x1.8p20));
+    const int ev = (int)(__double_as_longlong(v) >> 52) & 0x7ff, ec = (int)(__double_as_longlong(c) >> 52) & 0x7ff;
+    const int e = ev + ec - 1023;
+    if (ev == 0 || ec == 0 || e <= 0 || e >= 0x7ff) return c * v;   // zero, or beyond the normal range
+    return __longlong_as_double(__double_as_longlong(v) + ((long long)(ec - 1023) << 52));
+}
+
 __device__ __forceinline__ void mma_f16_ss(uint32_t d, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
@@ -201,8 +215,9 @@ __global__ void __launch_bounds__(OZ_T, 1)
                         const uint32_t we = ent[4 * hk + h];
                         const double2 G = lds_d2(ph0 + c * sp.ph_bytes + 16 * ((we >> 20) & 63));
                         // W entries subtract conj(G) b in the even sector, C entries add conj(G) c
-                        const double s = (int)((we >> 26) & 1) == sec ? -1.0 : 1.0;
-                        const double bx = s * v.z, by = s * v.w;
+                        const long long neg = (int)((we >> 26) & 1) == sec ? (long long)(1ull << 63) : 0ll;   // off the FP64 pipe
+                        const double bx = __longlong_as_double(__double_as_longlong(v.z) ^ neg);
+                        const double by = __longlong_as_double(__double_as_longlong(v.w) ^ neg);
                         y.x = fma(G.x, v.x + bx, G.y * (by - v.y));
                         y.y = fma(G.x, v.y + by, G.y * (v.x - bx));
                     }
@@ -242,7 +257,7 @@ __global__ void __launch_bounds__(OZ_T, 1)
                         tc::bulk_g2s(smraw + sl * OZ_SLOT, X + (size_t)s * OZ_A, OZ_A, &full[sl]);
                         tc::bulk_g2s(smraw + sl * OZ_SLOT + OZ_A, tile + (size_t)s * bb, bb, &full[sl]);
                     }
-                } else if (warp == 1 && lane == 0) {
+                } else if (warp == 1 && tc::elect_one()) {
                     const uint32_t idesc = tc::idesc_bf16(128, N);
                     const uint64_t pa = 4096 >> 4, pb = (uint32_t)(N * 32) >> 4;
                     for (int s = 0; s < nk; ++s) {
@@ -284,8 +299,7 @@ __global__ void __launch_bounds__(OZ_T, 1)
                             auto a = [&](int d) { return __float2int_rn(__uint_as_float(v[d][i])); };
                             const long long hi = (((long long)a(0) << 16) + ((long long)a(1) << 8) + a(2)) * 256 + a(3);
                             const long long lo = (((long long)a(4) << 16) + ((long long)a(5) << 8) + a(6)) * 256 + a(7);
-                            const double c1 = rs[r];                    // 2^(row exponent - 38)
-                            const double y = c1 * ((double)hi + 0x1p-32 * (double)lo);
+                            const double y = oz_value(hi, lo, rs[r]);
                             ((double *)(Y + (size_t)(row >> 1) * sp.rows + (sec ? sp.D[0] : 0) + r))[row & 1] = y;
                         }
                     }

@@ -13,10 +13,9 @@
 // (the tensor core truncates small addends against a large accumulator).
 //
 // Blocks of up to 192 padded rows (p <= 10) take one tile, larger ones two, so that the
-// accumulators leave tensor memory for the X ring.  An MMA into the accumulator of the
-// one before it waits for it (measured: 108 cycles per MMA whatever N from 112 to 176,
-// against N / 2 of arithmetic), so the five small products alternate between two
-// accumulators where three fit (N <= 128, p <= 8).
+// accumulators leave tensor memory for the X ring.  The five small products alternate
+// between two accumulators where three fit (N <= 128, p <= 8), so that fewer MMAs follow one
+// into the same accumulator.
 // Roles (864 threads, one CTA per SM):
 //   warps 0-7   X producers, two groups of four warps (one per tensor-memory lane
 //               quadrant), group g writing K-step g of every chunk: the two coefficients of
@@ -259,7 +258,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
         }
     } else if (warp == SC_WMMA) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0) {
+        if (tc::elect_one()) {
             // descriptor of ring slot 0; the address field counts 16-byte units
             const uint64_t dring0 = tc::sdesc(tc::smem_u32(smraw), 128, 256);
             const uint64_t d_slot = sp.slot >> 4;

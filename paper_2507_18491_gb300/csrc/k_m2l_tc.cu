@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(V2_THREADS, 1)
         }
     } else if (warp == V2_WMMA) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0) {
+        if (tc::elect_one()) {
             const uint32_t idesc = tc::idesc_bf16(128, NR);
             // descriptor of ring slot 0; the address field counts 16-byte units,
             // so slot, K-step and lo-plane offsets add to it directly

@@ -52,6 +52,16 @@ __device__ __forceinline__ void mma_f16_ta(uint32_t dtmem, uint32_t atmem, uint6
         "r"(atmem), "l"(db), "r"(idesc), "r"(accumulate));
 }
 
+// true in one lane of the (converged) warp.  The operands of tcgen05.mma are warp-uniform
+// registers: behind elect.sync the compiler knows that one thread runs and moves them there
+// directly; behind `lane == 0` it has to allow for several.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t *dst_smem, uint32_t ncols)
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
