@@ -38,6 +38,8 @@ sys.path.insert(0, ROOT)
 SM_COUNT, SM_MHZ = 152, 2070.0
 FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MHZ * 1e6 / 1e12
 FP64_PEAK_TFLOPS = SM_COUNT * 2 * 2 * SM_MHZ * 1e6 / 1e12
+# DRAM bytes of k_m2l_sec over its matrix image (profiles/)
+TRAFFIC_RATIO = 1.08
 # dense TF32 tensor peak: the measured bf16 burst peak times the nominal
 # TF32 / bf16 ratio (1.1 / 2.25 PFLOP/s); fallback 1.9 PFLOP/s bf16
 TF32_PER_BF16 = 1.1 / 2.25
@@ -337,20 +339,23 @@ def main():
         lmfmm.matvec_host(op.ctx, Jh, Ph)
     e2e_ms = allmax((time.time() - t1) * 1e3 / args.steps, ws)
     P = (p + 1) ** 2
-    flops = 8.0 * P * P * st["m2l_columns"]
+    # the sector kernels (FP64 form, mixed form on the tensor cores) need 36 P^2 flops per box pair,
+    # the five-table ones 8 P^2 per helical column (nine columns per pair)
+    sector = st["m2l_kernel"] in (0, 3)
+    flops = (4.0 if sector else 8.0) * P * P * st["m2l_columns"]
     m2l_s = float(np.mean(m2l_ms)) * 1e-3
     achieved = flops / m2l_s / 1e12
-    kern = {0: "k_m2l<double>", 1: "k_m2l<float>", 2: "k_m2l_tc", 3: "k_m2l_tc2"}[st["m2l_kernel"]]
-    # DRAM bytes per launch of k_m2l_tc2: the table image times the read + write / image
-    # ratio of an ncu capture of the same kernel (dram__bytes_read.sum 2.780 GB +
-    # dram__bytes_write.sum 0.042 GB for a 2.622 GB image, three-layer N = 8192,
+    kern = {0: "k_m2l_oz", 1: "k_m2l<float>", 2: "k_m2l_tc", 3: "k_m2l_sec"}[st["m2l_kernel"]]
+    # DRAM bytes per launch of k_m2l_sec: the matrix image times the read + write / image
+    # ratio of an ncu capture of the same kernel (TRAFFIC_RATIO, three-layer N = 8192,
     # p = 12, depth 4, theta 0.55).  The image, read once per launch, is most of it; the
-    # multipole expansions fit in L2 in that case but not at N = 2^20 (152 MB), so the
+    # multipole expansions fit in L2 in that case but not at N = 2^20, so the
     # scaled figure is a lower bound there.  Other kernels: not captured
-    traffic = st["bytes_tables"] * (2.8226 / 2.6224) if st["m2l_kernel"] == 3 else None
-    bound = "tensor" if st["m2l_kernel"] >= 2 else "alu"
+    traffic = st["bytes_tables"] * TRAFFIC_RATIO if st["m2l_kernel"] == 3 else None
+    bound = "alu" if st["m2l_kernel"] == 1 else "tensor"
     if prec == lmfmm.FP64:
-        peak, peak_src = FP64_PEAK_TFLOPS, "derived (not measured) FP64 ALU: 152 SM x 2 FMA/clk x 2 x 2070 MHz"
+        peak, peak_src = tensor_peak(tf32=False)
+        peak, peak_src = peak / 36, peak_src + " / 36 digit products of an FP64 one"
     elif bound == "tensor":
         peak, peak_src = tensor_peak(tf32=st["m2l_kernel"] == 2)
     else:
@@ -387,9 +392,11 @@ def main():
         "roofline": {"kernel": kern, "bound": bound, "achieved": achieved,
                      "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
                      "peak_source": peak_src, "flops_per_launch": flops,
-                     "flops_definition": "algorithmic: 8 P^2 real flops per M2L column (complex P x P "
-                                         "product); the tensor path executes more: 6 bf16 products of "
-                                         "three-piece splits (k_m2l_tc2) or 3 TF32 terms (k_m2l_tc)"},
+                     "flops_definition": "algorithmic: 36 P^2 real flops per box pair (two mirror sectors "
+                                         "of 3P/2) in k_m2l_sec and k_m2l_oz, 8 P^2 per helical column in "
+                                         "the five-table kernels; the tensor path executes more: 6 bf16 "
+                                         "products of three-piece splits (k_m2l_sec), 36 of digits "
+                                         "(k_m2l_oz) or 3 TF32 terms (k_m2l_tc)"},
     }
     if rank == 0 and not args.no_cpu:
         acc = accuracy(op, w, cdt)

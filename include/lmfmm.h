@@ -107,11 +107,12 @@ typedef struct {
     int64_t n_near_pairs;  /* near box pairs */
     int64_t n_near_point_pairs;
     int64_t n_quad_nodes;  /* k_rho nodes summed over all tabulated geometries */
-    double bytes_tables;   /* device bytes held by M2L tables (or their tiled tensor-core image) */
+    double bytes_tables;   /* device bytes held by M2L tables (or their tiled tensor-core images) */
     double ms_setup;       /* wall time of the last lmfmm_build */
     double ms_stage[8];    /* last matvec: P2M, M2M, M2L, L2L, L2P, S2T, permute, total */
     int64_t m2l_columns;   /* helical columns pushed through M2L tables per matvec */
-    int m2l_kernel;        /* M2L product of the built form: 0 FP64 SIMT, 1 FP32 SIMT,
+    int m2l_kernel;        /* M2L product of the built form: 0 FP64 (tcgen05 on base-256 digits;
+                              SIMT where its images do not fit in memory), 1 FP32 SIMT,
                               2 tcgen05 streamed-operand kernel, 3 tcgen05 persistent kernel */
     int launches;          /* kernels launched by the last matvec */
     int64_t n_geometries_same_layer;  /* of n_geometries: components with l = l' (their tables
