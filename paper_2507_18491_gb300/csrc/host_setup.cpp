@@ -9,6 +9,7 @@
 #include <map>
 #include <numeric>
 #include <tuple>
+#include <system_error>
 #include <thread>
 #include <unordered_map>
 
@@ -541,21 +542,34 @@ void chebyshev_tables(lmfmm_ctx *ctx)
     ctx->LMAXC = p + 2;
     const int LM = ctx->LMAXC, KM = ctx->KMAX;
     std::map<std::pair<int, int>, int> seen;
+    std::vector<std::pair<int, int>> keys;
     ctx->comp_gidx.assign(ctx->comps.size(), 0);
-    ctx->Gten.clear();
     for (size_t ci = 0; ci < ctx->comps.size(); ++ci) {
-        int l = ctx->comps[ci].l, lp = ctx->comps[ci].lp;
-        auto key = std::make_pair(l, lp);
-        auto it = seen.find(key);
-        if (it != seen.end()) { ctx->comp_gidx[ci] = it->second; continue; }
-        int gi = (int)seen.size();
-        seen[key] = gi;
-        ctx->comp_gidx[ci] = gi;
-        size_t base = ctx->Gten.size();
-        ctx->Gten.resize(base + (size_t)T * T * LM, cd{0, 0});
-        gtensor(p, ctx->Bcoef, KM, zc(ctx->med.k[l].x, ctx->med.k[l].y),
-                zc(ctx->med.k[lp].x, ctx->med.k[lp].y), &ctx->Gten[base]);
+        const auto key = std::make_pair(ctx->comps[ci].l, ctx->comps[ci].lp);
+        const auto it = seen.emplace(key, (int)keys.size());
+        if (it.second) keys.push_back(key);
+        ctx->comp_gidx[ci] = it.first->second;
     }
+    const size_t one = (size_t)T * T * LM;
+    ctx->Gten.assign(keys.size() * one, cd{0, 0});
+    // one thread per (source layer, target layer): long double arithmetic, which is software on
+    // the Arm host (60 ms per tensor at p = 12)
+    const size_t nth = std::max(1u, std::min(32u, std::thread::hardware_concurrency()));
+    std::vector<std::thread> pool;
+    auto share = [&](size_t w) {
+        for (size_t i = w; i < keys.size(); i += nth) {
+            const cd k = ctx->med.k[keys[i].first], kp = ctx->med.k[keys[i].second];
+            gtensor(p, ctx->Bcoef, KM, zc(k.x, k.y), zc(kp.x, kp.y), &ctx->Gten[i * one]);
+        }
+    };
+    for (size_t w = 0; w < std::min(nth, keys.size()); ++w) {
+        try {
+            pool.emplace_back(share, w);
+        } catch (const std::system_error &) {   // no more threads to be had
+            share(w);
+        }
+    }
+    for (auto &t : pool) t.join();
 }
 
 }  // namespace lmf
