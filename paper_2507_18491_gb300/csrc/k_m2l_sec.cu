@@ -26,9 +26,8 @@
 //               pairs at p = 7); then one phase per input, the split into three pieces (the
 //               two rows of a pair share them) and the store into the tensor-memory ring;
 //   warps 8-23  epilogue: accumulators -> a per-CTA scratch in global memory (L2-resident)
-//               as four-row groups, 16 bytes per real column, so that every store
-//               instruction writes 512 contiguous bytes and tensor memory is free again at
-//               once; after the item's last tile one warp per pair combines the two
+//               ([pair][row], through a tile in shared memory), so that tensor memory is free
+//               again at once; after the item's last tile one warp per pair combines the two
 //               sectors, applies the output phases into a shared staging row [3][P] and
 //               adds it to the pair's local expansions with one bulk reduction;
 //   warp 24     one bulk copy per matrix chunk into a shared-memory ring;
@@ -63,6 +62,8 @@ constexpr uint32_t SC_XROW = 144;  // bytes of a pair's K-step there: 8 inputs o
 constexpr uint32_t SC_XST = 16 * SC_XROW;
 constexpr int SC_PT = 256, SC_ET = 512;     // producer, epilogue threads
 constexpr int SC_EW = SC_ET / 32;
+constexpr int SC_DS = 34;          // row stride (words) of an epilogue warp's 16-row drain tile
+constexpr uint32_t SC_TILE = 16 * SC_DS * 4;
 constexpr int SC_WTMA = (SC_PT + SC_ET) / 32, SC_WMMA = SC_WTMA + 1, SC_WMETA = SC_WTMA + 2;
 constexpr int SC_THREADS = (SC_WMETA + 1) * 32;
 constexpr int SC_PMAX = 12;
@@ -123,13 +124,15 @@ SecPlan sec_plan(int p)
     s.ews = s.D0 <= 128 ? SC_EW : SC_EW / 2;   // epilogue warps that scatter: their staging rows take shared memory
     const uint32_t bars = (2 * SC_ST_MAX + 2 * SC_SX_MAX + 12) * 8 + 16;
     const uint32_t ent = (uint32_t)s.nchunk0 * SC_KC * 4;
-    const uint32_t fixed = 2 * s.meta_bytes + ent + SC_PT / 32 * SC_XD * SC_XST + s.ews * s.stage_bytes + bars;
+    // staging rows of the scatter; the drain tiles of all epilogue warps lie there too
+    const uint32_t stages = std::max(s.ews * s.stage_bytes, (uint32_t)SC_EW * SC_TILE);
+    const uint32_t fixed = 2 * s.meta_bytes + ent + SC_PT / 32 * SC_XD * SC_XST + stages + bars;
     s.ST = (int)std::min<uint32_t>(SC_ST_MAX, (SC_SMEM_MAX - fixed) / s.slot);
     s.o_meta = s.ST * s.slot;
     s.o_ent = s.o_meta + 2 * s.meta_bytes;
     s.o_xsrc = s.o_ent + ent;
     s.o_stage = s.o_xsrc + SC_PT / 32 * SC_XD * SC_XST;
-    s.o_bars = s.o_stage + s.ews * s.stage_bytes;
+    s.o_bars = s.o_stage + stages;
     s.smem = s.o_bars + bars;
     return s;
 }
@@ -174,7 +177,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
     auto meta_pair = [&](int slot) { return (const M2LPair *)(meta_ph(slot) + SC_BN * sp.ph_bytes); };
     auto prob = [&](const M2LWork &w) { return probs ? probs[w.prob] : one; };
 
-    float *Y = yscr + (size_t)blockIdx.x * sp.yrows * 128;   // [row / 4][real column][row % 4]
+    float2 *Y = (float2 *)(yscr + (size_t)blockIdx.x * sp.yrows * 128);   // [pair][row]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (warp == 0) tc::tmem_alloc(tslot, 512);
@@ -466,7 +469,7 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
         for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x, ++li) {
             const M2LWork w = work[it];
             const int slot = li & 1;
-            // the previous item's scatter has read the scratch
+            // the previous item's scatter has read the scratch, and its reductions the staging rows
             bool ok = li == 0 || tc::mbar_wait(yfree, (li - 1) & 1, SC_POLLS);
             if (__any_sync(0xffffffffu, !ok)) {
                 failed = true;
@@ -480,7 +483,12 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
                 }
                 tc::fence_after();
                 const int N = sp.t[t].N;
-                float4 *Yt = (float4 *)Y + (size_t)(sp.t[t].y0 >> 2) * 128 + 32 * q4 + lane;
+                // a 16-row slab of the warp's 16 pairs goes through its tile, so that a store
+                // instruction writes four whole 128-byte lines (lane: pair 4h + lane / 8, rows
+                // 2 (lane % 8), + 1) and the scatter reads whole lines
+                float *T = (float *)(smraw + sp.o_stage + ew * SC_TILE);
+                const int lr = 2 * (lane & 7), lc = lane >> 3;
+                float4 *Yt = (float4 *)(Y + (size_t)(16 * q4) * sp.yrows + sp.t[t].y0);
                 for (int c0 = 16 * part; c0 < N; c0 += SC_ET / 8) {   // N is a multiple of 16
                     uint32_t va[16], vb[16];
                     tc::tmem_ld16(lane_base + sp.nmax + c0, va);
@@ -494,14 +502,16 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
                     tc::tmem_ld16(lane_base + c0, vb);
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        float4 o;
-                        o.x = __uint_as_float(va[4 * i]) + __uint_as_float(vb[4 * i]);
-                        o.y = __uint_as_float(va[4 * i + 1]) + __uint_as_float(vb[4 * i + 1]);
-                        o.z = __uint_as_float(va[4 * i + 2]) + __uint_as_float(vb[4 * i + 2]);
-                        o.w = __uint_as_float(va[4 * i + 3]) + __uint_as_float(vb[4 * i + 3]);
-                        Yt[(size_t)((c0 >> 2) + i) * 128] = o;
+                    for (int i = 0; i < 16; ++i) T[i * SC_DS + lane] = __uint_as_float(va[i]) + __uint_as_float(vb[i]);
+                    __syncwarp();
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int cl = 4 * h + lc;
+                        const float2 x0 = *(const float2 *)(T + lr * SC_DS + 2 * cl);
+                        const float2 x1 = *(const float2 *)(T + (lr + 1) * SC_DS + 2 * cl);
+                        Yt[((size_t)cl * sp.yrows + c0 + lr) >> 1] = make_float4(x0.x, x0.y, x1.x, x1.y);
                     }
+                    __syncwarp();
                 }
                 tc::fence_before();
                 tc::mbar_arrive(accempty);
@@ -521,10 +531,8 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
 #pragma unroll
                     for (int i = 0; i < RB; ++i) {
                         const int r = min(lane + 32 * (i0 + i), sp.D0 - 1), ro = yodd + min(r, sp.D1 - 1);
-                        const float *a = Y + (size_t)(r >> 2) * 512 + 8 * c + (r & 3);
-                        const float *b = Y + (size_t)(ro >> 2) * 512 + 8 * c + (ro & 3);
-                        ye[i] = float2{a[0], a[4]};
-                        yo[i] = float2{b[0], b[4]};
+                        ye[i] = Y[(size_t)c * sp.yrows + r];
+                        yo[i] = Y[(size_t)c * sp.yrows + ro];
                     }
                 };
                 float2 ye[RB], yo[RB];
@@ -573,8 +581,9 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
                     atomicAdd((float2 *)dst + head + body, sg[head + body]);
                 }
             }
-            tc::mbar_arrive(yfree);
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
             __syncwarp();
+            tc::mbar_arrive(yfree);
             if (lane == 0) tc::mbar_arrive(&metaempty[slot]);
         }
         asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // every reduction has landed
