@@ -39,7 +39,7 @@ SM_COUNT, SM_MHZ = 152, 2070.0
 FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MHZ * 1e6 / 1e12
 FP64_PEAK_TFLOPS = SM_COUNT * 2 * 2 * SM_MHZ * 1e6 / 1e12
 # DRAM bytes of k_m2l_sec over its matrix image (profiles/)
-TRAFFIC_RATIO = 1.08
+TRAFFIC_RATIO = 1.904
 # dense TF32 tensor peak: the measured bf16 burst peak times the nominal
 # TF32 / bf16 ratio (1.1 / 2.25 PFLOP/s); fallback 1.9 PFLOP/s bf16
 TF32_PER_BF16 = 1.1 / 2.25
@@ -348,9 +348,9 @@ def main():
     kern = {0: "k_m2l_oz", 1: "k_m2l<float>", 2: "k_m2l_tc", 3: "k_m2l_sec"}[st["m2l_kernel"]]
     # DRAM bytes per launch of k_m2l_sec: the matrix image times the read + write / image
     # ratio of an ncu capture of the same kernel (TRAFFIC_RATIO, three-layer N = 8192,
-    # p = 12, depth 4, theta 0.55).  The image, read once per launch, is most of it; the
+    # p = 12, depth 4, theta 0.55: the image once and the accumulator scratch leaving L2).  The
     # multipole expansions fit in L2 in that case but not at N = 2^20, so the
-    # scaled figure is a lower bound there.  Other kernels: not captured
+    # scaled figure is an estimate there.  Other kernels: not captured
     traffic = st["bytes_tables"] * TRAFFIC_RATIO if st["m2l_kernel"] == 3 else None
     bound = "alu" if st["m2l_kernel"] == 1 else "tensor"
     if prec == lmfmm.FP64:
