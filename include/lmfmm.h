@@ -336,7 +336,7 @@ lmfmm_status lmfmm_get_stats(const lmfmm_ctx *ctx, lmfmm_stats *out);
  * lmfmm_params), the distinct M2L geometries and their pair lists, the
  * free-space lists when params->components asks for them (Section 2), the
  * M2M / L2L translation groups and the 64-column M2L work items of the
- * persistent tensor-core kernel.  Checks:
+ * five-table kernels (the sector kernels cut the same pairs into runs of at most 64).  Checks:
  *   tree       every layer's points are partitioned by the boxes of each level,
  *              children partition their parent, every point lies in its leaf's
  *              cell, box radii bound their points;

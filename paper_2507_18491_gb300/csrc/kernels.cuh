@@ -59,7 +59,7 @@ struct GemmWork {       // M2M / L2L: pairs [pair0, pair0 + npair) of one transl
     int64_t pair0;
 };
 
-struct M2LWork {        // one M2L table applied to a chunk of pairs of one geometry
+struct M2LWork {        // one M2L table, or both sector blocks, applied to a chunk of pairs of one geometry
     int geom, t, npair;
     int flags;          // bit 0: odd input degrees change sign, bit 1: odd output degrees
     int64_t pair0;
