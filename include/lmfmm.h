@@ -214,15 +214,22 @@ lmfmm_status lmfmm_gradient(lmfmm_ctx *ctx, const void *J, const void *g, int dt
                             void *stream);
 
 /* Waits for `stream` and reads the context's device status word, which every
- * matvec clears (stream-ordered) before its first kernel.  Returns LMFMM_OK,
- * LMFMM_ERR_TIMEOUT if a bounded wait inside a tensor-core kernel of the
- * matvecs since then gave up (that result is incomplete), or LMFMM_ERR_CUDA. */
+ * matvec, transpose, adjoint and gradient call clears (stream-ordered) before its
+ * first kernel.  Returns LMFMM_OK, LMFMM_ERR_TIMEOUT if a bounded wait inside a
+ * tensor-core kernel of the last such call gave up, in either pass of a
+ * gradient (that result is incomplete), or LMFMM_ERR_CUDA. */
 lmfmm_status lmfmm_check(lmfmm_ctx *ctx, void *stream);
 
 /* Test hook for the error path above: ORs `bits` into the device status word
  * from the host (synchronous), as a tensor-core wait that gives up would.
  * Bit 4 is the only meaning defined today.  Requires lmfmm_build. */
 lmfmm_status lmfmm_test_set_status(lmfmm_ctx *ctx, int bits);
+
+/* Test hook: the next forward pass (a matvec or the first pass of a gradient;
+ * not a batch's merged M2L) leaves `bits` (0..255) in the status word after its
+ * M2L, in stream order, as if a wait of that M2L had given up.  Requires
+ * lmfmm_build. */
+lmfmm_status lmfmm_test_fail_m2l(lmfmm_ctx *ctx, int bits);
 
 /* Direct evaluation of the same operator over ALL point pairs with the
  * device near-field kernel (Sommerfeld integral per pair, Section 3.5);

@@ -66,6 +66,7 @@ struct DevState {
     cd *le_ck = nullptr, *qh_ck = nullptr, *gfield = nullptr, *s2tg = nullptr;
     int *flag = nullptr;
     int *mvstatus = nullptr;         // matvec status word (bit 4: tensor-core wait gave up)
+    int fail_m2l = 0;                // test hook: status bits the next forward M2L leaves
     int m2l_kernel = 0;              // 0 FP64 SIMT, 1 FP32 SIMT, 2 tcgen05 streamed, 3 tcgen05 persistent
     cf *ephase = nullptr;            // sector kernel: phases G[d] per pair
     void *mepk = nullptr;            // ... and the packed multipole expansions it reads
@@ -163,9 +164,9 @@ lmfmm_status check_flag(lmfmm_ctx *ctx)
     return LMFMM_OK;
 }
 
-// Status word of the matvec kernels, cleared by every matvec before its first
-// kernel: a tensor-core wait that gave up leaves bit 4.  Reads it after the
-// stream's work is done.
+// Status word of the matvec kernels, cleared by every call before its first
+// kernel (a gradient is one call of two passes): a tensor-core wait that gave up
+// leaves bit 4.  Reads it after the stream's work is done.
 lmfmm_status check_mvstatus(lmfmm_ctx *ctx, cudaStream_t st)
 {
     int f = 0;
@@ -999,6 +1000,10 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
         launch_m2l_t<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
                         (const cx<T> *)d->tab, me, le, st);
     }
+    if (own_m2l && d->fail_m2l) {
+        CK(cudaMemsetAsync(d->mvstatus, d->fail_m2l, 1, st));
+        d->fail_m2l = 0;
+    }
     CK(cudaEventRecord(d->ev[3], st));
     }
     if (parts & MV_DOWN) {
@@ -1040,9 +1045,11 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
 // the point values against L2P's functions (P2M's kernel), L2L^T and M2M^T run
 // the transposed matrices up and down the tree, M2L^T applies the transposed
 // tables, P2M^T evaluates with P2M's functions (L2P's kernel).  With cj the
-// input and output are conjugated: conj(A^T conj y) = A^H y.
+// input and output are conjugated: conj(A^T conj y) = A^H y.  first: the call's
+// first pass, which clears the status word (a later one keeps what an earlier left).
 template <typename T>
-static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *out, cudaStream_t st, bool cj)
+static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *out, cudaStream_t st, bool cj,
+                                bool first = true)
 {
     DevState *d = DS(ctx);
     const int p = ctx->prm.p, P = (p + 1) * (p + 1);
@@ -1051,7 +1058,7 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     const cx<T> *tupT = (const cx<T> *)d->tupT, *tdnT = (const cx<T> *)d->tdnT;
     int nl = 0;
     CK(cudaEventRecord(d->ev[0], st));
-    CK(cudaMemsetAsync(d->mvstatus, 0, sizeof(int), st));
+    if (first) CK(cudaMemsetAsync(d->mvstatus, 0, sizeof(int), st));
     launch_gather_tr(N, d->perm, y, dtype, d->ph, cj, st);   // ph <- S^T y
     CK(cudaMemsetAsync(le, 0, (size_t)nbox * 3 * P * sizeof(cx<T>), st));
     leaf_p2m<T>(ctx, d->ph, le, true, st);
@@ -1212,7 +1219,7 @@ lmfmm_status lmfmm_gradient(lmfmm_ctx *ctx, const void *J, const void *g, int dt
     CK(cudaMemcpyAsync(d->le_ck, d->le, (size_t)nbox * 3 * P * sizeof(cd), cudaMemcpyDeviceToDevice, st));
     CK(cudaMemcpyAsync(d->qh_ck, d->qh, (size_t)N * 3 * sizeof(cd), cudaMemcpyDeviceToDevice, st));
     // transposed pass of conj(g): gJ = A^H g; leaves ph = S^T conj(g), me = its multipole expansions
-    TRY(matvec_tr_t<double>(ctx, g, dtype, gJ ? gJ : (void *)d->gfield, st, true));
+    TRY(matvec_tr_t<double>(ctx, g, dtype, gJ ? gJ : (void *)d->gfield, st, true, false));
     if (gxyz) {
         CK(cudaMemsetAsync(gxyz, 0, (size_t)N * 3 * sizeof(double), st));
         launch_grad_leaf(p, N, d->nleaves, d->leaves, d->boxes, d->xyz, d->perm, d->le_ck, (const cd *)d->me,
@@ -1535,6 +1542,17 @@ lmfmm_status lmfmm_test_set_status(lmfmm_ctx *ctx, int bits)
     CK(cudaMemcpy(&f, DS(ctx)->mvstatus, sizeof(int), cudaMemcpyDeviceToHost));
     f |= bits;
     CK(cudaMemcpy(DS(ctx)->mvstatus, &f, sizeof(int), cudaMemcpyHostToDevice));
+    return LMFMM_OK;
+}
+
+lmfmm_status lmfmm_test_fail_m2l(lmfmm_ctx *ctx, int bits)
+{
+    if (!ctx || bits < 0 || bits > 255) return LMFMM_ERR_ARG;
+    if (!ctx->built || !DS(ctx)) {
+        ctx->err = "test_fail_m2l: call lmfmm_build first";
+        return LMFMM_ERR_STATE;
+    }
+    DS(ctx)->fail_m2l = bits;
     return LMFMM_OK;
 }
 

@@ -67,7 +67,8 @@ class PlanInfo(ctypes.Structure):
 
 EXPORTS = ["lmfmm_default_params", "lmfmm_create", "lmfmm_set_layers", "lmfmm_set_points",
            "lmfmm_set_points_device", "lmfmm_build", "lmfmm_matvec", "lmfmm_matvec_host",
-           "lmfmm_matvec_adjoint", "lmfmm_matvec_transpose", "lmfmm_gradient", "lmfmm_check", "lmfmm_test_set_status", "lmfmm_direct",
+           "lmfmm_matvec_adjoint", "lmfmm_matvec_transpose", "lmfmm_gradient", "lmfmm_check", "lmfmm_test_set_status", "lmfmm_test_fail_m2l",
+           "lmfmm_direct",
            "lmfmm_direct_noalloc", "lmfmm_densities", "lmfmm_m2l_table", "lmfmm_translation_matrix",
            "lmfmm_free_m2l_table", "lmfmm_legendre_chebyshev", "lmfmm_legendre_product",
            "lmfmm_get_stats", "lmfmm_plan_check", "lmfmm_plan_depth", "lmfmm_last_error", "lmfmm_destroy", "lmfmm_batch_create",
@@ -110,6 +111,7 @@ def load():
         "lmfmm_gradient": [P, P, P, i, P, P, P],
         "lmfmm_check": [P, P],
         "lmfmm_test_set_status": [P, i],
+        "lmfmm_test_fail_m2l": [P, i],
         "lmfmm_direct": [P, P, P, P],
         "lmfmm_direct_noalloc": [P, P, P, P],
         "lmfmm_densities": [P, i, i, i64, P, P, P],
@@ -262,6 +264,10 @@ def check(ctx, stream=None):
 
 def test_set_status(ctx, bits):
     _check(load().lmfmm_test_set_status(ctx, int(bits)), ctx)
+
+
+def test_fail_m2l(ctx, bits):
+    _check(load().lmfmm_test_fail_m2l(ctx, int(bits)), ctx)
 
 
 def matvec_host(ctx, J: np.ndarray, Phi: np.ndarray, stream=None):
