@@ -134,12 +134,22 @@ void dfree(lmfmm_ctx *ctx, void *p)
     }
 }
 
+// Host to device on the stream of the kernels that read the copy, complete on return.  A plain
+// cudaMemcpy from pageable memory runs on the legacy stream and may return before its last
+// transfer has landed, and a non-blocking stream does not wait for that one.
+cudaError_t copy_in(void *dst, const void *src, size_t bytes, cudaStream_t st)
+{
+    if (bytes == 0) return cudaSuccess;
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(st);
+}
+
 template <typename T>
-lmfmm_status dupload(lmfmm_ctx *ctx, T **p, const std::vector<T> &h)
+lmfmm_status dupload(lmfmm_ctx *ctx, cudaStream_t st, T **p, const std::vector<T> &h)
 {
     lmfmm_status s = dalloc(ctx, p, h.size());
     if (s) return s;
-    if (!h.empty()) CK(cudaMemcpy(*p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice));
+    CK(copy_in(*p, h.data(), h.size() * sizeof(T), st));
     return LMFMM_OK;
 }
 
@@ -278,9 +288,7 @@ lmfmm_status tabulate(lmfmm_ctx *ctx, std::vector<GeomDev> &hg, const CompDev *d
     }
     scr = (cd *)qs;
     lmfmm_status rc = LMFMM_OK;
-    if (!hg.empty() &&
-        cudaMemcpy(dgeo, hg.data(), hg.size() * sizeof(GeomDev), cudaMemcpyHostToDevice))
-        rc = LMFMM_ERR_CUDA;
+    if (copy_in(dgeo, hg.data(), hg.size() * sizeof(GeomDev), st)) rc = LMFMM_ERR_CUDA;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     const bool timed = ms && cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
     if (timed) cudaEventRecord(e0, st);
@@ -507,15 +515,15 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     }
     CK(cudaMalloc((void **)&d->flag, sizeof(int)));
     d->allocs.push_back(d->flag);
-    CK(cudaMemset(d->flag, 0, sizeof(int)));
+    CK(cudaMemsetAsync(d->flag, 0, sizeof(int), st));
     CK(cudaMalloc((void **)&d->mvstatus, sizeof(int)));
     d->allocs.push_back(d->mvstatus);
-    CK(cudaMemset(d->mvstatus, 0, sizeof(int)));
+    CK(cudaMemsetAsync(d->mvstatus, 0, sizeof(int), st));
     for (auto &e : d->ev) CK(cudaEventCreate(&e));
     d->ev_ok = true;
     // points and boxes
-    TRY(dupload(ctx, &d->xyz, ctx->sxyz));
-    TRY(dupload(ctx, &d->perm, ctx->perm));
+    TRY(dupload(ctx, st, &d->xyz, ctx->sxyz));
+    TRY(dupload(ctx, st, &d->perm, ctx->perm));
     std::vector<BoxDev> hb(nbox);
     std::vector<int64_t> leaves;
     for (int64_t i = 0; i < nbox; ++i) {
@@ -523,8 +531,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         hb[i] = BoxDev{b.p0, b.p1, {b.c[0], b.c[1], b.c[2]}, b.layer, 0};
         if (b.level == ctx->depth) leaves.push_back(i);
     }
-    TRY(dupload(ctx, &d->boxes, hb));
-    TRY(dupload(ctx, &d->leaves, leaves));
+    TRY(dupload(ctx, st, &d->boxes, hb));
+    TRY(dupload(ctx, st, &d->leaves, leaves));
     d->nleaves = (int64_t)leaves.size();
     if (ctx->prm.precision == LMFMM_MIXED && leaf_fast_supported(p)) {
         std::vector<int> ptb(N > 0 ? N : 1, 0);
@@ -538,8 +546,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         // largest units first, so that the last wave is made of small ones
         std::stable_sort(units.begin(), units.end(),
                          [](const LeafUnit &a, const LeafUnit &b) { return a.i1 - a.i0 > b.i1 - b.i0; });
-        TRY(dupload(ctx, &d->pt_box, ptb));
-        TRY(dupload(ctx, &d->units, units));
+        TRY(dupload(ctx, st, &d->pt_box, ptb));
+        TRY(dupload(ctx, st, &d->units, units));
         d->nunits = (int64_t)units.size();
         // k_p2m_ms takes a time per point, k_p2m_pt one per unit (two layers at depth 5, 7.5 / 30 / 60 /
         // 120 points per unit: p = 6 45 / 84 / 143 / 239 against 65 / 74 / 86 / 127 us, p = 8 53 / 98 /
@@ -567,11 +575,11 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     auto lev_size = [&](int lev) { return Sroot / (double)(1u << lev); };
     auto kabs = [&](int layer) { return std::hypot(ctx->med.k[layer].x, ctx->med.k[layer].y); };
     for (int j = 0; j <= ctx->med.L; ++j) d->lscale.s[j] = kabs(j) * lev_size(ctx->depth);
-    TRY(dupload(ctx, &d->comps, ctx->comps));
+    TRY(dupload(ctx, st, &d->comps, ctx->comps));
     cd *dG = nullptr;
     int *dcg = nullptr;
-    TRY(dupload(ctx, &dG, ctx->Gten));
-    TRY(dupload(ctx, &dcg, ctx->comp_gidx));
+    TRY(dupload(ctx, st, &dG, ctx->Gten));
+    TRY(dupload(ctx, st, &dcg, ctx->comp_gidx));
     // M2L geometries, tables and work items
     const double a = medium_a(ctx->med);
     std::vector<GeomDev> hg(ctx->geoms.size());
@@ -620,9 +628,9 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             TRY(tabulate(ctx, hr, d->comps, dG, dcg, tab64, st, &ms_tab));
         }
         if (!ctx->free_tables.empty())
-            CK(cudaMemcpy(tab64 + ctx->n_react_geoms * (size_t)NTAB * P * P, ctx->free_tables.data(),
-                          ctx->free_tables.size() * sizeof(cd), cudaMemcpyHostToDevice));
-        TRY(dupload(ctx, &d->geoms, hg));
+            CK(copy_in(tab64 + ctx->n_react_geoms * (size_t)NTAB * P * P, ctx->free_tables.data(),
+                       ctx->free_tables.size() * sizeof(cd), st));
+        TRY(dupload(ctx, st, &d->geoms, hg));
         if (d->m2l_kernel == 3) {
             unsigned char *img = nullptr;
             TRY(dalloc(ctx, &img, m2l_sec_image_bytes(p, (int64_t)hg.size())));
@@ -663,7 +671,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             d->tab = tab64;
         }
     }
-    TRY(dupload(ctx, &d->m2l, ctx->m2l));
+    TRY(dupload(ctx, st, &d->m2l, ctx->m2l));
     std::vector<M2LWork> mw;
     const int64_t ncols = 9 * (int64_t)ctx->m2l.size();   // helical columns: nine table applications per pair
     if (d->m2l_kernel == 3) {
@@ -689,7 +697,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     } else {
         m2l_work_items(ctx, d->m2l_kernel == 2 ? m2l_tc_cols() : f32 ? gemm_cols<float>() : gemm_cols<double>(), 0, mw);
     }
-    TRY(dupload(ctx, &d->m2lwork, mw));
+    TRY(dupload(ctx, st, &d->m2lwork, mw));
     d->n_m2lwork = (int64_t)mw.size();
     // translation matrices (exact addition theorem), on the device from the groups' factors
     {
@@ -707,10 +715,10 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         double *dw = nullptr, *dP = nullptr, *dGt = nullptr, *dfac = nullptr;
         double2 *dsc = nullptr;
         cd *up64 = nullptr, *dn64 = nullptr;
-        TRY(dupload(ctx, &dw, gw));
-        TRY(dupload(ctx, &dP, gP));
-        TRY(dupload(ctx, &dfac, fac));
-        TRY(dupload(ctx, &dsc, scl));
+        TRY(dupload(ctx, st, &dw, gw));
+        TRY(dupload(ctx, st, &dP, gP));
+        TRY(dupload(ctx, st, &dfac, fac));
+        TRY(dupload(ctx, st, &dsc, scl));
         TRY(dalloc(ctx, &dGt, (size_t)P * P * (p + 1)));
         TRY(dalloc(ctx, &up64, (size_t)ngr * P * P));
         TRY(dalloc(ctx, &dn64, (size_t)ngr * P * P));
@@ -736,8 +744,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
                 (q == 0 ? d->tup : q == 1 ? d->tdn : q == 2 ? d->tupT : d->tdnT) = a1;
             }
         }
-        TRY(dupload(ctx, &d->tchild, ctx->tpair_child));
-        TRY(dupload(ctx, &d->tparent, ctx->tpair_parent));
+        TRY(dupload(ctx, st, &d->tchild, ctx->tpair_child));
+        TRY(dupload(ctx, st, &d->tparent, ctx->tpair_parent));
         if (d->trans_tc) {
             // M2M / L2L on the persistent tensor-core kernel: tiled bf16 three-piece
             // images of the scaled FP64 matrices, items of 21 pairs (63 helical columns)
@@ -766,7 +774,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
                 }
             }
             d->twork_off[ctx->depth + 1] = (int64_t)tw.size();
-            TRY(dupload(ctx, &d->twork, tw));
+            TRY(dupload(ctx, st, &d->twork, tw));
         }
         // work items per child level
         std::vector<GemmWork> gwk;
@@ -782,7 +790,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             }
         }
         d->gwork_off[ctx->depth + 1] = (int64_t)gwk.size();
-        TRY(dupload(ctx, &d->gwork, gwk));
+        TRY(dupload(ctx, st, &d->gwork, gwk));
         CK(cudaStreamSynchronize(st));
         for (void *q : {(void *)dw, (void *)dP, (void *)dGt, (void *)dfac, (void *)dsc}) dfree(ctx, q);
         if (f32) {
@@ -791,7 +799,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         }
     }
     // near field
-    TRY(dupload(ctx, &d->near, ctx->near));
+    TRY(dupload(ctx, st, &d->near, ctx->near));
     {
         // five Sommerfeld integrals per point pair, then the 8 combined coefficients
         cd *s2t5 = nullptr;
@@ -811,14 +819,14 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             for (int64_t s0 = 0; s0 < bs.p1 - bs.p0; s0 += S2T_SRC)
                 for (int64_t ii = 0; ii < bt.p1 - bt.p0; ++ii) sw.push_back(S2TRow{(int64_t)i, (int)ii, (int)s0});
         }
-        TRY(dupload(ctx, &d->s2twork, sw));
+        TRY(dupload(ctx, st, &d->s2twork, sw));
         d->n_s2twork = (int64_t)sw.size();
         std::vector<S2TRowT> swT;
         for (size_t i = 0; i < ctx->near.size(); ++i) {
             const Box &bs = ctx->boxes[ctx->near[i].src];
             for (int64_t jj = 0; jj < bs.p1 - bs.p0; ++jj) swT.push_back(S2TRowT{(int64_t)i, (int)jj, 0});
         }
-        TRY(dupload(ctx, &d->s2tworkT, swT));
+        TRY(dupload(ctx, st, &d->s2tworkT, swT));
         d->n_s2tworkT = (int64_t)swT.size();
         // free-space near field: the near leaves of a leaf, consecutive sorted points joined
         d->free_near = !ctx->free_near.empty();
@@ -826,7 +834,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             std::vector<int> fb(N, 0);
             for (int64_t li : leaves)
                 for (int64_t q = ctx->boxes[li].p0; q < ctx->boxes[li].p1; ++q) fb[q] = (int)li;
-            TRY(dupload(ctx, &d->fbox, fb));
+            TRY(dupload(ctx, st, &d->fbox, fb));
             for (int tr = 0; tr < 2; ++tr) {
                 std::vector<std::pair<int64_t, int64_t>> pr(ctx->free_near.size());   // (row leaf, column leaf)
                 for (size_t i = 0; i < pr.size(); ++i) {
@@ -846,8 +854,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
                     }
                     off[b + 1] = (int)runs.size();
                 }
-                TRY(dupload(ctx, tr ? &d->froffT : &d->froff, off));
-                TRY(dupload(ctx, tr ? &d->frunsT : &d->fruns, runs));
+                TRY(dupload(ctx, st, tr ? &d->froffT : &d->froff, off));
+                TRY(dupload(ctx, st, tr ? &d->frunsT : &d->fruns, runs));
             }
         }
     }
@@ -1287,7 +1295,7 @@ lmfmm_status batch_work(lmfmm_batch *b, int variant, M2LWork **dst, int64_t *n)
     }
     void *q = nullptr;
     if (cudaMalloc(&q, std::max<size_t>(1, all.size()) * sizeof(M2LWork)) != cudaSuccess) return LMFMM_ERR_OOM;
-    if (!all.empty() && cudaMemcpy(q, all.data(), all.size() * sizeof(M2LWork), cudaMemcpyHostToDevice)) {
+    if (copy_in(q, all.data(), all.size() * sizeof(M2LWork), b->cap)) {
         cudaFree(q);
         return LMFMM_ERR_CUDA;
     }
@@ -1345,7 +1353,8 @@ lmfmm_status lmfmm_batch_create(lmfmm_batch **out, lmfmm_ctx *const *ctxs, int n
     for (int i = 0; i < n; ++i) b->merged = b->merged && DS(ctxs[i])->m2l_kernel == 3;
     lmfmm_status rc = LMFMM_OK;
     if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaMalloc((void **)&b->status, sizeof(int)) != cudaSuccess || cudaMemset(b->status, 0, sizeof(int)))
+        cudaMalloc((void **)&b->status, sizeof(int)) != cudaSuccess ||
+        cudaMemsetAsync(b->status, 0, sizeof(int), b->cap) != cudaSuccess || cudaStreamSynchronize(b->cap) != cudaSuccess)
         rc = LMFMM_ERR_CUDA;
     if (!rc && b->merged) {
         std::vector<TcProb> hp(n);
@@ -1354,7 +1363,7 @@ lmfmm_status lmfmm_batch_create(lmfmm_batch **out, lmfmm_ctx *const *ctxs, int n
             hp[i] = TcProb{d->m2l, d->ephase, d->tab, d->mepk, (cf *)d->le};
         }
         if (cudaMalloc((void **)&b->dprobs, n * sizeof(TcProb)) != cudaSuccess ||
-            cudaMemcpy(b->dprobs, hp.data(), n * sizeof(TcProb), cudaMemcpyHostToDevice) != cudaSuccess)
+            copy_in(b->dprobs, hp.data(), n * sizeof(TcProb), b->cap) != cudaSuccess)
             rc = LMFMM_ERR_CUDA;
         if (!rc) rc = batch_work(b, 0, &b->dwork, &b->nwork);
     }
@@ -1465,7 +1474,8 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream)
     batch_drop_graph(b);   // the next matvec captures the chosen list
     int f = 0;
     cudaMemcpy(&f, b->status, sizeof(int), cudaMemcpyDeviceToHost);
-    cudaMemset(b->status, 0, sizeof(int));
+    if (cudaMemsetAsync(b->status, 0, sizeof(int), st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+        return LMFMM_ERR_CUDA;
     if (f) {
         b->err = "batch_tune: a bounded tensor-core wait gave up during the timing runs";
         return LMFMM_ERR_TIMEOUT;
@@ -1541,7 +1551,7 @@ lmfmm_status lmfmm_test_set_status(lmfmm_ctx *ctx, int bits)
     CK(cudaDeviceSynchronize());
     CK(cudaMemcpy(&f, DS(ctx)->mvstatus, sizeof(int), cudaMemcpyDeviceToHost));
     f |= bits;
-    CK(cudaMemcpy(DS(ctx)->mvstatus, &f, sizeof(int), cudaMemcpyHostToDevice));
+    CK(copy_in(DS(ctx)->mvstatus, &f, sizeof(int), cudaStreamLegacy));
     return LMFMM_OK;
 }
 
@@ -1589,9 +1599,7 @@ lmfmm_status lmfmm_direct(lmfmm_ctx *ctx, const lmfmm_c128 *J, lmfmm_c128 *Phi, 
     }
     coef = (cd *)q2;
     lmfmm_status rc = LMFMM_OK;
-    if (!all.empty() &&
-        cudaMemcpy(dn, all.data(), all.size() * sizeof(NearPair), cudaMemcpyHostToDevice))
-        rc = LMFMM_ERR_CUDA;
+    if (copy_in(dn, all.data(), all.size() * sizeof(NearPair), st)) rc = LMFMM_ERR_CUDA;
     if (!rc) {
         double a = medium_a(ctx->med);
         cudaMemsetAsync(d->flag, 0, sizeof(int), st);
@@ -1671,7 +1679,7 @@ lmfmm_status lmfmm_m2l_table(lmfmm_ctx *ctx, int l, int lp, int tgt_up, int src_
     if (!d->flag) {
         CK(cudaMalloc((void **)&d->flag, sizeof(int)));
         d->allocs.push_back(d->flag);
-        CK(cudaMemset(d->flag, 0, sizeof(int)));
+        CK(cudaMemsetAsync(d->flag, 0, sizeof(int), (cudaStream_t)stream));
     }
     std::vector<GeomDev> hg(1);
     hg[0].comp = 0;
@@ -1687,9 +1695,9 @@ lmfmm_status lmfmm_m2l_table(lmfmm_ctx *ctx, int l, int lp, int tgt_up, int src_
     CK(cudaMalloc(&qG, G.size() * sizeof(cd)));
     CK(cudaMalloc(&qi, sizeof(int)));
     int zero = 0;
-    CK(cudaMemcpy(qc, &c, sizeof(CompDev), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(qG, G.data(), G.size() * sizeof(cd), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(qi, &zero, sizeof(int), cudaMemcpyHostToDevice));
+    CK(copy_in(qc, &c, sizeof(CompDev), (cudaStream_t)stream));
+    CK(copy_in(qG, G.data(), G.size() * sizeof(cd), (cudaStream_t)stream));
+    CK(copy_in(qi, &zero, sizeof(int), (cudaStream_t)stream));
     lmfmm_status rc = tabulate(ctx, hg, (const CompDev *)qc, (const cd *)qG, (const int *)qi,
                                (cd *)out, (cudaStream_t)stream);
     cudaFree(qc);

@@ -82,7 +82,10 @@ cudaError_t configure_leaf_kernels()
     if ((e = cudaMemcpyToSymbol(c_ld, ld, sizeof(ld))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_lc, lc, sizeof(lc))) != cudaSuccess) return e;
     if ((e = cudaMemcpyToSymbol(c_sk, sk, sizeof(sk))) != cudaSuccess) return e;
-    return cudaMemcpyToSymbol(c_idf, idf, sizeof(idf));
+    if ((e = cudaMemcpyToSymbol(c_idf, idf, sizeof(idf))) != cudaSuccess) return e;
+    // small copies may return before they have landed, and kernels of non-blocking streams do not
+    // wait for this stream
+    return cudaStreamSynchronize(cudaStreamLegacy);
 }
 
 bool leaf_fast_supported(int p) { return p >= 1 && p <= LF_PMAX; }

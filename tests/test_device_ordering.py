@@ -37,3 +37,16 @@ def test_shared_memory_filled_by_other_lanes_is_read_behind_a_barrier():
             seen += 1
             assert BARRIER.search(m.group(0)), "%s: a stage is refilled without a barrier" % name
     assert seen >= 2
+
+
+def test_uploads_run_on_the_stream_that_reads_them():
+    """A cudaMemcpy from pageable memory or a cudaMemset runs on the legacy stream and may return
+    before it has landed; a non-blocking stream is not ordered behind it.  So device memory is
+    written by the asynchronous forms on the reading stream, and symbols are followed by a wait."""
+    for name, text in _sources():
+        for m in re.finditer(r"\bcudaMemcpy\s*\(", text):
+            call = text[m.start():text.index(";", m.start())]
+            assert "DeviceToHost" in call, "%s: %s" % (name, call)
+        assert not re.search(r"\bcudaMemset\s*\(", text), name
+        last = text.rfind("cudaMemcpyToSymbol(")
+        assert last < 0 or "cudaStreamSynchronize(cudaStreamLegacy)" in text[last:], name
