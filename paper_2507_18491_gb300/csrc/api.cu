@@ -75,6 +75,7 @@ struct DevState {
     bool oz = false;
     void *ozimg = nullptr, *ozimgT = nullptr, *ozpk = nullptr, *ozscr = nullptr;
     int nsm = 0;
+    int ncta = 0;                    // CTAs that yscr and ozscr hold (none of their launches has more)
     cd *stage = nullptr;             // [2][N][3] for host-buffer matvec
     cudaEvent_t ev[9]{};
     bool ev_ok = false;
@@ -639,8 +640,6 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             CK(cudaStreamSynchronize(st));
             dfree(ctx, tab64);
             d->tab = img;
-            // one scratch for the M2L and the translations, which run one after the other
-            TRY(dalloc(ctx, &d->yscr, std::max(m2l_sec_scratch_floats(p, d->nsm), trans_tc2_scratch_floats(p, d->nsm))));
         } else if (f32) {
             cf *t32 = nullptr;
             TRY(dalloc(ctx, &t32, ctx->geoms.size() * (size_t)NTAB * P * P));
@@ -651,11 +650,10 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             d->tab = t32;
         } else if (d->oz) {
             const int64_t ng = (int64_t)hg.size();
-            unsigned char *q[4] = {};
+            unsigned char *q[3] = {};
             TRY(dalloc(ctx, &q[0], m2l_oz_image_bytes(p, ng)));
             TRY(dalloc(ctx, &q[1], m2l_oz_image_bytes(p, ng)));
             TRY(dalloc(ctx, &q[2], m2l_oz_packed_bytes(p, nbox)));
-            TRY(dalloc(ctx, &q[3], m2l_oz_scratch_bytes(p, d->nsm)));
             launch_oz_image(p, false, ng, d->geoms, d->comps, tab64, q[0], st);
             launch_oz_image(p, true, ng, d->geoms, d->comps, tab64, q[1], st);
             CK(cudaGetLastError());
@@ -664,7 +662,6 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             d->ozimg = q[0];
             d->ozimgT = q[1];
             d->ozpk = q[2];
-            d->ozscr = q[3];
         } else {
             launch_scale_tables<double>(p, 0, (int64_t)hg.size(), d->geoms, tab64, tab64, st);
             CK(cudaGetLastError());
@@ -699,6 +696,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     }
     TRY(dupload(ctx, st, &d->m2lwork, mw));
     d->n_m2lwork = (int64_t)mw.size();
+    int64_t most_items = std::max<int64_t>(1, d->n_m2lwork);   // of one launch with a scratch per CTA
     // translation matrices (exact addition theorem), on the device from the groups' factors
     {
         const int64_t ngr = (int64_t)ctx->tgroups.size();
@@ -774,6 +772,8 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
                 }
             }
             d->twork_off[ctx->depth + 1] = (int64_t)tw.size();
+            for (int lev = 1; lev <= ctx->depth; ++lev)
+                most_items = std::max(most_items, d->twork_off[lev + 1] - d->twork_off[lev]);
             TRY(dupload(ctx, st, &d->twork, tw));
         }
         // work items per child level
@@ -797,6 +797,16 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             dfree(ctx, up64);
             dfree(ctx, dn64);
         }
+    }
+    // scratch of the CTAs that a launch can have: a small problem has fewer items than the chip has SMs
+    d->ncta = (int)std::min<int64_t>(d->nsm, most_items);
+    if (d->m2l_kernel == 3) {
+        // one scratch for the M2L and the translations, which run one after the other
+        TRY(dalloc(ctx, &d->yscr, std::max(m2l_sec_scratch_floats(p, d->ncta), trans_tc2_scratch_floats(p, d->ncta))));
+    } else if (d->oz) {
+        unsigned char *q = nullptr;
+        TRY(dalloc(ctx, &q, m2l_oz_scratch_bytes(p, d->ncta)));
+        d->ozscr = q;
     }
     // near field
     TRY(dupload(ctx, st, &d->near, ctx->near));
@@ -965,7 +975,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
             if (d->trans_tc) {
                 int64_t w0 = d->twork_off[lev], w1 = d->twork_off[lev + 1];
                 CK(launch_trans_tc2(p, w1 - w0, d->twork + w0, d->tchild, d->tparent, d->tupi, me, me,
-                                    d->yscr, d->nsm, d->mvstatus, st));
+                                    d->yscr, d->ncta, d->mvstatus, st));
                 nl += w1 > w0;
                 continue;
             }
@@ -992,7 +1002,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
     } else if constexpr (std::is_same<T, float>::value) {
         if (d->m2l_kernel == 3) {
             CK(launch_m2l_sec(p, d->n_m2lwork, d->m2lwork, TcProb{d->m2l, d->ephase, d->tab, d->mepk, le}, nullptr, d->yscr,
-                              d->nsm, d->mvstatus, st));
+                              d->ncta, d->mvstatus, st));
         }
         else if (d->m2l_kernel == 2)
             CK(launch_m2l_tc(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
@@ -1002,7 +1012,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
                             (const cx<T> *)d->tab, me, le, st);
     } else if (d->oz) {
         CK(launch_m2l_oz(p, false, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimg, nbox, me, le,
-                         d->ozpk, d->ozscr, d->nsm, d->mvstatus, st));
+                         d->ozpk, d->ozscr, d->ncta, d->mvstatus, st));
         ++nl;
     } else {
         launch_m2l_t<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
@@ -1020,7 +1030,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
             if (d->trans_tc) {
                 int64_t w0 = d->twork_off[lev], w1 = d->twork_off[lev + 1];
                 CK(launch_trans_tc2(p, w1 - w0, d->twork + w0, d->tparent, d->tchild, d->tdni, le, le,
-                                    d->yscr, d->nsm, d->mvstatus, st));
+                                    d->yscr, d->ncta, d->mvstatus, st));
                 nl += w1 > w0;
                 continue;
             }
@@ -1082,7 +1092,7 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     if constexpr (std::is_same<T, double>::value) {
         if (d->oz) {
             CK(launch_m2l_oz(p, true, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimgT, nbox, le, me,
-                             d->ozpk, d->ozscr, d->nsm, d->mvstatus, st));
+                             d->ozpk, d->ozscr, d->ncta, d->mvstatus, st));
             done = true;
             ++nl;
         }
@@ -1250,6 +1260,9 @@ struct lmfmm_batch {
     M2LWork *dwork = nullptr;
     int64_t nwork = 0;
     int *status = nullptr;
+    float *yscr = nullptr;        // scratch of the merged launch: a context's, or own
+    float *own_yscr = nullptr;
+    int ncta = 0;
     int variant = 0;
     double ms_variant[4] = {0, 0, 0, 0};
     cudaStream_t cap = nullptr;   // capture stream of the graph
@@ -1314,8 +1327,7 @@ lmfmm_status batch_record(lmfmm_batch *b, const void *const *J, void *const *Phi
     }
     if (b->merged) {
         if (cudaMemsetAsync(b->status, 0, sizeof(int), st) != cudaSuccess) return LMFMM_ERR_CUDA;
-        DevState *d0 = DS(b->ctxs[0]);
-        if (launch_m2l_sec(b->p, b->nwork, b->dwork, TcProb{}, b->dprobs, d0->yscr, d0->nsm, b->status, st) !=
+        if (launch_m2l_sec(b->p, b->nwork, b->dwork, TcProb{}, b->dprobs, b->yscr, b->ncta, b->status, st) !=
             cudaSuccess)
             return LMFMM_ERR_CUDA;
     }
@@ -1366,6 +1378,20 @@ lmfmm_status lmfmm_batch_create(lmfmm_batch **out, lmfmm_ctx *const *ctxs, int n
             copy_in(b->dprobs, hp.data(), n * sizeof(TcProb), b->cap) != cudaSuccess)
             rc = LMFMM_ERR_CUDA;
         if (!rc) rc = batch_work(b, 0, &b->dwork, &b->nwork);
+        // the merged launch has the items of all problems (twice as many where they are halved): the
+        // largest scratch of a context, which is idle then, or a larger one of the batch's own
+        for (lmfmm_ctx *c : b->ctxs)
+            if (DS(c)->ncta > b->ncta) {
+                b->ncta = DS(c)->ncta;
+                b->yscr = DS(c)->yscr;
+            }
+        const int want = (int)std::min<int64_t>(DS(ctxs[0])->nsm, 2 * b->nwork);
+        if (!rc && b->ncta < want) {
+            if (cudaMalloc((void **)&b->own_yscr, m2l_sec_scratch_floats(b->p, want) * sizeof(float)) != cudaSuccess)
+                rc = LMFMM_ERR_OOM;
+            b->yscr = b->own_yscr;
+            b->ncta = want;
+        }
     }
     if (rc) {
         g_err = "batch_create: device setup failed";
@@ -1434,7 +1460,6 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream)
     }
     if (cudaSetDevice(b->device) != cudaSuccess) return LMFMM_ERR_CUDA;
     cudaStream_t st = (cudaStream_t)stream;
-    DevState *d0 = DS(b->ctxs[0]);
     // defined inputs for the timing runs
     for (lmfmm_ctx *c : b->ctxs)
         if (cudaMemsetAsync(DS(c)->mepk, 0, m2l_sec_packed_bytes(b->p, (int64_t)c->boxes.size()), st) != cudaSuccess)
@@ -1450,7 +1475,7 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream)
         float tmin = 1e30f;
         for (int rep = 0; rep < 4; ++rep) {
             cudaEventRecord(e0, st);
-            launch_m2l_sec(b->p, nw, w, TcProb{}, b->dprobs, d0->yscr, d0->nsm, b->status, st);
+            launch_m2l_sec(b->p, nw, w, TcProb{}, b->dprobs, b->yscr, b->ncta, b->status, st);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0;
@@ -1525,6 +1550,7 @@ void lmfmm_batch_destroy(lmfmm_batch *b)
     cudaFree(b->dprobs);
     cudaFree(b->dwork);
     cudaFree(b->status);
+    cudaFree(b->own_yscr);
     delete b;
 }
 

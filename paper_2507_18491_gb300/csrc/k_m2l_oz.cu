@@ -488,10 +488,10 @@ size_t m2l_oz_image_bytes(int p, int64_t ngeom)
     return (size_t)ngeom * (sp.img_bytes + (size_t)sp.rows * sizeof(double));
 }
 size_t m2l_oz_packed_bytes(int p, int64_t nbox) { return (size_t)nbox * (oz_plan(p).nk[0] * 8 * sizeof(OzIn) + sizeof(double)); }
-size_t m2l_oz_scratch_bytes(int p, int nsm)
+size_t m2l_oz_scratch_bytes(int p, int ncta)
 {
     const OzPlan sp = oz_plan(p);
-    return (size_t)nsm * ((size_t)sp.nk[0] * OZ_A + (size_t)OZ_BN * sp.rows * sizeof(double2));
+    return (size_t)ncta * ((size_t)sp.nk[0] * OZ_A + (size_t)OZ_BN * sp.rows * sizeof(double2));
 }
 
 void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
@@ -509,20 +509,20 @@ void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, c
 }
 
 cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
-                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int nsm,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
                           int *status, cudaStream_t st)
 {
-    if (!m2l_oz_supported(p) || nsm < 1) return cudaErrorInvalidValue;
+    if (!m2l_oz_supported(p) || ncta < 1) return cudaErrorInvalidValue;
     const OzPlan sp = oz_plan(p);
     const int n8 = sp.nk[0] * 8;
     double *bs = (double *)((unsigned char *)packed + (size_t)nbox * n8 * sizeof(OzIn));
     if (nbox > 0) k_oz_pack<<<(unsigned)nbox, 128, 0, st>>>(p, n8, sp.D[0], in, (OzIn *)packed, bs, out);
     if (nwork <= 0) return cudaGetLastError();
     unsigned char *x = (unsigned char *)scratch;
-    k_m2l_oz<<<(unsigned)std::min<int64_t>(nwork, nsm), OZ_T, std::max<size_t>(sp.smem, 116 * 1024), st>>>(
+    k_m2l_oz<<<(unsigned)std::min<int64_t>(nwork, ncta), OZ_T, std::max<size_t>(sp.smem, 116 * 1024), st>>>(
         sp, transposed ? 1 : 0, nwork, work, pairs, (const unsigned char *)img,
         (const double *)((const unsigned char *)img + (size_t)ngeom * sp.img_bytes), (const OzIn *)packed, bs, out, x,
-        (double *)(x + (size_t)nsm * sp.nk[0] * OZ_A), status);
+        (double *)(x + (size_t)ncta * sp.nk[0] * OZ_A), status);
     return cudaGetLastError();
 }
 

@@ -692,12 +692,12 @@ __global__ void __launch_bounds__(128) k_sec_pack(int p, int n16, int D0, const 
 
 template <int RJ>
 cudaError_t launch_rj(const SecPlan &sp, int64_t nwork, const M2LWork *work, const TcProb &one, const TcProb *probs,
-                      float *yscr, int nsm, int *status, cudaStream_t st)
+                      float *yscr, int ncta, int *status, cudaStream_t st)
 {
     // each CTA takes all 512 tensor-memory columns: ask for more than half of an SM's
     // shared memory so that no two CTAs are resident on one SM
     const size_t smem = std::max<size_t>(sp.smem, 116 * 1024);
-    k_m2l_sec<RJ><<<(unsigned)std::min<int64_t>(nwork, nsm), SC_THREADS, smem, st>>>(sp, nwork, work, one, probs, yscr,
+    k_m2l_sec<RJ><<<(unsigned)std::min<int64_t>(nwork, ncta), SC_THREADS, smem, st>>>(sp, nwork, work, one, probs, yscr,
                                                                                      status);
     return cudaGetLastError();
 }
@@ -710,7 +710,7 @@ int m2l_sec_pairs() { return SC_BN; }
 // pairs lie in different shared-memory banks
 int m2l_sec_phases(int p) { return phase_row(p); }
 size_t m2l_sec_image_bytes(int p, int64_t ngeom) { return (size_t)ngeom * sec_plan(p).img_bytes; }
-size_t m2l_sec_scratch_floats(int p, int nsm) { return (size_t)nsm * 128 * sec_plan(p).yrows; }
+size_t m2l_sec_scratch_floats(int p, int ncta) { return (size_t)ncta * 128 * sec_plan(p).yrows; }
 
 void launch_sec_image(int p, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64, void *img,
                       cudaStream_t st)
@@ -742,19 +742,19 @@ void launch_sec_pack(int p, int64_t nbox, const cf *me, void *packed, cf *le, cu
 }
 
 cudaError_t launch_m2l_sec(int p, int64_t nwork, const M2LWork *work, const TcProb &one, const TcProb *probs,
-                           float *yscr, int nsm, int *status, cudaStream_t st)
+                           float *yscr, int ncta, int *status, cudaStream_t st)
 {
     if (nwork <= 0) return cudaSuccess;
-    if (!m2l_sec_supported(p) || nsm < 1) return cudaErrorInvalidValue;
+    if (!m2l_sec_supported(p) || ncta < 1) return cudaErrorInvalidValue;
     const SecPlan sp = sec_plan(p);
     switch ((sp.D0 + 31) / 32) {
     case 1:
     case 2:
-    case 3: return launch_rj<3>(sp, nwork, work, one, probs, yscr, nsm, status, st);   // p <= 6
-    case 4: return launch_rj<4>(sp, nwork, work, one, probs, yscr, nsm, status, st);   // p <= 8
+    case 3: return launch_rj<3>(sp, nwork, work, one, probs, yscr, ncta, status, st);   // p <= 6
+    case 4: return launch_rj<4>(sp, nwork, work, one, probs, yscr, ncta, status, st);   // p <= 8
     case 5:
-    case 6: return launch_rj<6>(sp, nwork, work, one, probs, yscr, nsm, status, st);   // p <= 10
-    default: return launch_rj<9>(sp, nwork, work, one, probs, yscr, nsm, status, st);  // p <= 12
+    case 6: return launch_rj<6>(sp, nwork, work, one, probs, yscr, ncta, status, st);   // p <= 10
+    default: return launch_rj<9>(sp, nwork, work, one, probs, yscr, ncta, status, st);  // p <= 12
     }
 }
 

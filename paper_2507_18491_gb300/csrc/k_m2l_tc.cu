@@ -866,18 +866,18 @@ bool trans_tc2_supported(int p)
            v2_plan(p).ST >= 4;
 }
 
-size_t trans_tc2_scratch_floats(int p, int nsm) { return (size_t)nsm * 128 * v2_plan(p).NR; }
+size_t trans_tc2_scratch_floats(int p, int ncta) { return (size_t)ncta * 128 * v2_plan(p).NR; }
 
 cudaError_t launch_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc,
-                             const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
+                             const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int ncta,
                              int *status, cudaStream_t st)
 {
     if (nwork <= 0) return cudaSuccess;
-    if (!trans_tc2_supported(p) || nsm < 1) return cudaErrorInvalidValue;
+    if (!trans_tc2_supported(p) || ncta < 1) return cudaErrorInvalidValue;
     // each CTA takes all 512 tensor-memory columns: ask for more than half of
     // an SM's shared memory so that no two CTAs are resident on one SM
     const size_t smem = std::max<size_t>(v2_plan(p).total, 116 * 1024);
-    k_trans_tc2<<<(unsigned)std::min<int64_t>(nwork, (int64_t)nsm), V2_THREADS, smem, st>>>(
+    k_trans_tc2<<<(unsigned)std::min<int64_t>(nwork, (int64_t)ncta), V2_THREADS, smem, st>>>(
         p, nwork, work, tsrc, tdst, (const unsigned char *)img, in, out, yscr, status);
     return cudaGetLastError();
 }

@@ -163,13 +163,13 @@ cudaError_t launch_m2l_tc(int p, int64_t nwork, const M2LWork *work, const GeomD
 // sectors of sector.cuh.  Items M2LWork{geom, npair <= 64, pair0, prob}; img is the
 // image of the sector matrices in three bf16 pieces (launch_sec_image from the FP64
 // tables); ephase holds G[d] = i^d e^{i d phi} of every pair, d = -(p+1)..p, in rows of
-// m2l_sec_phases(p) entries (FP32 from FP64); yscr holds m2l_sec_scratch_floats(p, nsm)
-// floats, nsm = CTAs of the launch (the SM count)
+// m2l_sec_phases(p) entries (FP32 from FP64); yscr holds m2l_sec_scratch_floats(p, ncta)
+// floats, ncta = the most CTAs that the launch may have (at most the SM count: one per SM)
 bool m2l_sec_supported(int p);
 int m2l_sec_pairs();             // pairs of a full work item
 int m2l_sec_phases(int p);
 size_t m2l_sec_image_bytes(int p, int64_t ngeom);
-size_t m2l_sec_scratch_floats(int p, int nsm);
+size_t m2l_sec_scratch_floats(int p, int ncta);
 cudaError_t configure_m2l_sec();
 void launch_sec_image(int p, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64, void *img,
                       cudaStream_t st);
@@ -180,7 +180,7 @@ size_t m2l_sec_packed_bytes(int p, int64_t nbox);
 void launch_sec_pack(int p, int64_t nbox, const cf *me, void *packed, cf *le, cudaStream_t st);
 // probs: the problems of a batched launch (device array), or null with one problem in `one`
 cudaError_t launch_m2l_sec(int p, int64_t nwork, const M2LWork *work, const TcProb &one, const TcProb *probs,
-                           float *yscr, int nsm, int *status, cudaStream_t st);
+                           float *yscr, int ncta, int *status, cudaStream_t st);
 // k_m2l_oz.cu: M2L of the FP64 form on the tensor cores, operands as eight base-256 digits.
 // out is cleared, then out[tgt] += M in[src] over the items' pairs (transposed: in over the
 // targets, out over the sources); img from launch_oz_image (m2l_oz_image_bytes), packed and
@@ -189,21 +189,21 @@ bool m2l_oz_supported(int p);
 int m2l_oz_pairs();
 size_t m2l_oz_image_bytes(int p, int64_t ngeom);
 size_t m2l_oz_packed_bytes(int p, int64_t nbox);
-size_t m2l_oz_scratch_bytes(int p, int nsm);
+size_t m2l_oz_scratch_bytes(int p, int ncta);
 cudaError_t configure_m2l_oz();
 void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
                      void *img, cudaStream_t st);
 cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
-                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int nsm,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
                           int *status, cudaStream_t st);
 // M2M or L2L on a persistent tensor-core kernel (k_m2l_tc.cu, p <= 12): items M2LWork{geom = translation group, t = 0,
 // npair, pair0} over pairs (tsrc[q], tdst[q]), 3 helical columns each; img holds
 // one tiled matrix per group (launch_tile_matrices, tc2_matrix_bytes(p) each)
 cudaError_t launch_trans_tc2(int p, int64_t nwork, const M2LWork *work, const int64_t *tsrc,
-                             const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int nsm,
+                             const int64_t *tdst, const void *img, const cf *in, cf *out, float *yscr, int ncta,
                              int *status, cudaStream_t st);
 bool trans_tc2_supported(int p);
-size_t trans_tc2_scratch_floats(int p, int nsm);
+size_t trans_tc2_scratch_floats(int p, int ncta);
 size_t tc2_matrix_bytes(int p);
 void launch_tile_matrices(int p, int64_t ng, const cd *M, void *img, cudaStream_t st);   // [ng][P][P], row = output index
 template <typename T>
