@@ -339,25 +339,28 @@ def main():
         lmfmm.matvec_host(op.ctx, Jh, Ph)
     e2e_ms = allmax((time.time() - t1) * 1e3 / args.steps, ws)
     P = (p + 1) ** 2
-    # the sector kernels (FP64 form, mixed form on the tensor cores) need 36 P^2 flops per box pair,
+    # the sector kernels (both forms on the tensor cores) need 36 P^2 flops per box pair,
     # the five-table ones 8 P^2 per helical column (nine columns per pair)
-    sector = st["m2l_kernel"] in (0, 3)
+    digits = bool(st["m2l_digits"])
+    sector = digits or st["m2l_kernel"] == 3
     flops = (4.0 if sector else 8.0) * P * P * st["m2l_columns"]
     m2l_s = float(np.mean(m2l_ms)) * 1e-3
     achieved = flops / m2l_s / 1e12
-    kern = {0: "k_m2l_oz", 1: "k_m2l<float>", 2: "k_m2l_tc", 3: "k_m2l_sec"}[st["m2l_kernel"]]
+    kern = {0: "k_m2l_oz" if digits else "k_m2l<double>", 1: "k_m2l<float>", 2: "k_m2l_tc", 3: "k_m2l_sec"}[st["m2l_kernel"]]
     # DRAM bytes per launch of k_m2l_sec: the matrix image times the read + write / image
     # ratio of an ncu capture of the same kernel (TRAFFIC_RATIO, three-layer N = 8192,
     # p = 12, depth 4, theta 0.55: the image once and the accumulator scratch leaving L2).  The
     # multipole expansions fit in L2 in that case but not at N = 2^20, so the
     # scaled figure is an estimate there.  Other kernels: not captured
     traffic = st["bytes_tables"] * TRAFFIC_RATIO if st["m2l_kernel"] == 3 else None
-    bound = "alu" if st["m2l_kernel"] == 1 else "tensor"
-    if prec == lmfmm.FP64:
+    bound = "tensor" if digits or st["m2l_kernel"] >= 2 else "alu"
+    if digits:
         peak, peak_src = tensor_peak(tf32=False)
         peak, peak_src = peak / 36, peak_src + " / 36 digit products of an FP64 one"
     elif bound == "tensor":
         peak, peak_src = tensor_peak(tf32=st["m2l_kernel"] == 2)
+    elif prec == lmfmm.FP64:
+        peak, peak_src = FP64_PEAK_TFLOPS, "derived (not measured) FP64 ALU: 152 SM x 2 FMA/clk x 2 x 2070 MHz"
     else:
         peak, peak_src = FP32_PEAK_TFLOPS, "derived (not measured) FP32 ALU: 152 SM x 128 FMA/clk x 2 x 2070 MHz"
     line = {
@@ -369,7 +372,7 @@ def main():
         "config": {"workload": w.name, "N": w.N, "layers": int(w.d.size + 1), "p": p,
                    "depth": st["depth"], "depth_tuner": tuner, "theta": opt["theta"],
                    "precision": args.precision,
-                   "tensor_cores": int(args.tensor_cores) if prec == lmfmm.MIXED else 0,
+                   "tensor_cores": int(args.tensor_cores) if prec == lmfmm.MIXED else st["m2l_digits"],
                    "components": st["n_components"], "m2l_pairs": st["n_m2l_pairs"],
                    "geometries": st["n_geometries"],
                    "geometries_same_layer": st["n_geometries_same_layer"],

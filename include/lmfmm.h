@@ -77,14 +77,17 @@ typedef struct {
     double eta;        /* ... and its vertical transmission distance is >= eta * |c_s - c_t| */
     double quad_tol;   /* relative cut-off of the k_rho tails (>= 1e-16) */
     int precision;     /* LMFMM_FP64 or LMFMM_MIXED (FP32 translation arithmetic) */
-    int tensor_cores;  /* mixed form only: products on the tcgen05 tensor cores with FP32-level
+    int tensor_cores;  /* mixed form: products on the tcgen05 tensor cores with FP32-level
                           accuracy.  1: M2L on the persistent kernel (three-piece bf16 split,
                           pre-tiled table image) for p <= 12, else the streamed-operand kernel
                           (three-term TF32 split, p <= 15); 2: the streamed-operand kernel;
                           3: as 1, and M2M / L2L on the persistent kernel too (inputs taken from
                           the highest degree down; four-layer N = 2^20, p = 12: 7.3e-7 against
                           the direct sum, 6.4e-7 with 1); 0: FP32 SIMT pipes.  Beyond p = 15 the
-                          SIMT kernel runs.  Ignored by the FP64 form. */
+                          SIMT kernel runs.  FP64 form: 1, 2 or 3 M2L and its transpose on the
+                          tensor cores (products of base-256 digits, two images of 4.33 MB per
+                          geometry at p = 12) where the images fit in memory, 0 (or where they do
+                          not) the FP64 SIMT kernels (tables of 2.28 MB; 8 to 30 times slower) */
     int quad_node_cap; /* largest k_rho node count of one Sommerfeld integral (an M2L table
                           or a near box pair); beyond it lmfmm_build returns LMFMM_ERR_QUAD
                           (table: checked on the host before any launch; near pair: the
@@ -111,8 +114,7 @@ typedef struct {
     double ms_setup;       /* wall time of the last lmfmm_build */
     double ms_stage[8];    /* last matvec: P2M, M2M, M2L, L2L, L2P, S2T, permute, total */
     int64_t m2l_columns;   /* helical columns pushed through M2L tables per matvec */
-    int m2l_kernel;        /* M2L product of the built form: 0 FP64 (tcgen05 on base-256 digits;
-                              SIMT where its images do not fit in memory), 1 FP32 SIMT,
+    int m2l_kernel;        /* M2L product of the built form: 0 FP64 (m2l_digits says which), 1 FP32 SIMT,
                               2 tcgen05 streamed-operand kernel, 3 tcgen05 persistent kernel */
     int launches;          /* kernels launched by the last matvec */
     int64_t n_geometries_same_layer;  /* of n_geometries: components with l = l' (their tables
@@ -128,6 +130,8 @@ typedef struct {
     int adjoint_transposed; /* 1: lmfmm_matvec_adjoint applies the transposed operators (FP64
                                form, mixed form with tensor_cores = 0); 0: the reciprocity
                                identity with the forward kernels (tensor-core forms) */
+    int m2l_digits;         /* FP64 form: 1 the M2L runs on the tensor cores, on base-256 digits;
+                               0 on the SIMT kernels.  Mixed form: 0 */
     int64_t n_free_geometries;        /* free-space M2L tables (of n_geometries) */
     int64_t n_free_near_point_pairs;  /* free-space near-field point pairs */
 } lmfmm_stats;

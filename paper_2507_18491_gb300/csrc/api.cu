@@ -67,7 +67,7 @@ struct DevState {
     int *flag = nullptr;
     int *mvstatus = nullptr;         // matvec status word (bit 4: tensor-core wait gave up)
     int fail_m2l = 0;                // test hook: status bits the next forward M2L leaves
-    int m2l_kernel = 0;              // 0 FP64 SIMT, 1 FP32 SIMT, 2 tcgen05 streamed, 3 tcgen05 persistent
+    int m2l_kernel = 0;              // 0 FP64 (oz: which), 1 FP32 SIMT, 2 tcgen05 streamed, 3 tcgen05 persistent
     cf *ephase = nullptr;            // sector kernel: phases G[d] per pair
     void *mepk = nullptr;            // ... and the packed multipole expansions it reads
     // FP64 form on the tensor cores (k_m2l_oz.cu): images of the sector blocks and their
@@ -507,9 +507,10 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         return LMFMM_ERR_OOM;
     }
     CK(cudaDeviceGetAttribute(&d->nsm, cudaDevAttrMultiProcessorCount, ctx->device));
-    // FP64 form: the tensor-core M2L holds two images of 16 bytes per sector entry (the SIMT
-    // kernels one table of 16 bytes); where both do not fit, the SIMT kernels run
-    if (ctx->prm.precision == LMFMM_FP64 && m2l_oz_supported(p)) {
+    // FP64 form: the tensor-core M2L holds two images of 32 bytes per sector entry (eight digits of
+    // a complex number; 4.33 MB each per geometry at p = 12, where the five tables of the SIMT kernels
+    // take 2.28 MB).  The SIMT kernels run where both do not fit, or on request
+    if (ctx->prm.precision == LMFMM_FP64 && ctx->prm.tensor_cores != 0 && m2l_oz_supported(p)) {
         const double oz_need = 2.0 * (double)m2l_oz_image_bytes(p, (int64_t)ctx->geoms.size()) +
                                (double)m2l_oz_packed_bytes(p, nbox) + (double)m2l_oz_scratch_bytes(p, d->nsm);
         d->oz = need + oz_need <= 0.85 * (double)fr;
@@ -896,6 +897,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     S.n_free_near_point_pairs = ctx->n_free_pp;
     S.ms_tabulate = ms_tab;
     S.adjoint_transposed = d->m2l_kernel <= 1;
+    S.m2l_digits = d->oz;
     S.tab_flops = 8.0 * tab_terms * (p + 2) * (p + 2) +
                   8.0 * (double)ctx->geoms.size() * NTAB * (double)P * P * (p + 2);
     return LMFMM_OK;

@@ -46,7 +46,7 @@ class Stats(ctypes.Structure):
                 ("ms_stage", ctypes.c_double * 8), ("m2l_columns", ctypes.c_int64),
                 ("m2l_kernel", ctypes.c_int), ("launches", ctypes.c_int),
                 ("n_geometries_same_layer", ctypes.c_int64), ("ms_tabulate", ctypes.c_double),
-                ("tab_flops", ctypes.c_double), ("adjoint_transposed", ctypes.c_int),
+                ("tab_flops", ctypes.c_double), ("adjoint_transposed", ctypes.c_int), ("m2l_digits", ctypes.c_int),
                 ("n_free_geometries", ctypes.c_int64), ("n_free_near_point_pairs", ctypes.c_int64)]
 
 
