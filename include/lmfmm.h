@@ -296,6 +296,15 @@ lmfmm_status lmfmm_m2l_table(lmfmm_ctx *ctx, int l, int lp, int tgt_up, int src_
 lmfmm_status lmfmm_translation_matrix(int p, lmfmm_c128 k, const double *t, lmfmm_c128 *m2m,
                                       lmfmm_c128 *l2l);
 
+/* The matrices of translation group `group` (0, 1, ... until LMFMM_ERR_ARG: one per
+ * layer, level and octant) as lmfmm_build formed them on the device, FP64 form only:
+ * layer, t[3] = child centre - parent centre and scales[2] = {s_c, s_p}, |k| times the
+ * cell size of the child and the parent level; m2m and l2l (host, [P][P], as
+ * lmfmm_translation_matrix) carry the scaling of the expansions, m2m s_c^n' / s_p^n
+ * and l2l s_c^nu / s_p^n' for row degree n or nu and column degree n'. */
+lmfmm_status lmfmm_built_translation(lmfmm_ctx *ctx, int64_t group, int *layer, double *t, double *scales,
+                                     lmfmm_c128 *m2m, lmfmm_c128 *l2l);
+
 /* Host-only (no device, no context): the free-space M2L of the FMM's free
  * part (Section 2, eq. maxwell_M2L_freespace with the Hessian of eq.
  * GEandGH) between a source box centre c_s and a target centre c_t with

@@ -702,26 +702,24 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
     {
         const int64_t ngr = (int64_t)ctx->tgroups.size();
         const int nfac = trans_factor_count(p);
-        std::vector<double> fac((size_t)ngr * nfac), gw, gP;
-        std::vector<double2> scl(ngr);
+        std::vector<dd> fac((size_t)ngr * nfac), gw, gP;
         for (int64_t i = 0; i < ngr; ++i) {
-            const TransGroup &g = ctx->tgroups[i];
-            trans_factors(p, zc(ctx->med.k[g.layer].x, ctx->med.k[g.layer].y), g.t, &fac[i * nfac]);
             // scaled expansions: M~ = M / s^n, L~ = L s^nu, s = |k| S_level
-            scl[i] = double2{kabs(g.layer) * lev_size(g.level), kabs(g.layer) * lev_size(g.level - 1)};
+            const TransGroup &g = ctx->tgroups[i];
+            trans_factors(p, zc(ctx->med.k[g.layer].x, ctx->med.k[g.layer].y), g.t, kabs(g.layer) * lev_size(g.level),
+                          kabs(g.layer) * lev_size(g.level - 1), &fac[i * nfac]);
         }
         gaunt_nodes(p, gw, gP);
-        double *dw = nullptr, *dP = nullptr, *dGt = nullptr, *dfac = nullptr;
-        double2 *dsc = nullptr;
+        dd *dw = nullptr, *dP = nullptr, *dfac = nullptr;
+        double *dGt = nullptr;
         cd *up64 = nullptr, *dn64 = nullptr;
         TRY(dupload(ctx, st, &dw, gw));
         TRY(dupload(ctx, st, &dP, gP));
         TRY(dupload(ctx, st, &dfac, fac));
-        TRY(dupload(ctx, st, &dsc, scl));
         TRY(dalloc(ctx, &dGt, (size_t)P * P * (p + 1)));
         TRY(dalloc(ctx, &up64, (size_t)ngr * P * P));
         TRY(dalloc(ctx, &dn64, (size_t)ngr * P * P));
-        launch_trans_build(p, (int)gw.size(), dw, dP, dGt, ngr, dfac, dsc, up64, dn64, st);
+        launch_trans_build(p, (int)gw.size(), dw, dP, dGt, ngr, dfac, up64, dn64, st);
         CK(cudaGetLastError());
         d->trans_tc = d->m2l_kernel == 3 && ctx->prm.tensor_cores == 3 && trans_tc2_supported(p);
         // the SIMT forms also keep the transposes (the transposed operator runs on them)
@@ -793,7 +791,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         d->gwork_off[ctx->depth + 1] = (int64_t)gwk.size();
         TRY(dupload(ctx, st, &d->gwork, gwk));
         CK(cudaStreamSynchronize(st));
-        for (void *q : {(void *)dw, (void *)dP, (void *)dGt, (void *)dfac, (void *)dsc}) dfree(ctx, q);
+        for (void *q : {(void *)dw, (void *)dP, (void *)dGt, (void *)dfac}) dfree(ctx, q);
         if (f32) {
             dfree(ctx, up64);
             dfree(ctx, dn64);
@@ -1747,6 +1745,36 @@ lmfmm_status lmfmm_translation_matrix(int p, lmfmm_c128 k, const double *t, lmfm
     std::vector<double> gv;
     gaunt_table(p, goff, gl, gv);
     translation_matrix(p, zc(k.re, k.im), t, goff, gl, gv, (cd *)m2m, (cd *)l2l);
+    return LMFMM_OK;
+}
+
+lmfmm_status lmfmm_built_translation(lmfmm_ctx *ctx, int64_t group, int *layer, double *t, double *scales, lmfmm_c128 *m2m,
+                                     lmfmm_c128 *l2l)
+{
+    if (!ctx) return LMFMM_ERR_ARG;
+    if (!ctx->built) {
+        ctx->err = "built_translation: call lmfmm_build first";
+        return LMFMM_ERR_STATE;
+    }
+    if (ctx->prm.precision != LMFMM_FP64) {
+        ctx->err = "built_translation: the mixed form holds its matrices in other formats";
+        return LMFMM_ERR_UNSUPPORTED;
+    }
+    if (group < 0 || group >= (int64_t)ctx->tgroups.size() || !layer || !t || !scales || !m2m || !l2l) {
+        ctx->err = "built_translation: no such group or NULL buffer";
+        return LMFMM_ERR_ARG;
+    }
+    CK(cudaSetDevice(ctx->device));
+    const DevState *d = DS(ctx);
+    const TransGroup &g = ctx->tgroups[group];
+    const int P = (ctx->prm.p + 1) * (ctx->prm.p + 1);
+    const double s1 = std::hypot(ctx->med.k[g.layer].x, ctx->med.k[g.layer].y) * 2.0 * ctx->root_h;
+    *layer = g.layer;
+    std::copy(g.t, g.t + 3, t);
+    scales[0] = s1 / (double)(1u << g.level);
+    scales[1] = s1 / (double)(1u << (g.level - 1));
+    CK(cudaMemcpy(m2m, (const cd *)d->tup + group * P * P, (size_t)P * P * sizeof(cd), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(l2l, (const cd *)d->tdn + group * P * P, (size_t)P * P * sizeof(cd), cudaMemcpyDeviceToHost));
     return LMFMM_OK;
 }
 

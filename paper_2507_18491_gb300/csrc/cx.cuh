@@ -12,6 +12,11 @@ struct cx {
 using cd = cx<double>;
 using cf = cx<float>;
 
+// a value as the unevaluated sum of two doubles, |l| <= ulp(h) / 2
+struct dd {
+    double h, l;
+};
+
 template <typename T> LMF_HD cx<T> mk(T a, T b) { return cx<T>{a, b}; }
 LMF_HD cd mkd(double a, double b = 0.0) { return cd{a, b}; }
 

@@ -680,9 +680,16 @@ static void sph_bessel_ld(lz z, int L, std::vector<lz> &j)
     for (auto &v : j) v *= sc;
 }
 
+// a long double as two doubles
+static dd two_doubles(ld v)
+{
+    const double h = (double)v;
+    return dd{h, (double)(v - (ld)h)};
+}
+
 // Gauss-Legendre nodes of the Gaunt integrals of orders up to (2p, p, p): weights (times
 // 2 pi) and P~_l^m (l <= 2p, m >= 0) at every node
-void gaunt_nodes(int p, std::vector<double> &w, std::vector<double> &Pq)
+void gaunt_nodes(int p, std::vector<dd> &w, std::vector<dd> &Pq)
 {
     const int nq = 2 * p + 4, nt = (2 * p + 1) * (2 * p + 2) / 2;
     w.resize(nq);
@@ -703,15 +710,16 @@ void gaunt_nodes(int p, std::vector<double> &w, std::vector<double> &Pq)
             x -= dx;
             if (std::fabs((double)dx) < 1e-22) break;
         }
-        w[i] = (double)(4 * pi / ((1 - x * x) * dp * dp));
+        w[i] = two_doubles(4 * pi / ((1 - x * x) * dp * dp));
         legendre_ld(2 * p, x, std::sqrt(1 - x * x), P);
-        for (int e = 0; e < nt; ++e) Pq[(size_t)i * nt + e] = (double)P[e];
+        for (int e = 0; e < nt; ++e) Pq[(size_t)i * nt + e] = two_doubles(P[e]);
     }
 }
 
-// factors of W(t) that do not depend on the entry, as doubles: i^l j_l(k |t|) (complex,
-// l <= 2p), P~_l^m(t^) (m >= 0), 4 pi e^{-i mu phi} (complex, mu = -2p..2p)
-void trans_factors(int p, zc kk, const double t[3], double *out)
+// factors of W(t) that do not depend on the entry: i^l j_l(k |t|) (complex, l <= 2p), P~_l^m(t^)
+// (m >= 0), 4 pi e^{-i mu phi} (complex, mu = -2p..2p), and the powers sc^n, sp^n (n <= p) of the
+// child and the parent level's scale
+void trans_factors(int p, zc kk, const double t[3], double sc, double sp, dd *out)
 {
     const int lmax = 2 * p;
     const ld tn = std::sqrt((ld)t[0] * t[0] + (ld)t[1] * t[1] + (ld)t[2] * t[2]);
@@ -719,17 +727,19 @@ void trans_factors(int p, zc kk, const double t[3], double *out)
     sph_bessel_ld(lz(kk.real(), kk.imag()) * tn, lmax, jl);
     for (int l = 0; l <= lmax; ++l) {
         const lz v = ((l & 1) ? lz(0, 1) : lz(1)) * jl[l] * (ld)((l & 2) ? -1 : 1);
-        *out++ = (double)v.real();
-        *out++ = (double)v.imag();
+        *out++ = two_doubles(v.real());
+        *out++ = two_doubles(v.imag());
     }
     std::vector<ld> Pt;
     legendre_ld(lmax, tn > 0 ? t[2] / tn : 1, tn > 0 ? std::sqrt((ld)t[0] * t[0] + (ld)t[1] * t[1]) / tn : 0, Pt);
-    for (int e = 0; e < (lmax + 1) * (lmax + 2) / 2; ++e) *out++ = (double)Pt[e];
+    for (int e = 0; e < (lmax + 1) * (lmax + 2) / 2; ++e) *out++ = two_doubles(Pt[e]);
     const ld phi = std::atan2((ld)t[1], (ld)t[0]), fourpi = 4 * 3.14159265358979323846264338327950288L;
     for (int mu = -lmax; mu <= lmax; ++mu) {
-        *out++ = (double)(fourpi * std::cos(mu * phi));
-        *out++ = (double)(-fourpi * std::sin(mu * phi));
+        *out++ = two_doubles(fourpi * std::cos(mu * phi));
+        *out++ = two_doubles(-fourpi * std::sin(mu * phi));
     }
+    for (int n = 0; n <= p; ++n) *out++ = dd{std::pow(sc, n), 0.0};
+    for (int n = 0; n <= p; ++n) *out++ = dd{std::pow(sp, n), 0.0};
 }
 
 void translation_matrix(int p, zc kk, const double t[3], const std::vector<int64_t> &off,

@@ -160,9 +160,12 @@ void bcoef_table(int p, int KMAX, std::vector<double> &B);
 void gtensor(int p, const std::vector<double> &Bcoef, int KM, zc k, zc kp, cd *dst);
 lmfmm_status classify_and_sort(lmfmm_ctx *ctx);
 void gaunt_table(int p, std::vector<int64_t> &off, std::vector<int> &lval, std::vector<double> &gval);
-void gaunt_nodes(int p, std::vector<double> &w, std::vector<double> &Pq);
-inline int trans_factor_count(int p) { return 2 * (2 * p + 1) + (2 * p + 1) * (2 * p + 2) / 2 + 2 * (4 * p + 1); }
-void trans_factors(int p, zc k, const double t[3], double *out);
+void gaunt_nodes(int p, std::vector<dd> &w, std::vector<dd> &Pq);
+inline int trans_factor_count(int p)
+{
+    return 2 * (2 * p + 1) + (2 * p + 1) * (2 * p + 2) / 2 + 2 * (4 * p + 1) + 2 * (p + 1);
+}
+void trans_factors(int p, zc k, const double t[3], double sc, double sp, dd *out);
 void translation_matrix(int p, zc k, const double t[3], const std::vector<int64_t> &off,
                         const std::vector<int> &lval, const std::vector<double> &gval, cd *up,
                         cd *dn);

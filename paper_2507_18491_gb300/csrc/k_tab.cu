@@ -244,16 +244,40 @@ cudaError_t configure_tab_kernels()
                                 160 * 1024);
 }
 // ---------------------------------------------------- translation matrices
+// Sums and products of double-doubles (Dekker, Numer. Math. 18 (1971); Knuth's two-sum):
+// some 100 bits, so that an entry below is rounded once, like the long double of the host's
+// translation_matrix.  In plain FP64 the quadrature and the sum over l left 5e-16 of a degree
+// block's largest entry instead of 1.1e-16.
+__device__ __forceinline__ dd dd_norm(double h, double l)   // |h| >= |l|
+{
+    const double s = h + l;
+    return dd{s, l - (s - h)};
+}
+
+__device__ __forceinline__ dd dd_add(dd a, dd b)
+{
+    const double s = a.h + b.h, t = s - a.h;
+    return dd_norm(s, ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l));
+}
+
+__device__ __forceinline__ dd dd_mul(dd a, dd b)
+{
+    const double q = a.h * b.h;
+    return dd_norm(q, fma(a.h, b.h, -q) + fma(a.h, b.l, a.l * b.h));
+}
+
+__device__ __forceinline__ dd dd_neg(dd a) { return dd{-a.h, -a.l}; }
+
 // Gaunt coefficients G(l; n', n) = int Y_l^(m-m') Y_n'^m' conj(Y_n^m) for l = |n - n'|,
 // |n - n'| + 2, ... (zero where l < |m - m'|), p + 1 per entry, by the Gauss-Legendre rule
-// that is exact for them.  One thread per entry: the quadrature is some 10^7 FP64 operations
+// that is exact for them.  One thread per coefficient: the quadrature is some 10^7 products
 // at p = 12, which took the host (whose long double is software there) a second.
-__global__ void k_gaunt(int p, int nq, const double *w, const double *Pq, double *G)
+__global__ void k_gaunt(int p, int nq, const dd *w, const dd *Pq, double *G)
 {
     const int P = (p + 1) * (p + 1), nt = (2 * p + 1) * (2 * p + 2) / 2;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= P * P) return;
-    const int r = e / P, c = e % P;
+    const int id = blockIdx.x * blockDim.x + threadIdx.x;
+    if (id >= P * P * (p + 1)) return;
+    const int e = id / (p + 1), j = id % (p + 1), r = e / P, c = e % P;
     int n = (int)sqrtf((float)r + 0.5f), n1 = (int)sqrtf((float)c + 0.5f);
     while ((n + 1) * (n + 1) <= r) ++n;
     while (n * n > r) --n;
@@ -263,23 +287,22 @@ __global__ void k_gaunt(int p, int nq, const double *w, const double *Pq, double
     const int am = abs(m), am1 = abs(m1), amu = abs(mu);
     // P~_n^m = (-1)^m P~_n^|m| for m < 0
     const int neg = ((m < 0 ? am : 0) + (m1 < 0 ? am1 : 0) + (mu < 0 ? amu : 0)) & 1;
-    for (int j = 0; j <= p; ++j) {
-        const int l = abs(n - n1) + 2 * j;
-        double s = 0.0;
-        if (l <= n + n1 && l >= amu) {
-            for (int q = 0; q < nq; ++q) {
-                const double *Q = Pq + (int64_t)q * nt;
-                s += w[q] * Q[l * (l + 1) / 2 + amu] * Q[n1 * (n1 + 1) / 2 + am1] * Q[n * (n + 1) / 2 + am];
-            }
+    const int l = abs(n - n1) + 2 * j;
+    dd s{0.0, 0.0};
+    if (l <= n + n1 && l >= amu) {
+        for (int q = 0; q < nq; ++q) {
+            const dd *Q = Pq + (int64_t)q * nt;
+            s = dd_add(s, dd_mul(dd_mul(w[q], Q[l * (l + 1) / 2 + amu]),
+                                 dd_mul(Q[n1 * (n1 + 1) / 2 + am1], Q[n * (n + 1) / 2 + am])));
         }
-        G[(int64_t)e * (p + 1) + j] = neg ? -s : s;
     }
+    G[id] = neg ? -s.h : s.h;
 }
 
 // M2M = i^(n'-n) W(t) and L2L = i^(n-n') W(t) of every translation group, with the level
 // scaling M~ = M / s^n, L~ = L s^nu: W = sum_l i^l j_l(k |t|) P~_l^mu(t^) 4 pi e^{-i mu phi} G(l).
-// fac: trans_factors of the groups; sc: scales of the child and parent level
-__global__ void k_trans_build(int p, const double *G, const double *fac, int nfac, const double2 *sc, cd *up, cd *dn)
+// fac: trans_factors of the groups
+__global__ void k_trans_build(int p, const double *G, const dd *fac, int nfac, cd *up, cd *dn)
 {
     const int P = (p + 1) * (p + 1);
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -292,30 +315,23 @@ __global__ void k_trans_build(int p, const double *G, const double *fac, int nfa
     while ((n1 + 1) * (n1 + 1) <= c) ++n1;
     while (n1 * n1 > c) --n1;
     const int mu = (r - n * n - n) - (c - n1 * n1 - n1), amu = abs(mu);
-    const double *jl = fac + g * nfac, *Pt = jl + 2 * (2 * p + 1), *ep = Pt + (2 * p + 1) * (2 * p + 2) / 2;
-    cd s{0.0, 0.0};
+    const dd *jl = fac + g * nfac, *Pt = jl + 2 * (2 * p + 1), *ep = Pt + (2 * p + 1) * (2 * p + 2) / 2;
+    const dd *sc = ep + 2 * (4 * p + 1), *sp = sc + (p + 1);   // powers of the child and the parent scale
+    dd sx{0.0, 0.0}, sy{0.0, 0.0};
     for (int j = 0; j <= p; ++j) {
         const int l = abs(n - n1) + 2 * j;
         if (l > n + n1) break;
         if (l < amu) continue;
-        const double f = Pt[l * (l + 1) / 2 + amu] * G[(int64_t)e * (p + 1) + j];
-        s.x = fma(f, jl[2 * l], s.x);
-        s.y = fma(f, jl[2 * l + 1], s.y);
+        const dd f = dd_mul(Pt[l * (l + 1) / 2 + amu], dd{G[(int64_t)e * (p + 1) + j], 0.0});
+        sx = dd_add(sx, dd_mul(f, jl[2 * l]));
+        sy = dd_add(sy, dd_mul(f, jl[2 * l + 1]));
     }
+    const dd ex = ep[2 * (mu + 2 * p)], ey = ep[2 * (mu + 2 * p) + 1];
+    cd s{dd_add(dd_mul(sx, ex), dd_neg(dd_mul(sy, ey))).h, dd_add(dd_mul(sx, ey), dd_mul(sy, ex)).h};
     if (mu < 0 && (amu & 1)) s = -s;
-    s = s * cd{ep[2 * (mu + 2 * p)], ep[2 * (mu + 2 * p) + 1]};
-    double pc = 1.0, pr = 1.0, qc = 1.0, qr = 1.0;   // child, parent scale to the column's / row's degree
-    for (int i = 0; i < n1; ++i) {
-        pc *= sc[g].x;
-        qc *= sc[g].y;
-    }
-    for (int i = 0; i < n; ++i) {
-        pr *= sc[g].y;
-        qr *= sc[g].x;
-    }
     const int64_t o = g * P * P + e;
-    up[o] = (pc / pr) * (ipow<double>(n1 - n) * s);
-    dn[o] = (qr / qc) * (ipow<double>(n - n1) * s);
+    up[o] = (sc[n1].h / sp[n].h) * (ipow<double>(n1 - n) * s);
+    dn[o] = (sc[n].h / sp[n1].h) * (ipow<double>(n - n1) * s);
 }
 
 // out = in (T != double: rounded once), transposed per matrix if tr
@@ -329,12 +345,12 @@ __global__ void k_trans_copy(int P, int tr, const cd *in, cx<T> *out)
     out[g + e] = cx<T>{(T)v.x, (T)v.y};
 }
 
-void launch_trans_build(int p, int nq, const double *w, const double *Pq, double *G, int64_t ng, const double *fac,
-                        const double2 *sc, cd *up, cd *dn, cudaStream_t st)
+void launch_trans_build(int p, int nq, const dd *w, const dd *Pq, double *G, int64_t ng, const dd *fac, cd *up, cd *dn,
+                        cudaStream_t st)
 {
     const int P = (p + 1) * (p + 1), nb = (P * P + 127) / 128;
-    k_gaunt<<<nb, 128, 0, st>>>(p, nq, w, Pq, G);
-    if (ng > 0) k_trans_build<<<dim3(nb, (unsigned)ng), 128, 0, st>>>(p, G, fac, trans_factor_count(p), sc, up, dn);
+    k_gaunt<<<(P * P * (p + 1) + 127) / 128, 128, 0, st>>>(p, nq, w, Pq, G);
+    if (ng > 0) k_trans_build<<<dim3(nb, (unsigned)ng), 128, 0, st>>>(p, G, fac, trans_factor_count(p), up, dn);
 }
 
 template <typename T>

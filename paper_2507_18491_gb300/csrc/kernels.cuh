@@ -86,9 +86,9 @@ void launch_tab_batch(const GeomDev *dG, int g0, int nb, int qmax, const MediumD
 
 // translation matrices of ng groups on the device: the Gaunt coefficients (G: P^2 (p + 1)
 // doubles) from the nodes of gaunt_nodes, then M2M (up) and L2L (dn), [group][P][P]; fac
-// from trans_factors, sc the scales of the child and parent level
-void launch_trans_build(int p, int nq, const double *w, const double *Pq, double *G, int64_t ng, const double *fac,
-                        const double2 *sc, cd *up, cd *dn, cudaStream_t st);
+// from trans_factors
+void launch_trans_build(int p, int nq, const dd *w, const dd *Pq, double *G, int64_t ng, const dd *fac, cd *up, cd *dn,
+                        cudaStream_t st);
 template <typename T>
 void launch_trans_copy(int p, int64_t ng, bool tr, const cd *in, cx<T> *out, cudaStream_t st);
 

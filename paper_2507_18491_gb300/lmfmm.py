@@ -69,7 +69,7 @@ EXPORTS = ["lmfmm_default_params", "lmfmm_create", "lmfmm_set_layers", "lmfmm_se
            "lmfmm_set_points_device", "lmfmm_build", "lmfmm_matvec", "lmfmm_matvec_host",
            "lmfmm_matvec_adjoint", "lmfmm_matvec_transpose", "lmfmm_gradient", "lmfmm_check", "lmfmm_test_set_status", "lmfmm_test_fail_m2l",
            "lmfmm_direct",
-           "lmfmm_direct_noalloc", "lmfmm_densities", "lmfmm_m2l_table", "lmfmm_translation_matrix",
+           "lmfmm_direct_noalloc", "lmfmm_densities", "lmfmm_m2l_table", "lmfmm_translation_matrix", "lmfmm_built_translation",
            "lmfmm_free_m2l_table", "lmfmm_legendre_chebyshev", "lmfmm_legendre_product",
            "lmfmm_get_stats", "lmfmm_plan_check", "lmfmm_plan_depth", "lmfmm_last_error", "lmfmm_destroy", "lmfmm_batch_create",
            "lmfmm_batch_matvec", "lmfmm_batch_tune", "lmfmm_batch_check", "lmfmm_batch_info",
@@ -117,6 +117,7 @@ def load():
         "lmfmm_densities": [P, i, i, i64, P, P, P],
         "lmfmm_m2l_table": [P, i, i, i, i, d, d, d, P, P],
         "lmfmm_translation_matrix": [i, _Complex128, ctypes.POINTER(d), P, P],
+        "lmfmm_built_translation": [P, i64, ctypes.POINTER(i), P, P, P, P],
         "lmfmm_free_m2l_table": [i, _Complex128, d, d, P, P],
         "lmfmm_get_stats": [P, ctypes.POINTER(Stats)],
         "lmfmm_legendre_chebyshev": [i, P],
@@ -312,6 +313,21 @@ def translation_matrix(p, k, t):
                                            ctypes.c_void_p(up.ctypes.data),
                                            ctypes.c_void_p(dn.ctypes.data)))
     return up, dn
+
+
+def built_translation(ctx, p, group):
+    """(layer, t, (child scale, parent scale), m2m, l2l) of a translation group of a built FP64
+    operator, or None past the last group."""
+    P = (p + 1) ** 2
+    layer = ctypes.c_int()
+    t, sc = np.empty(3), np.empty(2)
+    up, dn = np.empty((P, P), np.complex128), np.empty((P, P), np.complex128)
+    rc = load().lmfmm_built_translation(ctx, group, ctypes.byref(layer), t.ctypes.data, sc.ctypes.data,
+                                        up.ctypes.data, dn.ctypes.data)
+    if rc == ERR_ARG:
+        return None
+    _check(rc, ctx)
+    return layer.value, t, sc, up, dn
 
 
 def free_m2l_table(p, k, rho, dz, blocks=False):
