@@ -507,9 +507,8 @@ static __device__ inline void bessel_012(int kind, cd z, cd &J0, cd &J1, cd &J2)
         J2 = 0.5 * H[2];
         return;
     }
-    // near pairs are close: most arguments are small, and Miller's recurrence takes some 40
-    // steps of a dozen operations for them
-    if (abs2(z) < 16.0) {
+    // near pairs are close: most arguments are small
+    if (bessel_series_holds(z)) {
         cd J[3];
         bessel_j_series<2>(z, J);
         J0 = J[0];
@@ -517,6 +516,8 @@ static __device__ inline void bessel_012(int kind, cd z, cd &J0, cd &J1, cd &J2)
         J2 = J[2];
         return;
     }
+    // real: CUDA's own, a third to a half of the recurrence's error from here on (3-4: J_0, J_2
+    // 0.6e-16 against 1.1e-16, 1.3e-16)
     if (z.y == 0.0) {
         double x = z.x;
         double j0v = j0(x), j1v = j1(x);

@@ -197,7 +197,7 @@ __global__ void k_s2t_pre_grad(const NearPair *near, const BoxDev *boxes, const 
                 if (s_kind[q] != 0) {
                     hankel1_seq(s_kind[q] == 2 ? conj(z) : z, 3, J);
                     for (int u = 0; u < 4; ++u) J[u] = 0.5 * (s_kind[q] == 2 ? conj(J[u]) : J[u]);
-                } else if (abs2(z) < 16.0) {
+                } else if (bessel_series_holds(z)) {
                     bessel_j_series<3>(z, J);
                 } else {
                     bessel_j_seq<4>(z, 3, J);
