@@ -846,7 +846,7 @@ __global__ void __launch_bounds__(128) k_p2p_free(int64_t N, const int *pt_box, 
         pos += 32;
         if (jc == ir) continue;
         const double Rx = xr - xyz[3 * jc], Ry = yr - xyz[3 * jc + 1], Rz = zr - xyz[3 * jc + 2];
-        const double R2 = Rx * Rx + Ry * Ry + Rz * Rz, iR = rsqrt(R2), R = R2 * iR, iR2 = iR * iR;
+        const double R2 = Rx * Rx + Ry * Ry + Rz * Rz, iR = rsqrt(R2), R = sqrt_from_rsqrt(R2, iR), iR2 = iR * iR;
         double s, c;
         sincos(k.x * R, &s, &c);
         double e = (0.25 / LMF_PI) * iR;

@@ -78,6 +78,14 @@ __device__ inline void hankel1_seq(cd z, int D, cd *H)
     for (int n = 1; n < D; ++n) H[n + 1] = (double)n * iz2 * H[n] - H[n - 1];
 }
 
+// sqrt(x) from y ~ 1 / sqrt(x) (an ulp off): x y is up to two ulps off, one Newton step from it
+// rounds like sqrt itself but for rare ties, in four operations
+__device__ inline double sqrt_from_rsqrt(double x, double y)
+{
+    const double r = x * y;
+    return fma(fma(-r, r, x), 0.5 * y, r);
+}
+
 // Where the power series below is no less accurate than Miller's recurrence (which takes some 40
 // steps of a dozen operations): |z| < 3 on the real axis, |z| < 2 off it.  J_0, rms error over
 // 400 points of an annulus, series / recurrence, GB300: real 0-1 0.8e-16 / 1.2e-16, 2-3 0.5e-16 /

@@ -12,8 +12,13 @@ CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
 HARNESS = r"""
 #include <cstdio>
 #include "specfun.cuh"
-int main()
+int main(int argc, char **)
 {
+    double x[2];
+    while (argc > 1 && std::fread(x, sizeof x, 1, stdin) == 1) {
+        const double r = sqrt_from_rsqrt(x[0], x[1]);
+        std::fwrite(&r, sizeof r, 1, stdout);
+    }
     cd z;
     while (std::fread(&z, sizeof z, 1, stdin) == 1) {
         cd S[4], M[5], h{bessel_series_holds(z) ? 1.0 : 0.0, 0.0};
@@ -65,3 +70,17 @@ def test_series_is_no_less_accurate_than_the_recurrence_where_it_runs(harness, l
     rms = np.sqrt((err ** 2).mean(1))
     # of 300 errors each: an rms is known to 1 / sqrt(2 x 300) = 4%, a ratio to 6%; two of these
     assert (rms[0] < 1.12 * rms[1]).all(), rms
+
+
+def test_distance_from_its_reciprocal_root(harness):
+    """The near field forms R from rsqrt(R^2), which CUDA gives to an ulp: R rounded like sqrt, but
+    for values next to a tie (2^-53 of an ulp's width in the correction's own rounding: rare)."""
+    rng = np.random.default_rng(4)
+    x = np.exp(rng.uniform(-20, 20, 20000))
+    y = 1 / np.sqrt(x)
+    y = np.where(rng.random(x.size) < 0.5, np.nextafter(y, 0), np.nextafter(y, np.inf))
+    out = subprocess.run([harness, "r"], input=np.stack([x, y], 1).tobytes(), stdout=subprocess.PIPE, check=True).stdout
+    r = np.frombuffer(out)
+    assert (np.abs(x * y - np.sqrt(x)) > 0).mean() > 0.3      # without the step
+    assert (r != np.sqrt(x)).mean() < 0.01
+    assert (np.abs(r - np.sqrt(x)) <= np.spacing(np.sqrt(x))).all()
