@@ -13,9 +13,15 @@
 // bits below an FP64 rounding.  The eight sums are put together as 64-bit integers and
 // converted once.
 //
-// Grids: the matrix rows carry their own power of two; the inputs carry one per
-// source box, after the degrees have been brought to one size by 2^c_n ~ (2n + 1)!! (the
-// scaled expansions fall like 1/(2n + 1)!!, the matrix columns grow like it and take 2^-c_n).
+// Grids: the matrix rows carry their own power of two, the inputs one per pair, after the
+// degrees have been brought to one size by 2^(c_n + a_n), which the matrix columns take out:
+// 2^c_n ~ (2n + 1)!! and 2^a_n ~ (S / r)^n, S the cell size, r the largest radius of the
+// geometry's source boxes.  The scaled expansions fall like (r / S)^n / (2n + 1)!!, the columns grow like
+// (S / R)^n (2n + 1)!!, R the distance of the centres, which admissibility bounds by the
+// radii alone: where the points lie far inside their cells, R may be far below S (a cell's centre
+// next to an interface), and without a_n the grid of a row went to columns whose inputs are tiny
+// (r = S / 200, R = S / 25, p = 12: 46% of the result).  With it the products of a row are within
+// max_n C(n + nu, n) (r / R)^n of the row's and the inputs' largest entries.
 //
 // One CTA per SM walks the work items (up to 64 pairs of one geometry).  Per sector: all
 // threads form the inputs (FP64 phases, digits by integer operations) into a per-CTA image
@@ -53,7 +59,7 @@ constexpr int OZ_PMAX = 16;
 struct OzPlan {
     int p, P, D[2], nk[2], rows;   // rows: D0 + D1
     uint32_t sec_img[2], img_bytes;
-    uint32_t o_ph, o_ent, o_pair, o_bars, smem, ph_bytes, stage_bytes;
+    uint32_t o_ph, o_ent, o_adj, o_pair, o_exp, o_bars, smem, ph_bytes, stage_bytes;
     int out_warps;
 };
 
@@ -81,8 +87,10 @@ OzPlan oz_plan(int p)
     s.stage_bytes = (uint32_t)(3 * s.P) * 16;
     s.o_ph = OZ_ST * OZ_SLOT;
     s.o_ent = s.o_ph + OZ_BN * s.ph_bytes;
-    s.o_pair = (s.o_ent + (uint32_t)s.nk[0] * 8 * 4 + 15) & ~15u;
-    s.o_bars = s.o_pair + OZ_BN * (uint32_t)sizeof(M2LPair);
+    s.o_adj = s.o_ent + (uint32_t)s.nk[0] * 8 * 4;
+    s.o_pair = (s.o_adj + (uint32_t)s.nk[0] * 8 * 4 + 15) & ~15u;
+    s.o_exp = s.o_pair + OZ_BN * (uint32_t)sizeof(M2LPair);
+    s.o_bars = s.o_exp + OZ_BN * 4 + (OZ_PMAX + 1 + 3) * 4;
     s.smem = s.o_bars + (2 * OZ_ST + 2) * 8 + 16;
     s.out_warps = std::min<int>(OZ_W, (OZ_ST * OZ_SLOT) / s.stage_bytes);
     return s;
@@ -98,19 +106,25 @@ __host__ __device__ inline int oz_cn(int n)
     return e - 1;
 }
 
+// ... and of the points' radius against the cell, lg = log2(S / r)
+__host__ __device__ inline int oz_an(int n, float lg) { return (int)rintf((float)n * lg); }
+
+constexpr int OZ_ZERO = -(1 << 14), OZ_BAD = 1 << 14;   // exponents of a degree of zeros, of one that is not finite
+
 struct __align__(16) OzIn {        // one input: its two coefficients
     double x, y, z, w;
 };
 
-// the eight digits of x, |x| < 1 - 2^-8 (the first digit would leave a byte beyond): x = sum_j s_j 2^(-7 - 8 j), s_j in [-128, 127], as floats'
-// upper halves (bf16, exact).  The fixed-point number comes from the bits of x; adding 128
-// to every digit but the first makes the bytes of the sum the digits plus 128.
-__device__ __forceinline__ void oz_digits(double x, uint32_t (&w)[OZ_S])
+// the eight digits of x 2^adj, below 1 - 2^-8 in size (the first digit would leave a byte beyond):
+// sum_j s_j 2^(-7 - 8 j), s_j in [-128, 127], as floats' upper halves (bf16, exact).  The
+// fixed-point number comes from the bits of x; adding 128 to every digit but the first makes the
+// bytes of the sum the digits plus 128.
+__device__ __forceinline__ void oz_digits(double x, int adj, uint32_t (&w)[OZ_S])
 {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const int ex = (int)(u >> 52) & 0x7ff;
     const unsigned long long man = (u & 0xfffffffffffffull) | (ex ? 1ull << 52 : 0ull);
-    const int sh = ex - 1012;                       // x 2^63 = man 2^sh
+    const int sh = max(ex, 1) - 1012 + adj;         // x 2^adj 2^63 = man 2^sh
     long long q = sh >= 0 ? (long long)(man << (sh > 10 ? 10 : sh)) : (long long)(sh > -64 ? man >> -sh : 0ull);
     if (u >> 63) q = -q;
     const unsigned long long t = (unsigned long long)q + 0x8080808080808080ull;   // first digit too: its byte is signed + 128
@@ -154,13 +168,15 @@ __device__ __forceinline__ double2 lds_d2(uint32_t a)
 // transposed: the same walk with the matrices transposed, the phases conjugated and the roles
 // of the pair's boxes exchanged (in: local, out: multipole expansions)
 __global__ void __launch_bounds__(OZ_T, 1)
-    k_m2l_oz(const __grid_constant__ OzPlan sp, int transposed, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
-             const unsigned char *img, const double *rscale, const OzIn *packed, const double *bscale, cd *out,
-             unsigned char *xscr, double *yscr, int *status)
+    k_m2l_oz(const __grid_constant__ OzPlan sp, int transposed, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
+             const M2LPair *pairs, const unsigned char *img, const double *rscale, const OzIn *packed, const int *bexp,
+             cd *out, unsigned char *xscr, double *yscr, int *status)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     const int p = sp.p, P = sp.P, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t *ent = (uint32_t *)(smraw + sp.o_ent);
+    // exponents per input, per pair, per degree
+    int *adj = (int *)(smraw + sp.o_adj), *pexp = (int *)(smraw + sp.o_exp), *cn = pexp + OZ_BN;
     M2LPair *pr = (M2LPair *)(smraw + sp.o_pair);
     uint64_t *full = (uint64_t *)(smraw + sp.o_bars), *empty = full + OZ_ST, *accfull = empty + OZ_ST;
     uint32_t *tslot = (uint32_t *)(accfull + 1);
@@ -179,6 +195,7 @@ __global__ void __launch_bounds__(OZ_T, 1)
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     for (int j = tid; j < D0e; j += OZ_T) ent[j] = j < sp.D[0] ? sec_word(p, j) : 0u;
+    if (tid <= p) cn[tid] = oz_cn(tid);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -189,10 +206,24 @@ __global__ void __launch_bounds__(OZ_T, 1)
 
     for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x) {
         const M2LWork w = work[it];
+        const float lg = transposed ? geoms[w.geom].lg_t : geoms[w.geom].lg_s;
+        // the inputs' exponents: adj takes the degrees to one size, pexp the pair below 2^-2 (two
+        // coefficients of parts below 2^(pexp - adj): below 2^(pexp + 1.5) each part)
+        for (int j = tid; j < D0e; j += OZ_T) {
+            const int n = j < sp.D[0] ? sec_entry(p, j).n : 0;
+            adj[j] = cn[n] + oz_an(n, lg);
+        }
         // pair records and phases G[d] (conjugated for the transpose), d = -(p+1)..p
         if (tid < w.npair) {
             const M2LPair q = pairs[w.pair0 + tid];
             pr[tid] = q;
+            const int *be = bexp + (transposed ? q.tgt : q.src) * (p + 1);
+            int top = OZ_ZERO;
+            for (int n = 0; n <= p; ++n) {
+                const int e = be[n];
+                if (e != OZ_ZERO) top = max(top, e == OZ_BAD ? OZ_BAD : e + cn[n] + oz_an(n, lg));
+            }
+            pexp[tid] = top == OZ_ZERO ? 0 : top == OZ_BAD ? OZ_BAD : top + 2;
             cd b = mul_i(cd{q.cphi, q.sphi}), e{1.0, 0.0};
             if (transposed) b = conj(b);
             double2 *row = (double2 *)(smraw + sp.o_ph + tid * sp.ph_bytes) + (p + 1);
@@ -211,6 +242,8 @@ __global__ void __launch_bounds__(OZ_T, 1)
                 uint32_t rr[OZ_S][4], ri[OZ_S][4];                    // rows 2c and 2c + 1, one word per input
                 const int64_t box = c < w.npair ? (transposed ? pr[c].tgt : pr[c].src) : 0;
                 const OzIn *src = packed + box * D0e + 4 * hk;
+                const int4 ad = *(const int4 *)(adj + 4 * hk);
+                const int pe = c < w.npair ? pexp[c] : 0;
 #pragma unroll
                 for (int h = 0; h < 4; ++h) {
                     cd y{0.0, 0.0};
@@ -226,8 +259,9 @@ __global__ void __launch_bounds__(OZ_T, 1)
                         y.y = fma(G.x, v.y + by, G.y * (v.x - bx));
                     }
                     uint32_t wr[OZ_S], wi[OZ_S];
-                    oz_digits(y.x, wr);
-                    oz_digits(y.y, wi);
+                    const int sc = (h == 0 ? ad.x : h == 1 ? ad.y : h == 2 ? ad.z : ad.w) - pe;
+                    oz_digits(y.x, sc, wr);
+                    oz_digits(y.y, sc, wi);
 #pragma unroll
                     for (int j = 0; j < OZ_S; ++j) {
                         rr[j][h] = __byte_perm(wr[j], wi[j] ^ 0x80000000u, 0x7632);   // (Re, -Im)
@@ -315,11 +349,11 @@ __global__ void __launch_bounds__(OZ_T, 1)
             }
         }
         if (failed) break;
-        // ---- outputs: the phases take the source box's power of two
+        // ---- outputs: the phases take the pair's power of two (not a number where an input is none)
         for (int e = tid; e < w.npair * (2 * p + 2); e += OZ_T) {
             const int c = e / (2 * p + 2), d = e - c * (2 * p + 2);
             double2 *G = (double2 *)(smraw + sp.o_ph + c * sp.ph_bytes) + d;
-            const double f = bscale[transposed ? pr[c].tgt : pr[c].src];
+            const double f = pexp[c] == OZ_BAD ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, pexp[c]);
             *G = double2{f * G->x, f * G->y};
         }
         __syncthreads();
@@ -395,6 +429,7 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
     const bool fi = (cp.s < 0) != (cp.has_src_refl != 0), fo = (cp.s < 0) != (cp.has_tgt_refl != 0);
     const cd *tab = tab64 + gi * NTAB * (int64_t)sp.P * sp.P;
     const SecEntry er = sec_entry(sp.p, r);
+    const float lg = transposed ? gm.lg_t : gm.lg_s;
     auto value = [&](int k) {
         const SecEntry ek = sec_entry(sp.p, k);
         cd v;
@@ -405,7 +440,7 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
             if (er.c && er.m == 0) v = 2.0 * v;
             if (ek.c && ek.m == 0) v = 0.5 * v;
         }
-        const double f = ldexp(1.0, -cn[ek.n]);
+        const double f = ldexp(1.0, -cn[ek.n] - oz_an(ek.n, lg));
         return f * v;
     };
     double mx = 0.0;
@@ -430,52 +465,45 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
         cd v{0.0, 0.0};
         if (k < D) v = f * value(k);
         uint32_t wr[OZ_S], wi[OZ_S];
-        oz_digits(v.x, wr);
-        oz_digits(v.y, wi);
+        oz_digits(v.x, 0, wr);
+        oz_digits(v.y, 0, wi);
         unsigned char *q = o + (size_t)(k >> 3) * (OZ_S * N * 32) + ((k & 7) >> 2) * 128 + (k & 3) * 4;
 #pragma unroll
         for (int j = 0; j < OZ_S; ++j) *(uint32_t *)(q + (size_t)j * N * 32) = __byte_perm(wr[j], wi[j], 0x7632);
     }
 }
 
-// packed inputs of every box: entry j's two coefficients, scaled by 2^c_n and by the box's
-// power of two so that the sum of two of them is below 1 in size (bscale: the power taken
-// out, NaN where a coefficient is not finite); clears the box's output expansion
-__global__ void __launch_bounds__(128) k_oz_pack(int p, int n8, int D0, const cd *in, OzIn *pk, double *bscale,
-                                                 cd *out)
+// packed inputs of every box: entry j's two coefficients side by side, and per degree the
+// exponent e of its largest part, |part| < 2^e; clears the box's output expansion
+__global__ void __launch_bounds__(128) k_oz_pack(int p, int n8, int D0, const cd *in, OzIn *pk, int *bexp, cd *out)
 {
-    __shared__ int emax[4], cn[OZ_PMAX + 1];
+    __shared__ int top[OZ_PMAX + 1];
     const int P = (p + 1) * (p + 1), P3 = 3 * P;
     const int64_t box = blockIdx.x;
     const cd *m = in + box * P3;
-    if (threadIdx.x <= p) cn[threadIdx.x] = oz_cn(threadIdx.x);
+    if (threadIdx.x <= p) top[threadIdx.x] = OZ_ZERO;
     __syncthreads();
-    int e = -4096;                              // exponent field of the largest scaled part
     for (int j = threadIdx.x; j < P3; j += blockDim.x) {
         const cd v = m[j];
         const int ex = max((int)(__double_as_longlong(v.x) >> 52) & 0x7ff, (int)(__double_as_longlong(v.y) >> 52) & 0x7ff);
-        if (ex == 0x7ff) e = 8192;
-        else if (ex > 0) e = max(e, ex - 1022 + cn[sec_entry(p, j % P).n]);   // |v| 2^c_n < 2^e
+        int n = (int)sqrtf((float)(j % P) + 0.5f);
+        while ((n + 1) * (n + 1) <= j % P) ++n;
+        while (n * n > j % P) --n;
+        if (ex == 0x7ff) atomicMax(&top[n], OZ_BAD);
+        else if (v.x != 0.0 || v.y != 0.0) atomicMax(&top[n], max(ex, 1) - 1022);
         out[box * P3 + j] = cd{0.0, 0.0};
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
-    if ((threadIdx.x & 31) == 0) emax[threadIdx.x >> 5] = e;
-    __syncthreads();
-    e = max(max(emax[0], emax[1]), max(emax[2], emax[3]));
-    const bool bad = e >= 8192, zero = e == -4096;
-    const int sh = (bad || zero) ? 0 : e + 2;   // two coefficients of parts below 2^e: below 2^(e + 1.5) each part
-    if (threadIdx.x == 0) bscale[box] = bad ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, sh);
     for (int j = threadIdx.x; j < n8; j += blockDim.x) {
         OzIn v{0.0, 0.0, 0.0, 0.0};
-        if (j < D0 && !bad) {
+        if (j < D0) {
             const uint32_t w = sec_word(p, j);
             const cd a = m[w & 1023], b = m[(w >> 10) & 1023];
-            const int k = cn[sec_entry(p, j).n] - sh;
-            v = OzIn{ldexp(a.x, k), ldexp(a.y, k), ldexp(b.x, k), ldexp(b.y, k)};
+            v = OzIn{a.x, a.y, b.x, b.y};
         }
         pk[box * n8 + j] = v;
     }
+    __syncthreads();
+    if (threadIdx.x <= p) bexp[box * (p + 1) + threadIdx.x] = top[threadIdx.x];
 }
 
 }  // namespace
@@ -487,7 +515,7 @@ size_t m2l_oz_image_bytes(int p, int64_t ngeom)
     const OzPlan sp = oz_plan(p);
     return (size_t)ngeom * (sp.img_bytes + (size_t)sp.rows * sizeof(double));
 }
-size_t m2l_oz_packed_bytes(int p, int64_t nbox) { return (size_t)nbox * (oz_plan(p).nk[0] * 8 * sizeof(OzIn) + sizeof(double)); }
+size_t m2l_oz_packed_bytes(int p, int64_t nbox) { return (size_t)nbox * (oz_plan(p).nk[0] * 8 * sizeof(OzIn) + (p + 1) * sizeof(int)); }
 size_t m2l_oz_scratch_bytes(int p, int ncta)
 {
     const OzPlan sp = oz_plan(p);
@@ -508,20 +536,20 @@ void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, c
     }
 }
 
-cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
-                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
+cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
+                          const M2LPair *pairs, const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
                           int *status, cudaStream_t st)
 {
     if (!m2l_oz_supported(p) || ncta < 1) return cudaErrorInvalidValue;
     const OzPlan sp = oz_plan(p);
     const int n8 = sp.nk[0] * 8;
-    double *bs = (double *)((unsigned char *)packed + (size_t)nbox * n8 * sizeof(OzIn));
-    if (nbox > 0) k_oz_pack<<<(unsigned)nbox, 128, 0, st>>>(p, n8, sp.D[0], in, (OzIn *)packed, bs, out);
+    int *be = (int *)((unsigned char *)packed + (size_t)nbox * n8 * sizeof(OzIn));
+    if (nbox > 0) k_oz_pack<<<(unsigned)nbox, 128, 0, st>>>(p, n8, sp.D[0], in, (OzIn *)packed, be, out);
     if (nwork <= 0) return cudaGetLastError();
     unsigned char *x = (unsigned char *)scratch;
     k_m2l_oz<<<(unsigned)std::min<int64_t>(nwork, ncta), OZ_T, std::max<size_t>(sp.smem, 116 * 1024), st>>>(
-        sp, transposed ? 1 : 0, nwork, work, pairs, (const unsigned char *)img,
-        (const double *)((const unsigned char *)img + (size_t)ngeom * sp.img_bytes), (const OzIn *)packed, bs, out, x,
+        sp, transposed ? 1 : 0, nwork, work, geoms, pairs, (const unsigned char *)img,
+        (const double *)((const unsigned char *)img + (size_t)ngeom * sp.img_bytes), (const OzIn *)packed, be, out, x,
         (double *)(x + (size_t)ncta * sp.nk[0] * OZ_A), status);
     return cudaGetLastError();
 }

@@ -29,3 +29,40 @@ def test_digits_against_simt(p):
         op.close()
     for a, b in zip(*out):
         assert (a - b).norm() < 1e-13 * b.norm()
+
+
+def _near_centre(height, spread, k):
+    """Points within `spread` of the centre of a cell of side 1 that lies `height` above an interface,
+    and points elsewhere that span the root cell [-1, 1]^3: the image of the cell's centre is 2 height
+    away, a small part of the cell's side, and still far from the points by their radius."""
+    rng = np.random.default_rng(9)
+    near = 0.5 + spread * rng.uniform(-1, 1, (12, 3))
+    wide = np.array([[1, -1, -1], [-1, 1, -1], [-1, -1, 1], [-1, -1, -1]], float) * (1 - 1e-9)
+    below = np.array([0.5, 0.5, 0.5 - 2 * height]) + spread * rng.uniform(-1, 1, (12, 3))
+    xyz = np.concatenate([near, wide, below])
+    J = rng.standard_normal(xyz.shape) + 1j * rng.standard_normal(xyz.shape)
+    return [0.5 - height], k, xyz, J
+
+
+# the tables' entries grow like (side / distance)^(n + nu), the expansions fall like
+# (radius / side)^n: the products are of ordinary size, but a grid set by each side's own largest
+# entry has no bits left for them (46% of the result at p = 12, height 0.02).  Forward and
+# transposed; 1e-13 as above
+@pytest.mark.parametrize("p,height,spread", [(8, 0.1, 0.01), (12, 0.1, 0.01), (16, 0.1, 0.01), (12, 0.02, 0.002),
+                                             (16, 0.02, 0.002)])
+def test_expansions_far_inside_their_cells(p, height, spread):
+    d, k, xyz, J = _near_centre(height, spread, [1.3 + 0.01j, 2.1 + 0.02j])
+    Jt = torch.from_numpy(J).cuda()
+    out = []
+    for tc in (1, 0):
+        op = lmfmm.Operator(d, k, xyz, p=p, depth=1, theta=0.5, tensor_cores=tc).build()
+        assert op.stats()["m2l_digits"] == tc
+        out.append((op.matvec(Jt), op.tmatvec(Jt)))
+        ref = op.direct(Jt)
+        op.close()
+    for a, b in zip(*out):
+        print("p %d height %g: digits against SIMT %.2e" % (p, height, (a - b).norm() / b.norm()))
+    print("against the sum over all pairs: digits %.2e SIMT %.2e" %
+          ((out[0][0] - ref).norm() / ref.norm(), (out[1][0] - ref).norm() / ref.norm()))
+    for a, b in zip(*out):
+        assert (a - b).norm() < 1e-13 * b.norm()
