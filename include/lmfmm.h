@@ -355,8 +355,9 @@ lmfmm_status lmfmm_get_stats(const lmfmm_ctx *ctx, lmfmm_stats *out);
  * far box pairs and near leaf pairs (Sections 3.3 and 3.4.1; admissibility as in
  * lmfmm_params), the distinct M2L geometries and their pair lists, the
  * free-space lists when params->components asks for them (Section 2), the
- * M2M / L2L translation groups and the 64-column M2L work items of the
- * five-table kernels (the sector kernels cut the same pairs into runs of at most 64).  Checks:
+ * M2M / L2L translation groups, the 64-column M2L work items of the
+ * five-table kernels and the sector kernels' items (runs of at most 64, 32 and 16
+ * pairs).  Checks:
  *   tree       every layer's points are partitioned by the boxes of each level,
  *              children partition their parent, every point lies in its leaf's
  *              cell, box radii bound their points;
@@ -371,7 +372,7 @@ lmfmm_status lmfmm_get_stats(const lmfmm_ctx *ctx, lmfmm_stats *out);
  *              a kernel reads is in bounds, and pair ranges tile their arrays.
  * Arguments as lmfmm_create / lmfmm_set_layers / lmfmm_set_points (host xyz,
  * [N][3] double); flags: 0, or the test hooks below, which remove one pair
- * after the build so that a caller can see the check report it.  Coverage is
+ * (or the last sector item) after the build so that a caller can see the check report it.  Coverage is
  * checked per component and target leaf, as a tiling of the source leaves by
  * the intervals its ancestors' far pairs and its near pairs reach, while a
  * component has at most 2^25 such intervals (larger ones are counted in
@@ -379,7 +380,7 @@ lmfmm_status lmfmm_get_stats(const lmfmm_ctx *ctx, lmfmm_stats *out);
  * LMFMM_OK when every check holds, LMFMM_ERR_INTERNAL when one fails (the
  * count and the first failure are in *out), or the argument error of the
  * corresponding context call (message in out->message). */
-enum { LMFMM_PLAN_DROP_FAR_PAIR = 1, LMFMM_PLAN_DROP_NEAR_PAIR = 2 };
+enum { LMFMM_PLAN_DROP_FAR_PAIR = 1, LMFMM_PLAN_DROP_NEAR_PAIR = 2, LMFMM_PLAN_DROP_SECTOR_ITEM = 4 };
 
 typedef struct {
     int depth;                      /* leaf level */

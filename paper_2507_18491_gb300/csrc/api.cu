@@ -223,7 +223,7 @@ int64_t m2l_work_items(const lmfmm_ctx *ctx, int bn, int prob, std::vector<M2LWo
     return ncols;
 }
 
-// Work items of the sector kernel: per geometry, runs of at most `pairs` pairs.
+// Work items of the sector kernels: per geometry, runs of at most `pairs` pairs.
 void sec_work_items(const lmfmm_ctx *ctx, int pairs, int prob, std::vector<M2LWork> &mw)
 {
     for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
@@ -325,6 +325,8 @@ int64_t plan_work_items(const lmfmm_ctx *ctx, int bn, std::vector<M2LWork> &mw)
 {
     return m2l_work_items(ctx, bn, 0, mw);
 }
+
+void plan_sector_items(const lmfmm_ctx *ctx, int pairs, std::vector<M2LWork> &mw) { sec_work_items(ctx, pairs, 0, mw); }
 
 // read-only view of the device state for lmfmm_direct_noalloc (noalloc.cu)
 bool noalloc_state(lmfmm_ctx *ctx, const int64_t **perm, const BoxDev **boxes, const double **xyz,

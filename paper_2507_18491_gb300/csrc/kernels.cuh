@@ -156,6 +156,8 @@ int m2l_tc_cols();
 // M2L work items of a context whose host structures are built, cut to at most bn
 // helical columns, in the order the matvec launches them (api.cu)
 int64_t plan_work_items(const lmfmm_ctx *ctx, int bn, std::vector<M2LWork> &mw);
+// ... and those of the sector kernels, runs of at most `pairs` pairs of a geometry
+void plan_sector_items(const lmfmm_ctx *ctx, int pairs, std::vector<M2LWork> &mw);
 cudaError_t configure_m2l_tc();
 cudaError_t launch_m2l_tc(int p, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
                           const CompDev *comps, const M2LPair *pairs, const cf *tab, const cf *me,

@@ -416,6 +416,41 @@ void check_work(const lmfmm_ctx *ctx, Check &ck, int64_t &nitems, int64_t &ncols
     if (cols != ncols) ck.fail("work items hold %lld columns, the builder counted %lld", (ll)cols, (ll)ncols);
 }
 
+// items of the sector kernels, at every run length they are cut to (the FP64 form halves them twice at
+// most, a batch once): consecutive runs of each geometry's pairs, whose records, phases and boxes a
+// kernel reads at [pair0, pair0 + npair)
+void check_sector_work(const lmfmm_ctx *ctx, Check &ck, bool drop)
+{
+    static_assert(sizeof(M2LPair) % 16 == 0, "bulk copies of pair records");
+    for (int per : {m2l_sec_pairs(), m2l_sec_pairs() / 2, m2l_oz_pairs(), m2l_oz_pairs() / 2, m2l_oz_pairs() / 4}) {
+        std::vector<M2LWork> mw;
+        plan_sector_items(ctx, per, mw);
+        if (drop && !mw.empty()) mw.pop_back();
+        size_t w = 0;
+        int64_t end = 0;
+        for (size_t gi = 0; gi < ctx->geoms.size(); ++gi) {
+            const Geom &G = ctx->geoms[gi];
+            for (int64_t q = G.pair0; q < G.pair1;) {
+                if (w >= mw.size()) {
+                    ck.fail("sector items of %d pairs end before geometry %lld, pair %lld", per, (ll)gi, (ll)q);
+                    return;
+                }
+                const M2LWork &W = mw[w++];
+                if (W.geom != (int)gi || W.prob != 0 || W.pair0 != q || W.npair < 1 || W.npair > per ||
+                    W.pair0 + W.npair > G.pair1) {
+                    ck.fail("sector item %lld of %d pairs does not continue geometry %lld at pair %lld", (ll)(w - 1), per,
+                            (ll)gi, (ll)q);
+                    return;
+                }
+                q += W.npair;
+            }
+            end = std::max(end, G.pair1);
+        }
+        if (w != mw.size()) ck.fail("%lld sector items beyond the geometries", (ll)(mw.size() - w));
+        if (end != (int64_t)ctx->m2l.size()) ck.fail("geometries end at pair %lld of %lld", (ll)end, (ll)ctx->m2l.size());
+    }
+}
+
 }  // namespace
 
 extern "C" lmfmm_status lmfmm_plan_check(const lmfmm_params *prm, int L, const double *d, const lmfmm_c128 *k,
@@ -430,7 +465,7 @@ extern "C" lmfmm_status lmfmm_plan_check(const lmfmm_params *prm, int L, const d
     }
     if (prm->p < 1 || prm->p > 16 || !(prm->theta > 0 && prm->theta < 1) || !(prm->eta >= 0) || prm->depth > 20 ||
         (prm->depth < 0 && prm->leaf_cap < 1) || prm->components < LMFMM_REACTION || prm->components > LMFMM_TOTAL ||
-        (flags & ~(LMFMM_PLAN_DROP_FAR_PAIR | LMFMM_PLAN_DROP_NEAR_PAIR))) {
+        (flags & ~(LMFMM_PLAN_DROP_FAR_PAIR | LMFMM_PLAN_DROP_NEAR_PAIR | LMFMM_PLAN_DROP_SECTOR_ITEM))) {
         msg("plan_check: parameter out of range (1 <= p <= 16, 0 < theta < 1, eta >= 0, depth <= 20, "
             "components, flags)");
         return LMFMM_ERR_ARG;
@@ -508,6 +543,7 @@ extern "C" lmfmm_status lmfmm_plan_check(const lmfmm_params *prm, int L, const d
     // the coverage walk descends child links: only on a consistent tree
     if (tree_ok) check_coverage(ctx, ck, out->n_leaf_pairs_checked, out->n_components_unchecked);
     check_work(ctx, ck, out->n_work_items, out->n_columns);
+    check_sector_work(ctx, ck, (flags & LMFMM_PLAN_DROP_SECTOR_ITEM) != 0);
     out->n_violations = ck.n;
     if (ck.n) std::snprintf(out->message, sizeof out->message, "%s", ck.first);
     delete ctx;

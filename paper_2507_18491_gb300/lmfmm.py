@@ -18,7 +18,7 @@ _lib = None
 
 OK, ERR_ARG, ERR_CUDA, ERR_OOM, ERR_STATE, ERR_QUAD, ERR_UNSUPPORTED, ERR_TIMEOUT, ERR_INTERNAL = (
     0, -1, -2, -3, -4, -5, -6, -7, -8)
-PLAN_DROP_FAR_PAIR, PLAN_DROP_NEAR_PAIR = 1, 2
+PLAN_DROP_FAR_PAIR, PLAN_DROP_NEAR_PAIR, PLAN_DROP_SECTOR_ITEM = 1, 2, 4
 FP64, MIXED = 0, 1
 C128, C64 = 0, 1
 REACTION, FREE, TOTAL = 0, 1, 2

@@ -104,6 +104,16 @@ def test_a_missing_interaction_is_reported(flag):
     assert info["n_violations"] >= 1 and "reached 0 times" in info["message"]
 
 
+def test_a_missing_sector_item_is_reported():
+    """The items of the default M2L kernels are checked, not only the five-table ones'."""
+    w = W.two_layer_small(seed=1001)
+    opt = dict(p=6, depth=2, theta=0.4)
+    assert lmfmm.plan_check(w.d, w.k, w.xyz, **opt)[0] == lmfmm.OK
+    rc, info = lmfmm.plan_check(w.d, w.k, w.xyz, flags=lmfmm.PLAN_DROP_SECTOR_ITEM, **opt)
+    assert rc == lmfmm.ERR_INTERNAL
+    assert info["n_violations"] >= 1 and "sector items" in info["message"]
+
+
 def test_bad_arguments_are_rejected():
     w = W.two_layer_small(seed=1001)
     xyz = w.xyz.copy()
