@@ -247,7 +247,7 @@ lmfmm_status tabulate(lmfmm_ctx *ctx, std::vector<GeomDev> &hg, const CompDev *d
     const int p = ctx->prm.p;
     const int LM = p + 2, DJ = 2 * p + 3;
     const int64_t per_node = 5 + 4 + 4 + LM + DJ;
-    const int64_t ibr = (int64_t)NTAB * 4 * 4 * LM * DJ;
+    const int64_t ibr = tab_integrals(p);
     const size_t scratch_bytes = (size_t)1 << 30;
     // batches
     std::vector<int> bstart;

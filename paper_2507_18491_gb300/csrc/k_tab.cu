@@ -214,6 +214,9 @@ __global__ void k_tab_assemble(const GeomDev *G, int g0, const CompDev *comps, i
     tab[((int64_t)g.tab_index * NTAB + t) * P * P + e] = sgn * s;
 }
 
+// Chebyshev integrals of one geometry: [table][tau][tau'][l][h]
+int64_t tab_integrals(int p) { return (int64_t)NTAB * 16 * (p + 2) * tab_dh(2 * p + 3); }
+
 // One batch of geometries [g0, g0+nb): node factors, I-breve, I-hat.  The
 // scratch holds (5+4+4+LM+DJ) * stride node factors followed by nb I-breve
 // blocks; stride is the batch's total node count.
@@ -222,7 +225,7 @@ void launch_tab_batch(const GeomDev *dG, int g0, int nb, int qmax, const MediumD
                       cd *scratch, int64_t stride, cd *tab, int *dflag, cudaStream_t st)
 {
     const int LM = p + 2, DJ = 2 * p + 3, P = (p + 1) * (p + 1);
-    const int64_t ibr_stride = (int64_t)NTAB * 16 * LM * tab_dh(DJ);
+    const int64_t ibr_stride = tab_integrals(p);
     const int64_t S = stride;
     cd *Fb = scratch, *Fs = Fb + 5 * S, *Ft = Fs + 4 * S, *FT = Ft + 4 * S, *FJ = FT + LM * S;
     cd *Ibr = FJ + DJ * S;

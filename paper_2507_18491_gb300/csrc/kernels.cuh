@@ -81,6 +81,7 @@ struct TcProb {
 // k_tab.cu
 void launch_densities(const MediumDev &M, int l, int lp, int64_t n, const cd *kr, cd *out,
                       cudaStream_t st);
+int64_t tab_integrals(int p);   // complex numbers of scratch per geometry, beside the node factors
 void launch_tab_batch(const GeomDev *dG, int g0, int nb, int qmax, const MediumDev &M,
                       const CompDev *dcomps, int p, const cd *dGten, const int *dcgidx,
                       cd *scratch, int64_t stride, cd *tab, int *dflag, cudaStream_t st);
