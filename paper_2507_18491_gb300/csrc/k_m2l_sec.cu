@@ -389,15 +389,14 @@ __global__ void __launch_bounds__(SC_THREADS, 1)
             for (int t = 0; t < sp.ntile && !failed; ++t) {
                 const int odd = sp.t[t].sec, nch = sp.t[t].nchunk;
                 for (int ch = 0; ch < nch; ++ch) {
-                    // the stage that fetch fills was read by the whole warp in the last chunk; wait_group
-                    // covers a lane's own copies only, and the rows read below came with other lanes'
+                    // wait_group covers a lane's own copies only, and the rows read below came with other
+                    // lanes'; the stage that fetch fills was read by the whole warp in the last chunk
+                    asm volatile("cp.async.wait_group %0;" ::"n"(SC_XD - 2) : "memory");
                     __syncwarp();
                     if (!fetch()) {
                         failed = true;
                         break;
                     }
-                    asm volatile("cp.async.wait_group %0;" ::"n"(SC_XD - 1) : "memory");
-                    __syncwarp();
                     const bool okw = g < (uint32_t)SX || tc::mbar_wait(&xempty[xs], xph ^ 1, SC_POLLS);
                     if (__any_sync(0xffffffffu, !okw)) {
                         failed = true;
