@@ -231,8 +231,8 @@ lmfmm_status lmfmm_test_set_status(lmfmm_ctx *ctx, int bits);
 
 /* Test hook: the next forward pass (a matvec or the first pass of a gradient;
  * not a batch's merged M2L) leaves `bits` (0..255) in the status word after its
- * M2L, in stream order, as if a wait of that M2L had given up.  Requires
- * lmfmm_build. */
+ * M2L, in stream order, as if a wait of that M2L had given up (a pass under
+ * stream capture keeps it in the graph).  Requires lmfmm_build. */
 lmfmm_status lmfmm_test_fail_m2l(lmfmm_ctx *ctx, int bits);
 
 /* Direct evaluation of the same operator over ALL point pairs with the
@@ -410,7 +410,10 @@ lmfmm_status lmfmm_plan_check(const lmfmm_params *prm, int L, const double *d, c
  *       child-parent pairs) + u3 N   [ns],
  * with unit_ns = {u0, u1, u2, u3}, or NULL for costs measured on GB300 with the
  * mixed form and the tensor-core M2L / M2M / L2L at p = 12 (about 80, 0.27, 14.7
- * and 1.1 ns), scaled to other p by (P / 169)^2 (u0, u2) and P / 169 (u3).  The
+ * and 1.1 ns), scaled to other p by (P / 169)^2 (u0, u2) and P / 169 (u3).  u0 is
+ * the cost and the item of the five-table M2L; the sector M2L takes two thirds of it
+ * on the calibration workload (p = 12) and about a quarter at p = 8, so that
+ * predictions are too high, the more so where the M2L's share is large.  The
  * accuracy is set by theta and p, not by the depth.  predicted_ms[dmax - dmin + 1]
  * receives the predictions, *best the depth of the smallest.  Errors as
  * lmfmm_plan_check (LMFMM_ERR_ARG also for a bad depth range or NULL outputs). */
@@ -440,7 +443,7 @@ lmfmm_status lmfmm_batch_matvec(lmfmm_batch *b, const void *const *J, void *cons
 
 /* Autotuner of the merged M2L's work tiles: times the persistent launch
  * (device events, best of three after a warm run, on zeroed expansions) with
- * the work items cut to 64 or 32 helical columns (one MMA tile of 128 real
+ * the work items cut to 64 or 32 pairs (one MMA tile of 128 real
  * rows, or half of it) and ordered problem by problem or round robin, and
  * keeps the fastest (lmfmm_batch_info).  Synchronous.  LMFMM_ERR_UNSUPPORTED
  * when the batch has no merged M2L. */
@@ -451,7 +454,7 @@ lmfmm_status lmfmm_batch_tune(lmfmm_batch *b, void *stream);
 lmfmm_status lmfmm_batch_check(lmfmm_batch *b, void *stream);
 
 /* merged: 1 if the M2L runs as one launch; nwork: its work items; variant:
- * the tuned tiling (bit 0 round robin, bit 1 32-column items); ms_variant[4]:
+ * the tuned tiling (bit 0 round robin, bit 1 32-pair items); ms_variant[4]:
  * the tuner's timings (0 before lmfmm_batch_tune).  Any pointer may be NULL. */
 lmfmm_status lmfmm_batch_info(const lmfmm_batch *b, int *merged, int64_t *nwork, int *variant,
                               double *ms_variant);

@@ -623,7 +623,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         gd.tab_index = (int64_t)i;
         hg[i] = gd;
     }
-    for (size_t i = 0; i < ctx->geoms.size(); ++i) {
+    for (size_t i = 0; d->oz && i < ctx->geoms.size(); ++i) {   // the digit grids of k_m2l_oz
         const Geom &g = ctx->geoms[i];
         double rs = 0.0, rt = 0.0;
         for (int64_t q = g.pair0; q < g.pair1; ++q) {
@@ -1299,7 +1299,7 @@ void batch_drop_graph(lmfmm_batch *b)
 
 // merged work list of a batch: variant bit 0 interleaves the problems' items
 // round robin (else one problem after the other), bit 1 cuts items to 32
-// helical columns (else 64)
+// pairs (else 64)
 lmfmm_status batch_work(lmfmm_batch *b, int variant, M2LWork **dst, int64_t *n)
 {
     std::vector<std::vector<M2LWork>> per(b->ctxs.size());
