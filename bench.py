@@ -39,7 +39,7 @@ SM_COUNT, SM_MHZ = 152, 2070.0
 FP32_PEAK_TFLOPS = SM_COUNT * 128 * 2 * SM_MHZ * 1e6 / 1e12
 FP64_PEAK_TFLOPS = SM_COUNT * 2 * 2 * SM_MHZ * 1e6 / 1e12
 # DRAM bytes of k_m2l_sec over its matrix image (profiles/)
-TRAFFIC_RATIO = 1.904
+TRAFFIC_RATIO = 1.864
 # dense TF32 tensor peak: the measured bf16 burst peak times the nominal
 # TF32 / bf16 ratio (1.1 / 2.25 PFLOP/s); fallback 1.9 PFLOP/s bf16
 TF32_PER_BF16 = 1.1 / 2.25

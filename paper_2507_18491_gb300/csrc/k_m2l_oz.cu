@@ -6,12 +6,17 @@
 // Algorithms 59 (2012), with digits on a common grid per row): every operand is a 64-bit
 // fixed-point number, written as eight signed base-256 digits (a bf16 holds every integer
 // up to 256), and the products of digits i and j are summed per diagonal d = i + j in an FP32
-// accumulator of its own.  Digits are at most 128 in size, so a diagonal's sum over K real
-// inputs is an integer below (d + 1) K 2^14: exact (below 2^24) for d = 0 up to K = 1024, and
-// for the later diagonals, whose digits are spread evenly over +-128, sqrt(K) instead of K.
-// The 36 products with d <= 7 are formed; what is left out is 2^-64 of the largest entry, 11
-// bits below an FP64 rounding.  The eight sums are put together as 64-bit integers and
-// converted once.
+// accumulator of its own, which holds integers exactly below 2^24.  Digits are at most
+// 128 in size, leading ones at most 64 (the matrix) or 64 on average over an input's two parts, so
+// the sum over K real inputs is below K 2^14 for d = 1 and K 2^15 for d = 2: exact whatever the
+// operands for d <= 1 at every p <= 16 (K = 884) and for d = 2 up to p = 11.  Beyond, exactness rests
+// on digits that do not conspire: spread evenly over +-128, a sum's standard deviation is
+// sqrt((d + 1) K) 2^14 / 3, a 36th of 2^24 at d = 7, p = 16, a 48th at p = 12; nothing detects
+// a sum beyond (a rounding at d = 2 would be 2^-30 of the largest product).
+// The 36 products with d <= 7 are formed; what is left out is 2^-64 of the row's and the pair's
+// largest entries.  The eight sums are put together as 64-bit integers and converted once.
+// Measured against the M2L in double-double, rms error per degree block: 2.5 to 17e-16 over two
+// to four layers and p = 6 to 16, the FP64 SIMT kernels 7.8 to 24e-16.
 //
 // Grids: the matrix rows carry their own power of two, the inputs one per pair, after the
 // degrees have been brought to one size by 2^(c_n + a_n), which the matrix columns take out:
@@ -34,7 +39,7 @@
 // sets bit 4 of the status word.
 //
 // Measured (GB300, M2L stage; before: the SIMT five-table kernel at 73% of the FP64 peak): 140593
-// pairs at p = 10 142.8 -> 5.67 ms, 658907 pairs at p = 12 1469 -> 48.4 ms, 3583 pairs at p = 6
+// pairs at p = 10 142.8 -> 5.77 ms, 658907 pairs at p = 12 1469 -> 48.7 ms, 3583 pairs at p = 6
 // 0.90 -> 0.11 ms.
 #include <algorithm>
 

@@ -37,8 +37,8 @@
 // stops.
 //
 // Measured (GB300, M2L stage; before: nine applications of five P x P tables per pair on the
-// same pipeline): 1.70M pairs at p = 8 14.1 -> 3.31 ms, 397328 pairs at p = 7 2.9 -> 0.64 ms,
-// 136292 pairs at p = 12 1.8 -> 1.15 ms.  Per 64-pair item at p = 8 the MMAs take 12 thousand
+// same pipeline): 1.70M pairs at p = 8 14.1 -> 3.31 ms, 397328 pairs at p = 7 2.9 -> 0.65 ms,
+// 136292 pairs at p = 12 1.8 -> 1.17 ms.  Per 64-pair item at p = 8 the MMAs take 12 thousand
 // cycles, the producers 32, the scatter 18.
 #include <algorithm>
 
