@@ -623,17 +623,6 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
         gd.tab_index = (int64_t)i;
         hg[i] = gd;
     }
-    for (size_t i = 0; d->oz && i < ctx->geoms.size(); ++i) {   // the digit grids of k_m2l_oz
-        const Geom &g = ctx->geoms[i];
-        double rs = 0.0, rt = 0.0;
-        for (int64_t q = g.pair0; q < g.pair1; ++q) {
-            rs = std::max(rs, ctx->boxes[ctx->m2l[q].src].r);
-            rt = std::max(rt, ctx->boxes[ctx->m2l[q].tgt].r);
-        }
-        auto lg = [&](double r) { return (float)std::log2(lev_size(g.level) / std::max(r, 0x1p-48 * lev_size(g.level))); };
-        hg[i].lg_s = lg(rs);
-        hg[i].lg_t = lg(rt);
-    }
     {
         // FP64 Chebyshev tabulation, then level scaling (and cast for the mixed form)
         cd *tab64 = nullptr;
@@ -668,8 +657,7 @@ lmfmm_status lmfmm_build(lmfmm_ctx *ctx, void *stream)
             TRY(dalloc(ctx, &q[0], m2l_oz_image_bytes(p, ng)));
             TRY(dalloc(ctx, &q[1], m2l_oz_image_bytes(p, ng)));
             TRY(dalloc(ctx, &q[2], m2l_oz_packed_bytes(p, nbox)));
-            launch_oz_image(p, false, ng, d->geoms, d->comps, tab64, q[0], st);
-            launch_oz_image(p, true, ng, d->geoms, d->comps, tab64, q[1], st);
+            launch_oz_images(p, ng, d->geoms, d->comps, tab64, q[0], q[1], st);
             CK(cudaGetLastError());
             CK(cudaStreamSynchronize(st));
             dfree(ctx, tab64);
@@ -1024,7 +1012,7 @@ static lmfmm_status matvec_t(lmfmm_ctx *ctx, const void *J, int dtype, void *Phi
             launch_m2l_t<T>(p, d->n_m2lwork, d->m2lwork, d->geoms, d->comps, d->m2l,
                             (const cx<T> *)d->tab, me, le, st);
     } else if (d->oz) {
-        CK(launch_m2l_oz(p, false, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->geoms, d->m2l, d->ozimg, nbox, me, le,
+        CK(launch_m2l_oz(p, false, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimg, nbox, me, le,
                          d->ozpk, d->ozscr, d->ncta, d->mvstatus, st));
         ++nl;
     } else {
@@ -1104,7 +1092,7 @@ static lmfmm_status matvec_tr_t(lmfmm_ctx *ctx, const void *y, int dtype, void *
     bool done = false;
     if constexpr (std::is_same<T, double>::value) {
         if (d->oz) {
-            CK(launch_m2l_oz(p, true, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->geoms, d->m2l, d->ozimgT, nbox, le, me,
+            CK(launch_m2l_oz(p, true, (int64_t)ctx->geoms.size(), d->n_m2lwork, d->m2lwork, d->m2l, d->ozimgT, nbox, le, me,
                              d->ozpk, d->ozscr, d->ncta, d->mvstatus, st));
             done = true;
             ++nl;

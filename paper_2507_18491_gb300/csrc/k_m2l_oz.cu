@@ -15,18 +15,23 @@
 // a sum beyond (a rounding at d = 2 would be 2^-30 of the largest product).
 // The 36 products with d <= 7 are formed; what is left out is 2^-64 of the row's and the pair's
 // largest entries.  The eight sums are put together as 64-bit integers and converted once.
-// Measured against the M2L in double-double, rms error per degree block: 2.5 to 17e-16 over two
+// Measured against the M2L in double-double, rms error per degree block: 3.2 to 16e-16 over two
 // to four layers and p = 6 to 16, the FP64 SIMT kernels 7.8 to 24e-16.
 //
 // Grids: the matrix rows carry their own power of two, the inputs one per pair, after the
-// degrees have been brought to one size by 2^(c_n + a_n), which the matrix columns take out:
-// 2^c_n ~ (2n + 1)!! and 2^a_n ~ (S / r)^n, S the cell size, r the largest radius of the
-// geometry's source boxes.  The scaled expansions fall like (r / S)^n / (2n + 1)!!, the columns grow like
-// (S / R)^n (2n + 1)!!, R the distance of the centres, which admissibility bounds by the
-// radii alone: where the points lie far inside their cells, R may be far below S (a cell's centre
-// next to an interface), and without a_n the grid of a row went to columns whose inputs are tiny
-// (r = S / 200, R = S / 25, p = 12: 46% of the result).  With it the products of a row are within
-// max_n C(n + nu, n) (r / R)^n of the row's and the inputs' largest entries.
+// degrees have been brought to one size by 2^a_n, which the matrix columns take out.  A product
+// then misses the bits by which max |M| 2^-a max |x| 2^a exceeds max |M x| of its row.  Entries grow
+// like C(n + nu, n) (2n + 1)!! (2 nu + 1)!! (S / R)^(n + nu), S the cell size, R the distance of the
+// centres; the scaled expansions fall like (r / S)^n / (2n + 1)!!, r the points' radius, or stop falling
+// at what the truncated translations leave.  r may be far below S, and then R too (a cell's centre
+// next to an interface), so a_n comes from the matrix alone, per geometry: of the sum e_nu + a_n
+// closest to the binary exponents of its degree blocks, the column part, in the mean over the rows
+// of degree p / 2 and more (k_oz_degrees).  Whatever the inputs, the missing bits are then at most the
+// spread of log2 C(n + nu, n) about that sum: 2 to 5 (p = 6 to 16) in the rows of the upper degrees; in those
+// of degree 0, if the inputs' highest degree dominates there, 11 at p = 8, 18 at p = 12 and 25 at p = 16.  A 64-bit
+// grid has 11 more than FP64, before the roundings of FP64's own sums.  Other choices of a_n: (2n + 1)!!
+// alone lost a row's grid to columns whose inputs are tiny (r = S / 200, R = S / 25, p = 12: 46% of the
+// result), (S / r)^n the inputs' to the translations' remainders (74%).
 //
 // One CTA per SM walks the work items (up to 64 pairs of one geometry).  Per sector: all
 // threads form the inputs (FP64 phases, digits by integer operations) into a per-CTA image
@@ -95,24 +100,11 @@ OzPlan oz_plan(int p)
     s.o_adj = s.o_ent + (uint32_t)s.nk[0] * 8 * 4;
     s.o_pair = (s.o_adj + (uint32_t)s.nk[0] * 8 * 4 + 15) & ~15u;
     s.o_exp = s.o_pair + OZ_BN * (uint32_t)sizeof(M2LPair);
-    s.o_bars = s.o_exp + OZ_BN * 4 + (OZ_PMAX + 1 + 3) * 4;
+    s.o_bars = s.o_exp + OZ_BN * 4;
     s.smem = s.o_bars + (2 * OZ_ST + 2) * 8 + 16;
     s.out_warps = std::min<int>(OZ_W, (OZ_ST * OZ_SLOT) / s.stage_bytes);
     return s;
 }
-
-// exponent that brings degree n to the size of degree 0: 2^c_n ~ (2n + 1)!!
-__host__ __device__ inline int oz_cn(int n)
-{
-    double f = 1.0;
-    for (int i = 1; i <= n; ++i) f *= 2.0 * i + 1.0;
-    int e;
-    frexp(f, &e);
-    return e - 1;
-}
-
-// ... and of the points' radius against the cell, lg = log2(S / r)
-__host__ __device__ inline int oz_an(int n, float lg) { return (int)rintf((float)n * lg); }
 
 constexpr int OZ_ZERO = -(1 << 14), OZ_BAD = 1 << 14;   // exponents of a degree of zeros, of one that is not finite
 
@@ -173,15 +165,15 @@ __device__ __forceinline__ double2 lds_d2(uint32_t a)
 // transposed: the same walk with the matrices transposed, the phases conjugated and the roles
 // of the pair's boxes exchanged (in: local, out: multipole expansions)
 __global__ void __launch_bounds__(OZ_T, 1)
-    k_m2l_oz(const __grid_constant__ OzPlan sp, int transposed, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-             const M2LPair *pairs, const unsigned char *img, const double *rscale, const OzIn *packed, const int *bexp,
-             cd *out, unsigned char *xscr, double *yscr, int *status)
+    k_m2l_oz(const __grid_constant__ OzPlan sp, int transposed, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+             const unsigned char *img, const double *rscale, const int *dexp, const OzIn *packed, const int *bexp, cd *out,
+             unsigned char *xscr, double *yscr, int *status)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
     const int p = sp.p, P = sp.P, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     uint32_t *ent = (uint32_t *)(smraw + sp.o_ent);
-    // exponents per input, per pair, per degree
-    int *adj = (int *)(smraw + sp.o_adj), *pexp = (int *)(smraw + sp.o_exp), *cn = pexp + OZ_BN;
+    // exponents per input and per pair
+    int *adj = (int *)(smraw + sp.o_adj), *pexp = (int *)(smraw + sp.o_exp);
     M2LPair *pr = (M2LPair *)(smraw + sp.o_pair);
     uint64_t *full = (uint64_t *)(smraw + sp.o_bars), *empty = full + OZ_ST, *accfull = empty + OZ_ST;
     uint32_t *tslot = (uint32_t *)(accfull + 1);
@@ -200,7 +192,6 @@ __global__ void __launch_bounds__(OZ_T, 1)
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     for (int j = tid; j < D0e; j += OZ_T) ent[j] = j < sp.D[0] ? sec_word(p, j) : 0u;
-    if (tid <= p) cn[tid] = oz_cn(tid);
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
@@ -211,13 +202,10 @@ __global__ void __launch_bounds__(OZ_T, 1)
 
     for (int64_t it = blockIdx.x; it < nwork && !failed; it += gridDim.x) {
         const M2LWork w = work[it];
-        const float lg = transposed ? geoms[w.geom].lg_t : geoms[w.geom].lg_s;
         // the inputs' exponents: adj takes the degrees to one size, pexp the pair below 2^-2 (two
-        // coefficients of parts below 2^(pexp - adj): below 2^(pexp + 1.5) each part)
-        for (int j = tid; j < D0e; j += OZ_T) {
-            const int n = j < sp.D[0] ? sec_entry(p, j).n : 0;
-            adj[j] = cn[n] + oz_an(n, lg);
-        }
+        // coefficients of parts below 2^(pexp - adj - 2): below 2^-1.5 of it each)
+        const int *an = dexp + (int64_t)w.geom * (p + 1);
+        for (int j = tid; j < D0e; j += OZ_T) adj[j] = an[j < sp.D[0] ? sec_entry(p, j).n : 0];
         // pair records and phases G[d] (conjugated for the transpose), d = -(p+1)..p
         if (tid < w.npair) {
             const M2LPair q = pairs[w.pair0 + tid];
@@ -226,7 +214,7 @@ __global__ void __launch_bounds__(OZ_T, 1)
             int top = OZ_ZERO;
             for (int n = 0; n <= p; ++n) {
                 const int e = be[n];
-                if (e != OZ_ZERO) top = max(top, e == OZ_BAD ? OZ_BAD : e + cn[n] + oz_an(n, lg));
+                if (e != OZ_ZERO) top = max(top, e == OZ_BAD ? OZ_BAD : e + an[n]);
             }
             pexp[tid] = top == OZ_ZERO ? 0 : top == OZ_BAD ? OZ_BAD : top + 2;
             cd b = mul_i(cd{q.cphi, q.sphi}), e{1.0, 0.0};
@@ -405,15 +393,77 @@ __global__ void __launch_bounds__(OZ_T, 1)
     if (warp == 0) tc::tmem_dealloc(tbase, 512);
 }
 
+// exponents a_n (0 <= n <= p, a_0 = 0) of the degrees of a geometry's columns: source degrees into
+// dexp, target degrees (the transpose's columns) into dexpT.  Of the binary exponents l[nu][n] of the
+// largest entry of every degree block of the five tables: the mean over the rows of degree p / 2 and
+// more of l less the row's own mean.  The upper rows, whose blocks spread most, have it fit them
+// closest: rms errors per degree block at p = 12, three layers, N = 1503, 0.9e-15 (SIMT 1.7e-15), with
+// the mean over all rows 1.9e-15.  One block per geometry; a thread takes a table's row.
+__global__ void __launch_bounds__(256) k_oz_degrees(int p, const GeomDev *geoms, const cd *tab64, int *dexp, int *dexpT)
+{
+    constexpr int NONE = -(1 << 20);
+    __shared__ int l[OZ_PMAX + 1][OZ_PMAX + 1];
+    __shared__ float mean[2][OZ_PMAX + 1];
+    const int P = (p + 1) * (p + 1);
+    const int64_t gi = blockIdx.x;
+    for (int e = threadIdx.x; e < (OZ_PMAX + 1) * (OZ_PMAX + 1); e += blockDim.x) (&l[0][0])[e] = NONE;
+    __syncthreads();
+    for (int tr = threadIdx.x; tr < NTAB * P; tr += blockDim.x) {
+        const cd *row = tab64 + (gi * NTAB * P + tr) * P;
+        int nu = (int)sqrtf((float)(tr % P) + 0.5f);
+        while ((nu + 1) * (nu + 1) <= tr % P) ++nu;
+        while (nu * nu > tr % P) --nu;
+        for (int n = 0, k = 0; n <= p; ++n) {
+            int ex = 0;
+            for (; k < (n + 1) * (n + 1); ++k)
+                ex = max(ex, max((int)(__double_as_longlong(row[k].x) >> 52) & 0x7ff,
+                                 (int)(__double_as_longlong(row[k].y) >> 52) & 0x7ff));
+            if (ex > 0) atomicMax(&l[nu][n], ex - 1023);
+        }
+    }
+    __syncthreads();
+    // means over what is there of a row, then over the differences in a column
+    const int i = threadIdx.x;
+    auto at = [&](int c, int a, int b) { return c ? l[b][a] : l[a][b]; };   // c = 0: rows are target degrees
+    for (int c = 0; c < 2; ++c)
+        if (i <= p) {
+            float s = 0.f;
+            int n = 0;
+            for (int b = 0; b <= p; ++b)
+                if (at(c, i, b) != NONE) {
+                    s += (float)at(c, i, b);
+                    ++n;
+                }
+            mean[c][i] = n ? s / n : 0.f;
+        }
+    __syncthreads();
+    if (i <= p)
+        for (int c = 0; c < 2; ++c) {
+            auto part = [&](int b) {           // of column b
+                float s = 0.f;
+                int n = 0;
+                for (int a = (p + 1) / 2; a <= p; ++a)
+                    if (at(c, a, b) != NONE) {
+                        s += (float)at(c, a, b) - mean[c][a];
+                        ++n;
+                    }
+                return n ? s / n : 0.f;
+            };
+            const GeomDev &g = geoms[gi];
+            const float lg = log2f((float)(c ? g.scale_t : g.scale_s));
+            const float v = part(i) - part(0) + (float)i * lg;
+            (c ? dexpT : dexp)[gi * (p + 1) + i] = (int)rintf(fminf(fmaxf(v, -900.f), 900.f));
+        }
+}
+
 // one warp per row of a geometry's sector block (transposed: of its transpose, with the C
 // entries of order 0 doubled as outputs and halved as inputs, as the shared input and output
 // maps count them): the row's power of two, then its digits in the K-step images
 __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan sp, int transposed,
                                                   const GeomDev *geoms, const CompDev *comps, const cd *tab64,
-                                                  unsigned char *img, double *rscale)
+                                                  const int *dexp, unsigned char *img, double *rscale)
 {
-    __shared__ double ps[OZ_PMAX + 1], pt[OZ_PMAX + 1];
-    __shared__ int cn[OZ_PMAX + 1];
+    __shared__ double ps[OZ_PMAX + 1], pt[OZ_PMAX + 1], cs[OZ_PMAX + 1];
     const int64_t gi = blockIdx.y;
     const GeomDev &gm = geoms[gi];
     if (threadIdx.x <= sp.p) {
@@ -424,7 +474,7 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
         }
         ps[threadIdx.x] = a;
         pt[threadIdx.x] = b;
-        cn[threadIdx.x] = oz_cn(threadIdx.x);
+        cs[threadIdx.x] = ldexp(1.0, -dexp[gi * (sp.p + 1) + threadIdx.x]);
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -434,7 +484,6 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
     const bool fi = (cp.s < 0) != (cp.has_src_refl != 0), fo = (cp.s < 0) != (cp.has_tgt_refl != 0);
     const cd *tab = tab64 + gi * NTAB * (int64_t)sp.P * sp.P;
     const SecEntry er = sec_entry(sp.p, r);
-    const float lg = transposed ? gm.lg_t : gm.lg_s;
     auto value = [&](int k) {
         const SecEntry ek = sec_entry(sp.p, k);
         cd v;
@@ -445,8 +494,7 @@ __global__ void __launch_bounds__(256) k_oz_image(const __grid_constant__ OzPlan
             if (er.c && er.m == 0) v = 2.0 * v;
             if (ek.c && ek.m == 0) v = 0.5 * v;
         }
-        const double f = ldexp(1.0, -cn[ek.n] - oz_an(ek.n, lg));
-        return f * v;
+        return cs[ek.n] * v;
     };
     double mx = 0.0;
     for (int k = lane; k < D; k += 32) {
@@ -518,7 +566,7 @@ int m2l_oz_pairs() { return OZ_BN; }
 size_t m2l_oz_image_bytes(int p, int64_t ngeom)
 {
     const OzPlan sp = oz_plan(p);
-    return (size_t)ngeom * (sp.img_bytes + (size_t)sp.rows * sizeof(double));
+    return (size_t)ngeom * (sp.img_bytes + (size_t)sp.rows * sizeof(double) + (p + 1) * sizeof(int));
 }
 size_t m2l_oz_packed_bytes(int p, int64_t nbox) { return (size_t)nbox * (oz_plan(p).nk[0] * 8 * sizeof(OzIn) + (p + 1) * sizeof(int)); }
 size_t m2l_oz_scratch_bytes(int p, int ncta)
@@ -527,22 +575,30 @@ size_t m2l_oz_scratch_bytes(int p, int ncta)
     return (size_t)ncta * ((size_t)sp.nk[0] * OZ_A + (size_t)OZ_BN * sp.rows * sizeof(double2));
 }
 
-void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
-                     void *img, cudaStream_t st)
+// behind the images: the rows' powers of two, the degrees' exponents
+static double *oz_rscale(const OzPlan &sp, const void *img, int64_t ng) { return (double *)((unsigned char *)img + (size_t)ng * sp.img_bytes); }
+static int *oz_dexp(const OzPlan &sp, const void *img, int64_t ng) { return (int *)(oz_rscale(sp, img, ng) + (size_t)ng * sp.rows); }
+
+void launch_oz_images(int p, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64, void *img, void *imgT,
+                      cudaStream_t st)
 {
     const OzPlan sp = oz_plan(p);
-    double *rs = (double *)((unsigned char *)img + (size_t)ng * sp.img_bytes);
-    cudaMemsetAsync(img, 0, (size_t)ng * sp.img_bytes, st);   // rows beyond the block stay zero
-    for (int64_t g0 = 0; g0 < ng; g0 += 32768) {              // grid.y is limited to 65535
-        const int64_t nb = std::min<int64_t>(32768, ng - g0);
-        k_oz_image<<<dim3((sp.rows + 7) / 8, (unsigned)nb), 256, 0, st>>>(
-            sp, transposed, geoms + g0, comps, tab64 + g0 * NTAB * (int64_t)sp.P * sp.P,
-            (unsigned char *)img + (size_t)g0 * sp.img_bytes, rs + g0 * sp.rows);
+    if (ng <= 0) return;
+    k_oz_degrees<<<(unsigned)ng, 256, 0, st>>>(p, geoms, tab64, oz_dexp(sp, img, ng), oz_dexp(sp, imgT, ng));
+    for (int tr = 0; tr < 2; ++tr) {
+        void *q = tr ? imgT : img;
+        cudaMemsetAsync(q, 0, (size_t)ng * sp.img_bytes, st);     // rows beyond the block stay zero
+        for (int64_t g0 = 0; g0 < ng; g0 += 32768) {              // grid.y is limited to 65535
+            const int64_t nb = std::min<int64_t>(32768, ng - g0);
+            k_oz_image<<<dim3((sp.rows + 7) / 8, (unsigned)nb), 256, 0, st>>>(
+                sp, tr, geoms + g0, comps, tab64 + g0 * NTAB * (int64_t)sp.P * sp.P, oz_dexp(sp, q, ng) + g0 * (p + 1),
+                (unsigned char *)q + (size_t)g0 * sp.img_bytes, oz_rscale(sp, q, ng) + g0 * sp.rows);
+        }
     }
 }
 
-cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-                          const M2LPair *pairs, const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
+cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
                           int *status, cudaStream_t st)
 {
     if (!m2l_oz_supported(p) || ncta < 1) return cudaErrorInvalidValue;
@@ -553,8 +609,8 @@ cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, 
     if (nwork <= 0) return cudaGetLastError();
     unsigned char *x = (unsigned char *)scratch;
     k_m2l_oz<<<(unsigned)std::min<int64_t>(nwork, ncta), OZ_T, std::max<size_t>(sp.smem, 116 * 1024), st>>>(
-        sp, transposed ? 1 : 0, nwork, work, geoms, pairs, (const unsigned char *)img,
-        (const double *)((const unsigned char *)img + (size_t)ngeom * sp.img_bytes), (const OzIn *)packed, be, out, x,
+        sp, transposed ? 1 : 0, nwork, work, pairs, (const unsigned char *)img, oz_rscale(sp, img, ngeom),
+        oz_dexp(sp, img, ngeom), (const OzIn *)packed, be, out, x,
         (double *)(x + (size_t)ncta * sp.nk[0] * OZ_A), status);
     return cudaGetLastError();
 }

@@ -30,8 +30,7 @@ struct GeomDev {
     int64_t node0;      // first node within its tabulation batch
     int64_t stride;     // node count of its batch (factor-array stride)
     int64_t tab_index;  // table slot
-    // log2 of the cell size over the largest radius of the source / target boxes of its pairs
-    float lg_s, lg_t;
+    int batch, pad;
 };
 
 struct LayerScale {      // |k_l| S_leaf per layer (expansion scaling at the leaves)
@@ -187,18 +186,19 @@ cudaError_t launch_m2l_sec(int p, int64_t nwork, const M2LWork *work, const TcPr
                            float *yscr, int ncta, int *status, cudaStream_t st);
 // k_m2l_oz.cu: M2L of the FP64 form on the tensor cores, operands as eight base-256 digits.
 // out is cleared, then out[tgt] += M in[src] over the items' pairs (transposed: in over the
-// targets, out over the sources); img from launch_oz_image (m2l_oz_image_bytes), packed and
+// targets, out over the sources); img from launch_oz_images (m2l_oz_image_bytes), packed and
 // scratch of the sizes below
 bool m2l_oz_supported(int p);
 int m2l_oz_pairs();
-size_t m2l_oz_image_bytes(int p, int64_t ngeom);
+size_t m2l_oz_image_bytes(int p, int64_t ngeom);   // with the exponents of rows and degrees
 size_t m2l_oz_packed_bytes(int p, int64_t nbox);
 size_t m2l_oz_scratch_bytes(int p, int ncta);
 cudaError_t configure_m2l_oz();
-void launch_oz_image(int p, bool transposed, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64,
-                     void *img, cudaStream_t st);
-cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const GeomDev *geoms,
-                          const M2LPair *pairs, const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
+// the images of the blocks and of their transposes
+void launch_oz_images(int p, int64_t ng, const GeomDev *geoms, const CompDev *comps, const cd *tab64, void *img, void *imgT,
+                      cudaStream_t st);
+cudaError_t launch_m2l_oz(int p, bool transposed, int64_t ngeom, int64_t nwork, const M2LWork *work, const M2LPair *pairs,
+                          const void *img, int64_t nbox, const cd *in, cd *out, void *packed, void *scratch, int ncta,
                           int *status, cudaStream_t st);
 // M2M or L2L on a persistent tensor-core kernel (k_m2l_tc.cu, p <= 12): items M2LWork{geom = translation group, t = 0,
 // npair, pair0} over pairs (tsrc[q], tdst[q]), 3 helical columns each; img holds

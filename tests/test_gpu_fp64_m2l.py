@@ -31,14 +31,14 @@ def test_digits_against_simt(p):
         assert (a - b).norm() < 1e-13 * b.norm()
 
 
-def _near_centre(height, spread, k):
+def _near_centre(height, spread, k, offset=0.0):
     """Points within `spread` of the centre of a cell of side 1 that lies `height` above an interface,
     and points elsewhere that span the root cell [-1, 1]^3: the image of the cell's centre is 2 height
     away, a small part of the cell's side, and still far from the points by their radius."""
     rng = np.random.default_rng(9)
-    near = 0.5 + spread * rng.uniform(-1, 1, (12, 3))
+    near = 0.5 + offset + spread * rng.uniform(-1, 1, (12, 3))
     wide = np.array([[1, -1, -1], [-1, 1, -1], [-1, -1, 1], [-1, -1, -1]], float) * (1 - 1e-9)
-    below = np.array([0.5, 0.5, 0.5 - 2 * height]) + spread * rng.uniform(-1, 1, (12, 3))
+    below = np.array([0.5, 0.5, 0.5 - 2 * height]) + offset + spread * rng.uniform(-1, 1, (12, 3))
     xyz = np.concatenate([near, wide, below])
     J = rng.standard_normal(xyz.shape) + 1j * rng.standard_normal(xyz.shape)
     return [0.5 - height], k, xyz, J
@@ -51,11 +51,23 @@ def _near_centre(height, spread, k):
 @pytest.mark.parametrize("p,height,spread", [(8, 0.1, 0.01), (12, 0.1, 0.01), (16, 0.1, 0.01), (12, 0.02, 0.002),
                                              (16, 0.02, 0.002)])
 def test_expansions_far_inside_their_cells(p, height, spread):
-    d, k, xyz, J = _near_centre(height, spread, [1.3 + 0.01j, 2.1 + 0.02j])
+    _compare(p, height, spread, 1)
+
+
+# the same through M2M and L2L: at the cell, the expansions' high degrees are what the truncated
+# translations leave there, not (radius / side)^n, and a grid that follows the radius gives its bits to
+# them (74% off).  The points lie in one octant, so that every box has one child and both operators form the same expansions
+@pytest.mark.parametrize("p,height,offset", [(6, 0.4, 4e-6), (8, 0.4, 1.5e-4)])
+def test_translated_expansions_far_inside_their_cells(p, height, offset):
+    _compare(p, height, offset / 8, 4, offset)
+
+
+def _compare(p, height, spread, depth, offset=0.0):
+    d, k, xyz, J = _near_centre(height, spread, [1.3 + 0.01j, 2.1 + 0.02j], offset)
     Jt = torch.from_numpy(J).cuda()
     out = []
     for tc in (1, 0):
-        op = lmfmm.Operator(d, k, xyz, p=p, depth=1, theta=0.5, tensor_cores=tc).build()
+        op = lmfmm.Operator(d, k, xyz, p=p, depth=depth, theta=0.5, tensor_cores=tc).build()
         assert op.stats()["m2l_digits"] == tc
         out.append((op.matvec(Jt), op.tmatvec(Jt)))
         ref = op.direct(Jt)
