@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(256) k_oz_degrees(int p, const GeomDev *geoms,
                 return n ? s / n : 0.f;
             };
             const GeomDev &g = geoms[gi];
-            const float lg = log2f((float)(c ? g.scale_t : g.scale_s));
+            const float lg = (float)log2(c ? g.scale_t : g.scale_s);
             const float v = part(i) - part(0) + (float)i * lg;
             (c ? dexpT : dexp)[gi * (p + 1) + i] = (int)rintf(fminf(fmaxf(v, -900.f), 900.f));
         }

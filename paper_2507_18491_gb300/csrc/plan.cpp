@@ -558,7 +558,7 @@ extern "C" lmfmm_status lmfmm_plan_check(const lmfmm_params *prm, int L, const d
 // over 37447 (child, parent) pairs; 1.154 ms of P2M, L2P and permutation over
 // 2^20 points), scaled to other p by (P / 169)^2 for the M2L and translations
 // and by P / 169 for the point terms.  The M2L's is that of the five-table kernel;
-// the sector kernel that runs today takes 5.83 ms there.
+// the sector kernel that runs today takes 5.88 ms there.
 extern "C" lmfmm_status lmfmm_plan_depth(const lmfmm_params *prm, int L, const double *d, const lmfmm_c128 *k,
                                          int64_t N, const double *xyz, int dmin, int dmax, const double *unit_ns,
                                          int *best, double *predicted_ms)
